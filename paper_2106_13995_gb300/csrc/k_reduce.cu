@@ -137,13 +137,20 @@ __device__ __forceinline__ void block_sum_to(double v, double *dst) {
   }
 }
 
-// out[j] = sum_b partial[b * nvals + j]  (+ optional add into out)
-__global__ void k_finalize(const double *__restrict__ partial, int nblocks, int nvals, double *out) {
-  for (int j = threadIdx.x; j < nvals; j += blockDim.x) {
-    double s = 0;
-    for (int b = 0; b < nblocks; b++) s += partial[(size_t)b * nvals + j];
-    out[j] = s;
-  }
+// *out = sum of the blocks' partial sums: one block, each thread a strided
+// share (independent loads), then the block's tree.  One thread adding them
+// in turn is a chain of L2 latencies: 43 us for 608 partials against 3.
+__global__ void __launch_bounds__(kRedThreads) k_finalize(const double *__restrict__ partial, int nblocks, double *out) {
+  double s = 0;
+  for (int b = threadIdx.x; b < nblocks; b += kRedThreads) s += partial[b];
+  block_sum_to(s, out);
+}
+
+sv_status launch_finalize(sv_state *s, const double *partial, int nblocks, double *out_dev) {
+  k_finalize<<<1, kRedThreads, 0, s->stream>>>(partial, nblocks, out_dev);
+  g_launches++;
+  SV_CUDA(cudaGetLastError());
+  return SV_OK;
 }
 
 // ---- norm -----------------------------------------------------------------
@@ -179,10 +186,8 @@ sv_status launch_norm(sv_state *s, double *out_dev) {
     k_norm<float><<<g, kRedThreads, 0, s->stream>>>((const int4 *)s->amps, nunits, partial);
   else
     k_norm<double><<<g, kRedThreads, 0, s->stream>>>((const int4 *)s->amps, nunits, partial);
-  k_finalize<<<1, 32, 0, s->stream>>>(partial, g, 1, out_dev);
-  g_launches += 2;
-  SV_CUDA(cudaGetLastError());
-  return SV_OK;
+  g_launches++;
+  return launch_finalize(s, partial, g, out_dev);
 }
 
 // ---- Pauli-string group expectation --------------------------------------
@@ -295,9 +300,12 @@ __global__ void __launch_bounds__(kRedThreads) k_expect(const typename Cx<R>::T 
 // the sum over lanes of the lane's coefficient for L's pattern with the sign
 // of L's lane bits, so each lane accumulates its signed coefficients and
 // the block sums once at the end.  Terms sharing a low part form a group
-// whose chunk coefficient sums their high-part signs.  The group loop reads
-// the coefficients from shared memory, which keeps the code small (unrolled
-// over all patterns it missed the instruction cache).
+// whose chunk coefficient sums their high-part signs: a lane evaluates each
+// term's sign and a lane each group's sum (every lane doing all of them was
+// two thirds of the kernel's instructions: 25 ZZ terms on 26 qubits took
+// 126 us, now 86, HBM's share 79).  The group loop reads the
+// coefficients from shared memory, which keeps the code small (unrolled over
+// all patterns it missed the instruction cache).
 constexpr int kDiagTrips = 32;
 template <typename R> struct DiagArgs {
   uint32_t ng;                              // groups (terms sharing a low part)
@@ -318,7 +326,12 @@ __global__ void __launch_bounds__(kDiagThreads) k_expect_diag(const int4 *__rest
   constexpr int TRIPS = kDiagTrips;
   constexpr int NPAT = APU * TRIPS;
   __shared__ R sq[kDiagThreads / 32][NPAT][32];
+  __shared__ R sc[kDiagThreads / 32][kMaxGroupTerms];   // the chunk's signed term coefficients
+  __shared__ R sk[kDiagThreads / 32][kMaxGroupTerms];   // their sums by group
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  uint64_t lsign = 0;   // the lane's sign in each group
+  for (uint32_t g = 0; g < A.ng; g++) lsign |= (uint64_t)(__popc((uint32_t)lane & A.lm[g]) & 1) << g;
+  const int nt = (int)A.tstart[A.ng];
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   double acc = 0;
@@ -346,22 +359,22 @@ __global__ void __launch_bounds__(kDiagThreads) k_expect_diag(const int4 *__rest
 #pragma unroll
     for (int i = 0; i < NPAT; i++) sq[wi][i][lane] = q[i];
     __syncwarp();
-    // two accumulators each, so the sums are not one serial chain
+    // the terms' signs at this chunk, a lane per term, then a lane per group
+    for (int t = lane; t < nt; t += 32) sc[wi][t] = (__popcll(x0 & A.zm[t]) & 1) ? -A.c[t] : A.c[t];
+    __syncwarp();
+    for (uint32_t g = lane; g < A.ng; g += 32) {
+      R ck = 0;
+      for (uint32_t t = A.tstart[g]; t < A.tstart[g + 1]; t++) ck += sc[wi][t];
+      sk[wi][g] = ck;
+    }
+    __syncwarp();
+    // two accumulators, so the sum is not one serial chain
     R part0 = 0, part1 = 0;
     for (uint32_t g = 0; g < A.ng; g++) {
-      R ck0 = 0, ck1 = 0;
-      uint32_t t = A.tstart[g];
-      const uint32_t te = A.tstart[g + 1];
-      for (; t + 1 < te; t += 2) {
-        ck0 += (__popcll(x0 & A.zm[t]) & 1) ? -A.c[t] : A.c[t];
-        ck1 += (__popcll(x0 & A.zm[t + 1]) & 1) ? -A.c[t + 1] : A.c[t + 1];
-      }
-      if (t < te) ck0 += (__popcll(x0 & A.zm[t]) & 1) ? -A.c[t] : A.c[t];
-      const R ck = ck0 + ck1;
-      const R qv = sq[wi][A.gpat[g]][lane];
-      const R term = (__popc((uint32_t)lane & A.lm[g]) & 1) ? -ck * qv : ck * qv;
-      if (g & 1) part1 += term;
-      else part0 += term;
+      const R ck = sk[wi][g], qv = sq[wi][A.gpat[g]][lane];
+      const R cs = ((lsign >> g) & 1) ? -ck : ck;
+      if (g & 1) part1 = fma(cs, qv, part1);
+      else part0 = fma(cs, qv, part0);
     }
     acc += (double)part0 + (double)part1;
   }
@@ -417,10 +430,8 @@ static bool expect_diag_launch(sv_state *s, const uint64_t *zm, const double *cf
   const int g = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)s->sm_count * 8));
   k_expect_diag<R><<<g, kDiagThreads, 0, s->stream>>>(reinterpret_cast<const int4 *>(s->amps), nchunks, A,
                                                        partial);
-  k_finalize<<<1, 32, 0, s->stream>>>(partial, g, 1, out_dev);
-  g_launches += 2;
-  const cudaError_t e = cudaGetLastError();
-  st = e == cudaSuccess ? SV_OK : cuda_error(e, "k_expect_diag");
+  g_launches++;
+  st = launch_finalize(s, partial, g, out_dev);
   return true;
 }
 
@@ -450,10 +461,8 @@ static sv_status expect_launch(sv_state *s, uint64_t xm, const uint64_t *zm, con
   const int g = red_grid(s, na / 64 + 1);
   k_expect<R><<<g, kRedThreads, 0, s->stream>>>(reinterpret_cast<const typename Cx<R>::T *>(s->amps), na, A,
                                                 partial);
-  k_finalize<<<1, 32, 0, s->stream>>>(partial, g, 1, out_dev);
-  g_launches += 2;
-  SV_CUDA(cudaGetLastError());
-  return SV_OK;
+  g_launches++;
+  return launch_finalize(s, partial, g, out_dev);
 }
 
 sv_status launch_expect_group(sv_state *s, uint64_t xm, const uint64_t *zm, const double *cf,
@@ -546,20 +555,22 @@ __global__ void k_zall_small(const typename Cx<R>::T *__restrict__ a, int n, dou
   for (int q = threadIdx.x; q <= n; q += blockDim.x) out[q] = q < n ? sm[q] : sm[64];
 }
 
-// z[q] = total - 2 S_q from the reduced S_q (in place: buf[0..n] -> z[0..n-1])
-__global__ void k_zall_finish(const double *__restrict__ partial, int nblocks, int n, double *out) {
-  __shared__ double tot;
-  if (threadIdx.x == 0) {
-    double t = 0;
-    for (int b = 0; b < nblocks; b++) t += partial[(size_t)b * (n + 1) + n];
-    tot = t;
+// z[q] = total - 2 S_q from the blocks' partial sums: a warp per value, its
+// lanes striding over the blocks.  A thread per value was a chain of one L2
+// latency per block (63-126 us for 608 blocks; now 6).
+constexpr int kZFinishThreads = 1024;
+__global__ void __launch_bounds__(kZFinishThreads) k_zall_finish(const double *__restrict__ partial, int nblocks, int n,
+                                                                 double *out) {
+  __shared__ double sum[64 + 1];
+  const int lane = threadIdx.x & 31;
+  for (int q = threadIdx.x >> 5; q <= n; q += kZFinishThreads / 32) {
+    double s = 0;
+    for (int b = lane; b < nblocks; b += 32) s += partial[(size_t)b * (n + 1) + q];
+    s = warp_sum(s);
+    if (lane == 0) sum[q] = s;
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < n; q += blockDim.x) {
-    double s = 0;
-    for (int b = 0; b < nblocks; b++) s += partial[(size_t)b * (n + 1) + q];
-    out[q] = tot - 2.0 * s;
-  }
+  for (int q = threadIdx.x; q < n; q += kZFinishThreads) out[q] = sum[n] - 2.0 * sum[q];
 }
 
 sv_status launch_z_all(sv_state *s, double *out_dev) {
@@ -572,7 +583,7 @@ sv_status launch_z_all(sv_state *s, double *out_dev) {
       k_zall_small<float><<<1, 256, 0, s->stream>>>((const float2 *)s->amps, s->n, partial);
     else
       k_zall_small<double><<<1, 256, 0, s->stream>>>((const double2 *)s->amps, s->n, partial);
-    k_zall_finish<<<1, 64, 0, s->stream>>>(partial, 1, s->n, out_dev);
+    k_zall_finish<<<1, kZFinishThreads, 0, s->stream>>>(partial, 1, s->n, out_dev);
   } else {
     const uint64_t nchunks = namps / chunk_amps;
     const uint64_t warps_per_block = kRedThreads / 32;
@@ -582,7 +593,7 @@ sv_status launch_z_all(sv_state *s, double *out_dev) {
       k_zall<float><<<g, kRedThreads, 0, s->stream>>>((const int4 *)s->amps, s->n, nchunks, partial);
     else
       k_zall<double><<<g, kRedThreads, 0, s->stream>>>((const int4 *)s->amps, s->n, nchunks, partial);
-    k_zall_finish<<<1, 64, 0, s->stream>>>(partial, g, s->n, out_dev);
+    k_zall_finish<<<1, kZFinishThreads, 0, s->stream>>>(partial, g, s->n, out_dev);
   }
   g_launches += 2;
   SV_CUDA(cudaGetLastError());
@@ -637,7 +648,7 @@ sv_status zall_noalloc(const void *amps, int n, sv_dtype dt, double *out, cudaSt
       k_zall_small<float><<<1, 256, 0, stream>>>((const float2 *)amps, n, partial);
     else
       k_zall_small<double><<<1, 256, 0, stream>>>((const double2 *)amps, n, partial);
-    k_zall_finish<<<1, 64, 0, stream>>>(partial, 1, n, out);
+    k_zall_finish<<<1, kZFinishThreads, 0, stream>>>(partial, 1, n, out);
   } else {
     const uint64_t nchunks = namps / chunk_amps;
     const uint64_t wpb = kRedThreads / 32;
@@ -648,7 +659,7 @@ sv_status zall_noalloc(const void *amps, int n, sv_dtype dt, double *out, cudaSt
       k_zall<float><<<g, kRedThreads, 0, stream>>>((const int4 *)amps, n, nchunks, partial);
     else
       k_zall<double><<<g, kRedThreads, 0, stream>>>((const int4 *)amps, n, nchunks, partial);
-    k_zall_finish<<<1, 64, 0, stream>>>(partial, g, n, out);
+    k_zall_finish<<<1, kZFinishThreads, 0, stream>>>(partial, g, n, out);
   }
   g_launches += 2;
   SV_CUDA(cudaGetLastError());

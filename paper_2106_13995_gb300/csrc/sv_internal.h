@@ -445,6 +445,13 @@ sv_status launch_diag_gate(sv_state *s, const std::vector<int> &targets,
 sv_status launch_norm(sv_state *s, double *out_dev_scalar);
 sv_status launch_expect_group(sv_state *s, uint64_t xmask, const uint64_t *zm, const double *cf,
                               const int *ipow, int nt, double *out_dev);
+// strings with X or Y factors, many x masks per pass (k_expect_tile.cu); a
+// group lists the terms that share one x mask
+bool expect_tile_ok(const sv_state *s, uint64_t xmask, int nt);
+sv_status launch_expect_tiles(sv_state *s, const sv_pauli_term *terms, const std::vector<std::vector<int>> &groups,
+                              double *out_dev);
+// *out_dev = sum of nblocks FP64 partial sums
+sv_status launch_finalize(sv_state *s, const double *partial, int nblocks, double *out_dev);
 sv_status launch_z_all(sv_state *s, double *out_dev);
 sv_status zall_noalloc(const void *amps, int n, sv_dtype dt, double *out, cudaStream_t stream);
 sv_status launch_sample_prepare(sv_state *s);
