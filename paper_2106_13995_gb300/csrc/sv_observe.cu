@@ -33,14 +33,27 @@ extern "C" {
 sv_status sv_expect(sv_state *s, const sv_pauli_term *terms, int nt, double *out) {
   if (!s || !out) return set_error(SV_EINVAL, "null argument");
   SV_TRY(check_terms(s, terms, nt));
-  // group by x mask: each group is one read pass
+  // group by x mask: groups with X or Y factors share tile passes, each of
+  // the others is one read pass
   std::map<uint64_t, std::vector<int>> groups;
   for (int t = 0; t < nt; t++) groups[terms[t].x_mask].push_back(t);
-  std::vector<std::vector<int>> chunks;
-  for (auto &g : groups)
+  std::vector<std::vector<int>> chunks, tiled;
+  for (auto &g : groups) {
+    if (expect_tile_ok(s, g.first, (int)g.second.size())) {
+      tiled.push_back(g.second);
+      continue;
+    }
     for (size_t i = 0; i < g.second.size(); i += 64)
       chunks.emplace_back(g.second.begin() + i, g.second.begin() + std::min(g.second.size(), i + 64));
+  }
   double total = 0;
+  if (!tiled.empty()) {
+    // its slot is read back with the first chunks' (the last result slot)
+    SV_TRY(launch_expect_tiles(s, terms, tiled, scalars_dev(s) + kMaxSlots));
+    SV_CUDA(cudaMemcpyAsync(scalars_host(s) + kMaxSlots, scalars_dev(s) + kMaxSlots, sizeof(double),
+                            cudaMemcpyDeviceToHost, s->stream));
+    if (chunks.empty()) SV_CUDA(cudaStreamSynchronize(s->stream));
+  }
   for (size_t c0 = 0; c0 < chunks.size(); c0 += kMaxSlots) {
     const size_t c1 = std::min(chunks.size(), c0 + kMaxSlots);
     for (size_t c = c0; c < c1; c++) {
@@ -58,6 +71,7 @@ sv_status sv_expect(sv_state *s, const sv_pauli_term *terms, int nt, double *out
     SV_TRY(fetch(s, (int)(c1 - c0)));
     for (size_t c = c0; c < c1; c++) total += scalars_host(s)[c - c0];
   }
+  if (!tiled.empty()) total += scalars_host(s)[kMaxSlots];
   *out = total;
   return SV_OK;
 }
