@@ -240,13 +240,13 @@ sv_status sv_plan_fmas(sv_state *s, const sv_circuit *c, const double *params, c
 /* Apply circs[b] (with parameters params[b], host FP64, either may repeat)
  * to states[b] for b < B, states of any widths, in one call: every circuit
  * is fused and planned into tile passes as by sv_apply_circuit.  The narrow
- * states (passes with fewer tiles than the GPU has SMs) go through ONE
+ * states (below 19 qubits, below 14 when replayed from a graph) go through ONE
  * persistent launch: a cooperative kernel works through the queue of all
  * their (state, pass, tile) items in pass order, a tile of pass p waiting
  * until pass p-1 of its own state is complete (Sec. I motivates many
  * independent simulations: variational training evaluates many circuits).
  * The wide states, and programs with tensor-core passes, follow as ordinary
- * full-grid launches of their passes, spread over up to four library-owned
+ * full-grid launches of their passes, spread over up to eight library-owned
  * streams forked from the states' stream after that launch and joined back
  * into it (the call stays stream-ordered).  Waits are
  * bounded by opt->timeout_cycles polls (~128 ns each; 0 = about 1 s); a wait

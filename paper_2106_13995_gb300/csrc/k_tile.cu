@@ -35,9 +35,9 @@ __device__ __forceinline__ void cp_async16(uint32_t smem, const void *gmem) {
 // The work of one CTA on one tile.  COH selects L2-coherent loads and stores
 // (bypassing L1), needed when other CTAs of the same launch wrote the tile
 // earlier (the persistent batch kernel); otherwise streaming hints are used.
-template <typename R, bool COH, bool INL = false>
+template <typename R, bool COH, bool INL = false, class Inl = TileInline>
 __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int b, unsigned char *smem_raw,
-                                          const TileInline *I = nullptr) {
+                                          const Inl *I = nullptr) {
   using C = typename Cx<R>::T;
   const uint32_t TS = 1u << P.m;
   C *v0 = reinterpret_cast<C *>(smem_raw);
@@ -217,10 +217,11 @@ __global__ void __launch_bounds__(kTilePassThreads, kTilePassMinBlocks) k_tile(c
 
 // The same pass with its op list and small dense matrices in the parameter
 // block (complex64, one vector, one state).
+template <class Inl>
 __global__ void __launch_bounds__(kTilePassThreads, kTilePassMinBlocks)
-    k_tile_inl(const __grid_constant__ TilePass P, const __grid_constant__ TileInline I) {
+    k_tile_inl(const __grid_constant__ TilePass P, const __grid_constant__ Inl I) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  tile_body<float, false, true>(P, blockIdx.x, 0, smem_raw, &I);
+  tile_body<float, false, true, Inl>(P, blockIdx.x, 0, smem_raw, &I);
 }
 static_assert(sizeof(TilePass) + sizeof(TileInline) <= 32000, "kernel parameters exceed 32 KB");
 
@@ -264,8 +265,8 @@ void fill_op_pre(const TileOp &op, int threads, OpPre &pre) {
   for (int it = 0; it < 4; it++) pre.tc[it] = h_swb(h_ins0_mask((uint32_t)(it * G) << low, f));
 }
 
-static bool build_inline(const TilePass &p, const HostPass &h, TileInline &I, int threads) {
-  if (p.nops > kInlOps) return false;
+template <class Inl> static bool build_inline(const TilePass &p, const HostPass &h, Inl &I, int threads) {
+  if (p.nops > Inl::kOps) return false;
   I.nops = (uint32_t)p.nops;
   I.nmat = 0;
   for (int i = 0; i < p.nops; i++) {
@@ -273,7 +274,7 @@ static bool build_inline(const TilePass &p, const HostPass &h, TileInline &I, in
     if (op.kind == TOP_DENSE && op.k <= 3) {
       const uint32_t cnt = 1u << (2 * op.k);
       const uint32_t at = I.nmat;
-      if (op.gen != 0 || op.vmask != 1 || at + cnt > (uint32_t)kInlMat) return false;
+      if (op.gen != 0 || op.vmask != 1 || at + cnt > (uint32_t)Inl::kMat) return false;
       std::memcpy(&I.mats[at], h.mats + (size_t)op.mat * sizeof(float2), cnt * sizeof(float2));
       op.mat = at;
       op.gen = kGenInline;
@@ -368,11 +369,33 @@ __global__ void k_wait_selftest(const uint32_t *never, uint32_t *err, uint64_t l
   if (threadIdx.x == 0 && !bounded_wait(never, 1u, limit)) atomicExch(err, 1u);
 }
 
+// Launch the pass with a parameter block of this size; false (nothing
+// launched) when the pass does not fit it.
+template <class Inl>
+static bool launch_inl(sv_state *s, const TilePass &p, const HostPass &h, dim3 grid, int threads, size_t smem,
+                       cudaStream_t stream, sv_status &st) {
+  Inl inl;   // copied into the launch
+  if (!build_inline(p, h, inl, threads)) return false;
+  st = func_attr_once((const void *)k_tile_inl<Inl>, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10);
+  if (st == SV_OK) k_tile_inl<Inl><<<grid, threads, smem, stream>>>(p, inl);
+  return true;
+}
+
 int tile_threads(int m, sv_dtype dt) {
   const int units = (1 << m) / (dt == SV_C64 ? 2 : 1);
   int t = units / 16;
   if (t < 32) t = 32;
   if (t > kTilePassThreads) t = kTilePassThreads;
+  return t;
+}
+
+// Threads of a pass of `tiles` tiles.  32 amplitudes a thread pay each op's
+// set-up once for many, but a pass whose tiles leave the GPU mostly empty is a
+// chain of latencies: there, up to a thread per group of 8 amplitudes.
+static int pass_threads(const sv_state *s, int m, uint64_t tiles) {
+  int t = tile_threads(m, s->dt);
+  const int most = std::min(kTilePassThreads, std::max(32, 1 << std::max(0, m - 3)));
+  while (t < most && tiles * (uint64_t)t < (uint64_t)s->sm_count * 512) t *= 2;
   return t;
 }
 
@@ -482,16 +505,18 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
   const cudaFuncAttribute kSmemAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (s->dt == SV_C64) {
     SV_TRY(func_attr_once((const void *)k_tile<float>, s->device, kSmemAttr, 200 << 10));
-    SV_TRY(func_attr_once((const void *)k_tile_inl, s->device, kSmemAttr, 200 << 10));
   } else {
     SV_TRY(func_attr_once((const void *)k_tile<double>, s->device, kSmemAttr, 200 << 10));
   }
   if (smem > (200u << 10)) return set_error(SV_EINVAL, "tile too large for shared memory");
   dim3 grid((unsigned)(1ull << (p.n - p.m)), (unsigned)batch);
-  const int threads = tile_threads(p.m, s->dt);
-  TileInline inl;   // copied into the launch
-  if (host && s->dt == SV_C64 && batch == 1 && p.nvec == 1 && build_inline(p, *host, inl, threads))
-    k_tile_inl<<<grid, threads, smem, stream>>>(p, inl);
+  const int threads = pass_threads(s, p.m, (uint64_t)grid.x * grid.y);
+  sv_status st = SV_OK;
+  const bool try_inl = host && s->dt == SV_C64 && batch == 1 && p.nvec == 1;
+  if (try_inl && (launch_inl<TileInlineSmall>(s, p, *host, grid, threads, smem, stream, st) ||
+                  launch_inl<TileInlineMid>(s, p, *host, grid, threads, smem, stream, st) ||
+                  launch_inl<TileInline>(s, p, *host, grid, threads, smem, stream, st)))
+    SV_TRY(st);
   else if (s->dt == SV_C64)
     k_tile<float><<<grid, threads, smem, stream>>>(p);
   else
@@ -506,13 +531,16 @@ sv_status launch_tile_persist(sv_state *s, const PersistArgs &A, int m_max, int 
   if (smem > (200u << 10)) return set_error(SV_EINVAL, "tile too large for shared memory");
   const void *fn = s->dt == SV_C64 ? (const void *)k_tile_persist<float> : (const void *)k_tile_persist<double>;
   SV_TRY(func_attr_once(fn, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10));
+  // 16 amplitudes a thread: smaller tiles take smaller CTAs and more of them,
+  // so the items of many states are in flight at once
+  const int threads = std::max(128, std::min(kTileMaxThreads, 1 << std::max(0, m_max - 4)));
   int per_sm = 0;
-  SV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kTileMaxThreads, smem));
+  SV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
   if (per_sm < 1) return set_error(SV_EUNSUPPORTED, "persistent tile kernel does not fit on an SM");
   const int grid = per_sm * s->sm_count;
   PersistArgs a = A;
   void *args[] = {&a};
-  SV_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kTileMaxThreads), args, smem, st));
+  SV_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, smem, st));
   g_launches++;
   if (grid_out) *grid_out = grid;
   return SV_OK;

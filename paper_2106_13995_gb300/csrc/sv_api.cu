@@ -44,13 +44,29 @@ size_t red_bytes(int n) {
 // ---------------------------------------------------------------------------
 Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   Opts r;
-  r.fusion_k = (o && o->fusion_k > 0) ? o->fusion_k : (o && o->prec != SV_PREC_PLAIN ? 5 : 3);
+  // complex128 states of up to 17 qubits: fused pairs instead of triples.
+  // The few tiles leave the FP64 pipes waiting on each other's results, and
+  // a 2-qubit block's chains are half as long (20 layers of U3 + CZ, 7-qubit
+  // tiles: 12 qubits 467 against 687 us, 16 qubits 675 against 973; at 18
+  // qubits, 8-qubit tiles, no difference).
+  const bool small128 = s->dt == SV_C128 && s->n <= kSmall128 && nvec == 1 && !(o && o->prec != SV_PREC_PLAIN);
+  r.fusion_k = (o && o->fusion_k > 0) ? o->fusion_k : (o && o->prec != SV_PREC_PLAIN ? 5 : (small128 ? 2 : 3));
   // default tiles: 13 qubits for single-vector CUDA-core passes on complex64
   // (fewer passes; 32 amplitudes per thread at 256 threads), 12 otherwise
   // (tensor-core tile passes need 12; two-vector and complex128 tiles would
   // crowd shared memory)
   const bool plain64 = s->dt == SV_C64 && nvec == 1 && !(o && o->prec != SV_PREC_PLAIN);
-  r.tile_m = (o && o->tile_m > 0) ? o->tile_m : (plain64 ? 13 : 12 - (nvec - 1));
+  // Small states get smaller tiles, so that their passes reach more SMs:
+  // complex64 up to 2^8 tiles of 11 or 12 qubits (40 layers of U3 + CZ, 18
+  // qubits: 29 passes on 32 SMs 672 us, 40 passes on 128 SMs 382 us; smaller
+  // tiles than 11 qubits cost more in passes than they gain), complex128
+  // tiles of 7 or 8 qubits up to 21 qubits (12 qubits: one pass on one SM
+  // 1926 us, 25 passes 467 us; from 22 qubits on every size fills the GPU).
+  int small_m = 13;
+  if (plain64) small_m = std::max(11, std::min(13, s->n - 8));
+  else if (s->dt == SV_C128 && nvec == 1 && !(o && o->prec != SV_PREC_PLAIN))
+    small_m = s->n <= kSmall128 ? 7 : (s->n <= 21 ? 8 : 12);
+  r.tile_m = (o && o->tile_m > 0) ? o->tile_m : std::min(small_m, plain64 ? 13 : 12 - (nvec - 1));
   // contiguous low qubits in every tile: 64-byte runs for complex64 (three
   // rather than four fixed qubits leave the planner more choice: the
   // 30-qubit grid circuit takes 23 instead of 26 passes, 209 vs 216 ms; two

@@ -75,7 +75,7 @@ void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_load_locked();
   auto it = g_tune.find(tune_key(s->n, s->dt, c));
-  if (it == g_tune.end()) return;
+  if (it == g_tune.end() || it->second.first == 0) return;   // not tuned, or the defaults were fastest
   if (want_k) o.fusion_k = it->second.first;
   if (want_m) o.tile_m = std::min(it->second.second, s->n);
 }
@@ -111,20 +111,23 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
     for (const TilePass &tp : cps[b]->prog.passes) m_max = std::max(m_max, tp.m);
   }
   for (int b = 0; b < B; b++) SV_TRY(upload_program(states[b], *cps[b]));
-  // States whose passes have at least one tile per SM fill the GPU with one
-  // ordinary launch per pass (measured on 256 uneven circuits: 21-qubit
-  // states, 256 tiles a pass, take 15.6 ms as launches against 23.7 ms in
-  // the queue); the persistent queue is for the rest, whose passes alone
-  // would leave most SMs idle.
+  // Wide states run as one ordinary launch per pass, spread over the fan-out
+  // streams; the persistent queue is for the rest, whose passes cost less
+  // than a launch.  The launches take their matrices from parameter blocks
+  // and overlap freely; the queue's tile body reads them from memory and
+  // waits between passes.  48 circuits of depth 40 replayed from a graph:
+  // 20 qubits 40.7 ms in the queue, 18.1 as launches, 17-18 qubits 7.1 and
+  // 4.2, 14-16 qubits 1.84 and 1.97 (but 8.5 and 6.3 for 10-22 qubits
+  // together), 10-13 qubits 1.13 and 1.25.  Without a graph each launch costs
+  // the host 4-5 us, as much as a pass of 19 qubits.
+  const int wide_n = opt && opt->mode == SV_MODE_TILED_GRAPH ? 14 : 19;
   std::vector<char> wide(B, 0);
   for (int b = 0; b < B; b++) {
-    uint64_t min_tiles = ~0ull;
-    for (const TilePass &tp : cps[b]->prog.passes) min_tiles = std::min<uint64_t>(min_tiles, (uint64_t)1 << (tp.n - tp.m));
     bool has_tc = false;
     // (tensor-core and permutation passes have kernels of their own, which
     // the persistent queue does not run)
     for (const TilePass &tp : cps[b]->prog.passes) has_tc |= (tp.flags & (kPassTC | kPassHasTC | kPassTable)) != 0;
-    wide[b] = !cps[b]->prog.passes.empty() && (has_tc || min_tiles >= (uint64_t)s0->sm_count);
+    wide[b] = !cps[b]->prog.passes.empty() && (has_tc || states[b]->n >= wide_n);
   }
   // descriptors in wave order: pass 0 of every state, then pass 1, ...
   std::vector<TilePass> desc;
@@ -159,7 +162,7 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
   // The wide states' passes, as ordinary launches.  The states are
   // independent, so with two or more of them they are spread over the
   // library's fan-out streams (longest first onto the least-loaded stream,
-  // load = tiles x passes), forked from st and joined back into it: one
+  // load = amplitudes x passes), forked from st and joined back into it: one
   // state's passes fill the waves another leaves partly empty, and a stream
   // launches while another's kernel runs.  Recorded in a graph, the streams
   // become parallel branches.
@@ -168,7 +171,8 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
   for (int b = 0; b < B; b++)
     if (wide[b]) {
       wb.push_back(b);
-      for (const TilePass &tp : cps[b]->prog.passes) work[b] += std::ldexp(1.0, tp.n - tp.m);
+      // (a pass of a small state takes about as long as one over 2^18 amplitudes)
+      work[b] = (double)cps[b]->prog.passes.size() * std::ldexp(1.0, std::max(18, states[b]->n));
     }
   const int K = std::min<int>(kFanStreams, (int)wb.size());
   std::vector<int> lane(B, 0);
@@ -383,13 +387,36 @@ sv_status sv_autotune(sv_state *s, const sv_circuit *c, sv_options *inout) {
       }
       if (m == s->n) break;
     }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
   inout->fusion_k = bk;
   inout->tile_m = bm;
-  if (inout->prec != SV_PREC_PLAIN) return SV_OK;   // the cache serves CUDA-core defaults only
+  if (inout->prec != SV_PREC_PLAIN) {   // the cache serves CUDA-core defaults only
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    return SV_OK;
+  }
+  // the defaults for this width, with any earlier choice for the shape out of
+  // the way: where no pair beat them, options left at 0 keep them
+  {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    tune_load_locked();
+    g_tune.erase(tune_key(s->n, s->dt, c));
+  }
+  sv_options def = *inout;
+  def.fusion_k = def.tile_m = 0;
+  def.mode = SV_MODE_TILED;
+  float ms0 = 1e30f;
+  if (sv_apply_circuit(s, c, nullptr, &def) == SV_OK) {
+    cudaEventRecord(e0, s->stream);
+    sv_status st0 = SV_OK;
+    for (int r = 0; r < 2 && st0 == SV_OK; r++) st0 = sv_apply_circuit(s, c, nullptr, &def);
+    cudaEventRecord(e1, s->stream);
+    if (cudaEventSynchronize(e1) != cudaSuccess || st0 != SV_OK || cudaEventElapsedTime(&ms0, e0, e1) != cudaSuccess)
+      ms0 = 1e30f;
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (ms0 <= best) bk = bm = 0;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  tune_load_locked();
   g_tune[tune_key(s->n, s->dt, c)] = {bk, bm};
   tune_save_locked();
   return SV_OK;

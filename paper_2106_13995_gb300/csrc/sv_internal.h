@@ -80,9 +80,13 @@ constexpr uint8_t kGenInline = 0x40;     // TileOp.gen flag: matrix in the launc
 // Parameter block of a complex64 single-vector tile pass: its op list and
 // the matrices of its 1-3 qubit dense blocks, read by every CTA with
 // warp-uniform loads (matrices as row pairs, see dense_pairs).  Passes that
-// do not fit keep the global copies.
+// do not fit keep the global copies.  A launch copies its whole parameter
+// block (about 15 us of host time for 30 KB, 4 for 6), so blocks come in
+// three sizes: ten, twenty or fifty 3-qubit matrices.
 constexpr int kInlOps = 48;
 constexpr int kInlMat = 3200;    // complex64 entries
+constexpr int kInlMidOps = 24, kInlMidMat = 1280;
+constexpr int kInlSmallOps = 12, kInlSmallMat = 640;
 // groups per trip of the packed complex64 blocks from the parameter block
 constexpr int pairs_groups(int k) { return k <= 2 ? 4 : 2; }
 // Per-op set-up of a parameter-block dense block, computed on the host for
@@ -97,12 +101,16 @@ struct OpPre {
 };
 // OpPre of a 1-3 qubit dense op for a launch with `threads` threads (k_tile.cu)
 void fill_op_pre(const TileOp &op, int threads, OpPre &pre);
-struct TileInline {
+template <int NOPS, int NMAT> struct TileInlineN {
+  static constexpr int kOps = NOPS, kMat = NMAT;
   uint32_t nops, nmat;
-  TileOp ops[kInlOps];
-  OpPre pre[kInlOps];
-  float2 mats[kInlMat];
+  TileOp ops[NOPS];
+  OpPre pre[NOPS];
+  float2 mats[NMAT];
 };
+using TileInline = TileInlineN<kInlOps, kInlMat>;
+using TileInlineMid = TileInlineN<kInlMidOps, kInlMidMat>;
+using TileInlineSmall = TileInlineN<kInlSmallOps, kInlSmallMat>;
 // TilePass.flags: this entry is not a tile pass but one dense block of L = 5
 // or 6 qubits on the tensor cores; hi_pos[0..L) hold its targets, mat0 the
 // 16-byte index of its packed operand in the matrix pool, bits 9..10 the
@@ -233,7 +241,7 @@ struct DeviceProgram {
 }  // namespace sv
 
 // streams over which a batched call spreads its wide states
-constexpr int kFanStreams = 4;
+constexpr int kFanStreams = 8;
 
 struct sv_state {
   int n = 0;
@@ -318,9 +326,11 @@ struct Opts {   // all int: hashed as key bytes, so no padding
   int fusion_k, tile_m, L, prec, mode;
   int tc_in_tile = 0;
 };
+constexpr int kSmall128 = 17;   // widest complex128 state with the small-state plan
 Opts resolve(const sv_state *s, const sv_options *o, int nvec);
 // Fill fusion_k / tile_m that the caller left at 0 from the autotuner's
-// cache for this circuit's shape (sv_batch.cu).
+// cache for this circuit's shape (sv_batch.cu), if a pair in it beat the
+// defaults.
 void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt, Opts &o);
 // ---------------------------------------------------------------------------
 // program caches

@@ -233,9 +233,9 @@ __device__ __forceinline__ uint64_t lds_b64(uint32_t a) {
 // the launch's parameter block (warp-uniform reads take the uniform
 // datapath) or from global memory through L1, with the same arithmetic, so
 // every kernel that applies these blocks produces the same bits.
-struct ParamPairs {
+template <class Inl> struct ParamPairs {
   static constexpr bool kPre = true;   // set-up from the host (OpPre)
-  const TileInline &I;
+  const Inl &I;
   uint32_t base;
   uint32_t oi;
   template <int D>
@@ -370,9 +370,20 @@ __device__ __forceinline__ void dense_pairs_global(float2 *v, int m, const TileO
 
 // Dense complex64 block of 1-3 qubits whose matrix is in the launch's
 // parameter block (op.mat indexes TileInline::mats, stored as row pairs).
-__device__ __forceinline__ void apply_op_inl(float2 *v, int m, const TileOp &op, const TileInline &I, int oi,
-                                             uint32_t tid, uint32_t T) {
-  const ParamPairs src{I, op.mat, (uint32_t)oi};
+template <class Inl>
+__device__ __forceinline__ void apply_op_inl(float2 *v, int m, const TileOp &op, const Inl &I, int oi, uint32_t tid,
+                                             uint32_t T) {
+  const ParamPairs<Inl> src{I, op.mat, (uint32_t)oi};
+  if ((T << (op.k + __popc(op.lcmask))) >> m) {
+    // at most one group per thread (small states): further groups of a trip
+    // would only repeat its arithmetic
+    switch (op.k) {
+      case 1: dense_pairs<1, 1>(v, m, op, src, tid, T); break;
+      case 2: dense_pairs<2, 1>(v, m, op, src, tid, T); break;
+      default: dense_pairs<3, 1>(v, m, op, src, tid, T); break;
+    }
+    return;
+  }
   switch (op.k) {
     case 1: dense_pairs<1, kPairsG<1>>(v, m, op, src, tid, T); break;
     case 2: dense_pairs<2, kPairsG<2>>(v, m, op, src, tid, T); break;
