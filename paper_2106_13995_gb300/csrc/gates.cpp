@@ -118,55 +118,64 @@ std::vector<cd> adjoint_of(const std::vector<cd> &U, int k) {
   return A;
 }
 
-sv_status circuit_to_gates(const sv_circuit *c, const double *params, int n,
-                           std::vector<Gate> &out, bool keep_params_unfused) {
+static sv_status check_width(const sv_circuit *c, int n) {
   if (!c || (c->n_ops > 0 && !c->ops)) return set_error(SV_EINVAL, "null circuit");
   if (c->n_qubits != n)
     return set_error(SV_EINVAL, "circuit width " + std::to_string(c->n_qubits) +
                                     " does not match the state's " + std::to_string(n));
+  return SV_OK;
+}
+
+// Op i of a circuit of the right width, validated.  g's vectors are reused.
+static sv_status op_to_gate(const sv_circuit *c, int i, const double *params, int n, bool keep_params_unfused, Gate &g) {
+  const sv_op &op = c->ops[i];
+  auto fail = [&](const std::string &what) { return set_error(SV_EINVAL, "op " + std::to_string(i) + ": " + what); };
+  int ar = gate_arity(op.gate);
+  if (ar < 0) return fail("unknown gate id " + std::to_string(op.gate));
+  int k = op.n_targets;
+  if (ar == 0 ? (k < 1 || k > 6) : k != ar) return fail("wrong number of targets");
+  if (op.n_controls < 0 || op.n_controls > 8) return fail("0..8 controls allowed");
+  uint64_t seen = 0;
+  g.targets.clear();
+  g.controls.clear();
+  for (int j = 0; j < k + op.n_controls; j++) {
+    int q = j < k ? op.targets[j] : op.controls[j - k];
+    if (q < 0 || q >= n) return fail("qubit out of range");
+    if ((seen >> q) & 1) return fail("duplicate qubit");
+    seen |= 1ull << q;
+    (j < k ? g.targets : g.controls).push_back(q);
+  }
+  if (op.gate == SV_GATE_MATRIX) {
+    if (!c->matrices || op.matrix_offset < 0) return fail("MATRIX op without a matrix");
+    const int d = 1 << k;
+    g.U.resize(d * d);
+    const double *m = c->matrices + 2 * op.matrix_offset;
+    for (int e = 0; e < d * d; e++) g.U[e] = cd(m[2 * e], m[2 * e + 1]);
+    if (unitarity_checks() && unitarity_error(g.U, k) > kUnitaryTol)
+      return fail("matrix is not unitary (max |U^dagger U - I| = " + std::to_string(unitarity_error(g.U, k)) + ")");
+  } else {
+    double ang[3] = {op.angles[0], op.angles[1], op.angles[2]};
+    if (op.param >= 0) {
+      if (op.param >= c->n_params) return fail("param index out of range");
+      if (!params) return fail("parametric op but params is NULL");
+      ang[0] = params[op.param];
+      g.param = op.param;
+      g.param_gate = op.gate;
+      g.fixed_structure = keep_params_unfused;
+    }
+    gate_matrix(op.gate, ang, g.U);
+  }
+  return SV_OK;
+}
+
+sv_status circuit_to_gates(const sv_circuit *c, const double *params, int n,
+                           std::vector<Gate> &out, bool keep_params_unfused) {
+  SV_TRY(check_width(c, n));
   out.clear();
   out.reserve(c->n_ops);
   for (int i = 0; i < c->n_ops; i++) {
-    const sv_op &op = c->ops[i];
-    const std::string where = "op " + std::to_string(i) + ": ";
-    int ar = gate_arity(op.gate);
-    if (ar < 0) return set_error(SV_EINVAL, where + "unknown gate id " + std::to_string(op.gate));
-    int k = op.n_targets;
-    if (ar == 0 ? (k < 1 || k > 6) : k != ar)
-      return set_error(SV_EINVAL, where + "wrong number of targets");
-    if (op.n_controls < 0 || op.n_controls > 8)
-      return set_error(SV_EINVAL, where + "0..8 controls allowed");
-    uint64_t seen = 0;
     Gate g;
-    for (int j = 0; j < k + op.n_controls; j++) {
-      int q = j < k ? op.targets[j] : op.controls[j - k];
-      if (q < 0 || q >= n) return set_error(SV_EINVAL, where + "qubit out of range");
-      if ((seen >> q) & 1) return set_error(SV_EINVAL, where + "duplicate qubit");
-      seen |= 1ull << q;
-      (j < k ? g.targets : g.controls).push_back(q);
-    }
-    if (op.gate == SV_GATE_MATRIX) {
-      if (!c->matrices || op.matrix_offset < 0)
-        return set_error(SV_EINVAL, where + "MATRIX op without a matrix");
-      const int d = 1 << k;
-      g.U.resize(d * d);
-      const double *m = c->matrices + 2 * op.matrix_offset;
-      for (int e = 0; e < d * d; e++) g.U[e] = cd(m[2 * e], m[2 * e + 1]);
-      if (unitarity_checks() && unitarity_error(g.U, k) > kUnitaryTol)
-        return set_error(SV_EINVAL, where + "matrix is not unitary (max |U^dagger U - I| = " +
-                                        std::to_string(unitarity_error(g.U, k)) + ")");
-    } else {
-      double ang[3] = {op.angles[0], op.angles[1], op.angles[2]};
-      if (op.param >= 0) {
-        if (op.param >= c->n_params) return set_error(SV_EINVAL, where + "param index out of range");
-        if (!params) return set_error(SV_EINVAL, where + "parametric op but params is NULL");
-        ang[0] = params[op.param];
-        g.param = op.param;
-        g.param_gate = op.gate;
-        g.fixed_structure = keep_params_unfused;
-      }
-      gate_matrix(op.gate, ang, g.U);
-    }
+    SV_TRY(op_to_gate(c, i, params, n, keep_params_unfused, g));
     out.push_back(std::move(g));
   }
   return SV_OK;
@@ -195,30 +204,49 @@ bool unitarity_checks() {
 #endif
 }
 
-bool propagate_basis(const std::vector<Gate> &gates, uint64_t &index, cd &amp) {
-  for (const Gate &g : gates) {
-    if (g.grad_gen > 0) return false;
-    bool on = true;
-    for (int q : g.controls) on = on && ((index >> q) & 1ull);
-    if (!on) continue;
-    const int k = (int)g.targets.size(), d = 1 << k;
-    int c = 0;
-    for (int j = 0; j < k; j++) c |= (int)((index >> g.targets[j]) & 1ull) << j;
-    // column c of U must hold exactly one nonzero entry
-    int r1 = -1;
-    for (int r = 0; r < d; r++)
-      if (g.U[(size_t)r * d + c] != cd(0.0)) {
-        if (r1 >= 0) return false;
-        r1 = r;
-      }
-    if (r1 < 0) return false;
-    amp *= g.U[(size_t)r1 * d + c];
-    for (int j = 0; j < k; j++) {
-      const uint64_t bit = 1ull << g.targets[j];
-      index = ((r1 >> j) & 1) ? (index | bit) : (index & ~bit);
+// Follow a basis state through one gate.
+static bool propagate_gate(const Gate &g, uint64_t &index, cd &amp) {
+  if (g.grad_gen > 0) return false;
+  for (int q : g.controls)
+    if (!((index >> q) & 1ull)) return true;
+  const int k = (int)g.targets.size(), d = 1 << k;
+  int c = 0;
+  for (int j = 0; j < k; j++) c |= (int)((index >> g.targets[j]) & 1ull) << j;
+  // column c of U must hold exactly one nonzero entry
+  int r1 = -1;
+  for (int r = 0; r < d; r++)
+    if (g.U[(size_t)r * d + c] != cd(0.0)) {
+      if (r1 >= 0) return false;
+      r1 = r;
     }
+  if (r1 < 0) return false;
+  amp *= g.U[(size_t)r1 * d + c];
+  for (int j = 0; j < k; j++) {
+    const uint64_t bit = 1ull << g.targets[j];
+    index = ((r1 >> j) & 1) ? (index | bit) : (index & ~bit);
   }
   return true;
+}
+
+bool propagate_basis(const std::vector<Gate> &gates, uint64_t &index, cd &amp) {
+  for (const Gate &g : gates)
+    if (!propagate_gate(g, index, amp)) return false;
+  return true;
+}
+
+// Most circuits leave the basis states at their first gates, so ops are
+// converted one at a time: converting all of them cost a call on a small state
+// more than its launches (1080 gates: about 100 us).
+sv_status propagate_circuit(const sv_circuit *c, const double *params, int n, uint64_t &index, cd &amp, bool &stays) {
+  SV_TRY(check_width(c, n));
+  stays = false;
+  Gate g;
+  for (int i = 0; i < c->n_ops; i++) {
+    SV_TRY(op_to_gate(c, i, params, n, false, g));
+    if (!propagate_gate(g, index, amp)) return SV_OK;
+  }
+  stays = true;
+  return SV_OK;
 }
 
 }  // namespace sv

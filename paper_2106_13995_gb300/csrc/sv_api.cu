@@ -93,9 +93,23 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
 // ---------------------------------------------------------------------------
 uint64_t KeyBytes::hash() const {
   // 8 bytes per step, each word mixed by a multiply-xorshift (splitmix64's
-  // finaliser); only a bucket index: equal hashes are compared byte for byte
+  // finaliser), in four independent chains while 32 bytes are left; only a
+  // bucket index: equal hashes are compared byte for byte
   uint64_t h = 0x243F6A8885A308D3ull ^ (uint64_t)b.size();
   size_t i = 0;
+  uint64_t l[4] = {h, ~h, h + 0x9E3779B97F4A7C15ull, h ^ 0x94D049BB133111EBull};
+  for (; i + 32 <= b.size(); i += 32) {
+    uint64_t w[4];
+    std::memcpy(w, b.data() + i, 32);
+    for (int j = 0; j < 4; j++) {
+      l[j] = (l[j] ^ w[j]) * 0x9E3779B97F4A7C15ull;
+      l[j] ^= l[j] >> 29;
+    }
+  }
+  for (int j = 0; j < 4; j++) {
+    h = (h ^ l[j]) * 0x9E3779B97F4A7C15ull;
+    h ^= h >> 29;
+  }
   for (; i + 8 <= b.size(); i += 8) {
     uint64_t w;
     std::memcpy(&w, b.data() + i, 8);
@@ -109,6 +123,7 @@ uint64_t KeyBytes::hash() const {
 }
 
 void circuit_key(KeyBytes &k, const sv_circuit *c) {
+  k.b.reserve(k.b.size() + sizeof(sv_op) * (size_t)std::max(0, c->n_ops) + sizeof(double) * (size_t)std::max(0, c->n_params) + 256);
   k.val(c->n_qubits);
   k.val(c->n_ops);
   k.val(c->n_params);
@@ -1016,11 +1031,11 @@ sv_status sv_apply_circuit(sv_state *s, const sv_circuit *c, const double *param
     // a basis state through permutation and phase gates stays a basis
     // state: follow it on the host and rewrite two amplitudes, with no pass
     // over the state (exact: only the FP64 phases are rounded, once)
-    std::vector<Gate> gates;
-    SV_TRY(circuit_to_gates(c, params, s->n, gates, false));
     uint64_t idx = s->basis_index;
     cd amp = s->basis_amp;
-    if (propagate_basis(gates, idx, amp)) {
+    bool stays = false;
+    SV_TRY(propagate_circuit(c, params, s->n, idx, amp, stays));
+    if (stays) {
       SV_TRY(launch_move_basis(s, s->basis_index, idx, amp));
       s->basis_index = idx;
       s->basis_amp = amp;

@@ -447,6 +447,8 @@ sv_status launch_copy16(sv_state *s, const void *src, void *dst, size_t bytes);
 // phase (permutations, diagonal and monomial gates, with controls); false,
 // leaving index and amp unspecified, as soon as one gate does not.
 bool propagate_basis(const std::vector<Gate> &gates, uint64_t &index, cd &amp);
+// the same for a circuit, op by op; stays: every gate kept it a basis state
+sv_status propagate_circuit(const sv_circuit *c, const double *params, int n, uint64_t &index, cd &amp, bool &stays);
 sv_status launch_scale(sv_state *s, double factor);
 sv_status launch_dense_gate(sv_state *s, const std::vector<int> &targets,
                             const std::vector<int> &controls, const std::vector<cd> &U);
