@@ -392,8 +392,10 @@ int tile_threads(int m, sv_dtype dt) {
 // Threads of a pass of `tiles` tiles.  32 amplitudes a thread pay each op's
 // set-up once for many, but a pass whose tiles leave the GPU mostly empty is a
 // chain of latencies: there, up to a thread per group of 8 amplitudes.
-static int pass_threads(const sv_state *s, int m, uint64_t tiles) {
-  int t = tile_threads(m, s->dt);
+// Two-vector tiles take twice the threads: shared memory holds half as many of
+// them per SM.
+static int pass_threads(const sv_state *s, int m, int nvec, uint64_t tiles) {
+  int t = std::min(kTilePassThreads, tile_threads(m, s->dt) * nvec);
   const int most = std::min(kTilePassThreads, std::max(32, 1 << std::max(0, m - 3)));
   while (t < most && tiles * (uint64_t)t < (uint64_t)s->sm_count * 512) t *= 2;
   return t;
@@ -510,7 +512,8 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
   }
   if (smem > (200u << 10)) return set_error(SV_EINVAL, "tile too large for shared memory");
   dim3 grid((unsigned)(1ull << (p.n - p.m)), (unsigned)batch);
-  const int threads = pass_threads(s, p.m, (uint64_t)grid.x * grid.y);
+  const int threads = pass_threads(s, p.m, (int)p.nvec, (uint64_t)grid.x * grid.y);
+  if (host && sites_pass_ok(p, *host)) return launch_tile_sites(s, p, batch, threads, stream);
   sv_status st = SV_OK;
   const bool try_inl = host && s->dt == SV_C64 && batch == 1 && p.nvec == 1;
   if (try_inl && (launch_inl<TileInlineSmall>(s, p, *host, grid, threads, smem, stream, st) ||

@@ -253,4 +253,150 @@ std::vector<Block> merge_in_passes(const std::vector<PassPlan> &passes, int K) {
   return out;
 }
 
+// An op of site_blocks under construction.
+namespace {
+struct SiteOp {
+  Block b;
+  uint64_t touched_post = 0;   // qubits of moves after the sites
+  uint64_t has_site = 0;
+};
+// Append "member y of the gate's qubits goes to perm[y]" to a table over the
+// op's qubits.
+void append_move(uint8_t *tab, const std::vector<int> &opq, const std::vector<int> &Q, const int *perm) {
+  for (int y = 0; y < 8; y++) {
+    const int v = tab[y];
+    int c = 0;
+    for (size_t j = 0; j < Q.size(); j++) c |= ((v >> index_of(opq, Q[j])) & 1) << j;
+    const int r = perm[c];
+    int w = v;
+    for (size_t j = 0; j < Q.size(); j++) {
+      const int bit = 1 << index_of(opq, Q[j]);
+      w = ((r >> j) & 1) ? (w | bit) : (w & ~bit);
+    }
+    tab[y] = (uint8_t)w;
+  }
+}
+}  // namespace
+
+std::vector<Block> site_blocks(const std::vector<Gate> &gates, int K, std::vector<AdjSite> &sites) {
+  std::vector<SiteOp> ops;
+  std::vector<int> last(64, -1);
+  std::vector<std::vector<int>> waiting(64);   // parametric gates not placed yet, by qubit
+  auto is_sites = [&](int o) { return o >= 0 && ops[o].b.kind == TOP_SITES; };
+  // give qubit q (of op o) its waiting gates as a site; o's sites on q come
+  // before any move after the sites
+  auto place = [&](int o, int q) {
+    if (waiting[q].empty()) return;
+    Block &b = ops[o].b;
+    int &s = b.site[index_of(b.qubits, q)];
+    if (s < 0) {
+      s = (int)sites.size();
+      sites.emplace_back();
+    }
+    sites[s].insert(sites[s].end(), waiting[q].begin(), waiting[q].end());
+    waiting[q].clear();
+    ops[o].has_site |= 1ull << q;
+    last[q] = std::max(last[q], o);
+  };
+  auto new_op = [&]() {
+    SiteOp n;
+    n.b.kind = TOP_SITES;
+    n.b.fusable = false;
+    ops.push_back(std::move(n));
+    return (int)ops.size() - 1;
+  };
+  // waiting gates of q that can only go to an op of their own (with other
+  // qubits' waiting gates, neighbours first)
+  auto place_alone = [&](int q) {
+    if (waiting[q].empty()) return;
+    if (is_sites(last[q]) && !((ops[last[q]].touched_post >> q) & 1)) return place(last[q], q);
+    const int o = new_op();
+    for (int d = 0; d < 64 && ops[o].b.qubits.size() < 3; d++)
+      for (int x : {q + d, q - d}) {
+        if (x < 0 || x >= 64 || waiting[x].empty() || ops[o].b.qubits.size() >= 3) continue;
+        ops[o].b.qubits.push_back(x);
+        place(o, x);
+      }
+  };
+  for (const Gate &g : gates) {
+    std::vector<int> Q = g.targets;
+    Q.insert(Q.end(), g.controls.begin(), g.controls.end());
+    if (g.inst >= 0) {
+      const int q = Q[0], o = last[q];
+      waiting[q].push_back(g.inst);
+      // at once if the last op on q takes it; else with the next gate on q
+      if (is_sites(o) && !((ops[o].touched_post >> q) & 1)) place(o, q);
+      continue;
+    }
+    int perm[64];
+    std::vector<cd> E;
+    const bool narrow = Q.size() <= 3;
+    if (narrow) E = embed(g.U, g.targets, g.controls, Q);
+    if (narrow && permutation_of(E, (int)Q.size(), perm)) {
+      int o = -1;
+      for (int q : Q) o = std::max(o, last[q]);
+      bool join = is_sites(o);
+      if (join) {
+        std::vector<int> uni = ops[o].b.qubits;
+        for (int q : Q)
+          if (index_of(uni, q) < 0) uni.push_back(q);
+        join = uni.size() <= 3;
+        // a qubit with gates waiting behind a move of this op needs another op
+        for (int q : Q) join = join && (waiting[q].empty() || !((ops[o].touched_post >> q) & 1));
+        if (join) ops[o].b.qubits = uni;
+      }
+      if (!join) {
+        o = new_op();
+        ops[o].b.qubits = Q;
+      }
+      for (int q : Q) place(o, q);
+      const uint64_t m = qmask(Q);
+      const bool pre = !(m & (ops[o].has_site | ops[o].touched_post));
+      append_move(pre ? ops[o].b.pre : ops[o].b.post, ops[o].b.qubits, Q, perm);
+      if (!pre) ops[o].touched_post |= m;
+      for (int q : Q) last[q] = o;
+      continue;
+    }
+    // a dense block, fused as in fuse()
+    for (int q : Q) place_alone(q);
+    int o = -1;
+    for (int q : Q) o = std::max(o, last[q]);
+    const bool alone = K <= 1 || g.controls.size() >= 2 || (int)Q.size() > K;
+    if (!alone && o >= 0 && ops[o].b.kind == TOP_DENSE && ops[o].b.fusable) {
+      Block &b = ops[o].b;
+      std::vector<int> uni = b.qubits;
+      for (int q : Q)
+        if (index_of(uni, q) < 0) uni.push_back(q);
+      if ((int)uni.size() <= K) {
+        const std::vector<cd> Ub = embed(b.U, b.qubits, {}, uni);
+        const std::vector<cd> Ug = embed(g.U, g.targets, g.controls, uni);
+        b.U = matmul(Ug, Ub, 1 << (int)uni.size());
+        b.qubits = uni;
+        for (int q : uni) last[q] = std::max(last[q], o);
+        continue;
+      }
+    }
+    SiteOp n;
+    if (alone) {
+      n.b.qubits = g.targets;
+      n.b.controls = g.controls;
+      n.b.U = g.U;
+      n.b.fusable = K > 1 && g.controls.empty();
+    } else {
+      n.b.qubits = Q;
+      n.b.U = embed(g.U, g.targets, g.controls, Q);
+    }
+    ops.push_back(std::move(n));
+    for (int q : Q) last[q] = (int)ops.size() - 1;
+  }
+  for (int q = 0; q < 64; q++) place_alone(q);
+  std::vector<Block> out;
+  out.reserve(ops.size());
+  for (SiteOp &o : ops) {
+    if (o.b.kind == TOP_DENSE) o.b.diag = is_diagonal(o.b.U, (int)o.b.qubits.size());
+    out.push_back(std::move(o.b));
+  }
+  return out;
+}
+
 }  // namespace sv

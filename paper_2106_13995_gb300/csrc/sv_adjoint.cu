@@ -29,6 +29,14 @@ struct AdjointProgram {
   std::vector<int> inst_gate;    // sv_gate of each parametric instance
   int n_params = 0;
   int n_inst = 0;
+  // programs of sites (see site_blocks): the sites of both sweeps, and each
+  // reverse site's first accumulator and components (bits: X, Y, Z);
+  // without them one matrix per instance and one accumulator per parameter
+  bool sites = false;
+  std::vector<AdjSite> fwd_sites, rev_sites;
+  std::vector<int> rev_slot, rev_comps;
+  int n_acc = 0;                 // accumulators, the energy's excluded
+  int n_mats = 0;                // per-batch 2 x 2 matrices
 };
 
 static ProgCache<AdjointProgram> g_adj_cache(64);
@@ -62,6 +70,25 @@ void drop_adjoint_programs(const sv_state *s) {
   }
 }
 
+// Passes of TOP_SITES ops have a kernel of their own: split a pass where it
+// changes between them and other ops, and beyond the kernel's op count.
+static std::vector<PassPlan> split_sites(const std::vector<PassPlan> &passes) {
+  std::vector<PassPlan> out;
+  for (const PassPlan &P : passes) {
+    size_t i = 0;
+    do {
+      PassPlan Q;
+      Q.S = P.S;
+      const bool sites = i < P.ops.size() && P.ops[i].kind == TOP_SITES;
+      while (i < P.ops.size() && (P.ops[i].kind == TOP_SITES) == sites &&
+             (!sites || Q.ops.size() < (size_t)kMaxSitesOps))
+        Q.ops.push_back(P.ops[i++]);
+      out.push_back(std::move(Q));
+    } while (i < P.ops.size());
+  }
+  return out;
+}
+
 static void append_passes(DeviceProgram &prog, std::vector<uint32_t> &op0s, const std::vector<PassPlan> &passes,
                           const BuildCtx &b, const std::vector<int> &bmo, sv_status &st) {
   for (const PassPlan &P : passes) {
@@ -71,7 +98,7 @@ static void append_passes(DeviceProgram &prog, std::vector<uint32_t> &op0s, cons
 }
 
 static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *params0,
-                               const sv_pauli_term *terms, int nt, const Opts &o1, const Opts &o2,
+                               const sv_pauli_term *terms, int nt, const Opts &o1, const Opts &o2, bool sites,
                                AdjointProgram &A) {
   std::vector<Gate> gates;
   SV_TRY(circuit_to_gates(c, params0, s->n, gates, true));
@@ -86,6 +113,29 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     A.inst_gate.push_back(g.param_gate);
   }
   const int G = (int)gates.size();
+  A.sites = sites;
+  A.n_acc = A.n_params;
+  A.n_mats = 2 * A.n_inst;
+  std::vector<Block> fwd_blocks, rev_blocks;
+  std::vector<int> fwd_mat, rev_mat;
+  if (sites) {
+    fwd_blocks = site_blocks(gates, o1.fusion_k, A.fwd_sites);
+    std::vector<Gate> rev(gates.rbegin(), gates.rend());
+    for (Gate &g : rev) g.U = adjoint_of(g.U, (int)g.targets.size());
+    rev_blocks = site_blocks(rev, o2.fusion_k, A.rev_sites);
+    A.n_acc = 0;
+    for (const AdjSite &st : A.rev_sites) {
+      int c = 0;
+      for (int i : st) c |= 1 << (std::min(3, gate_generator(A.inst_gate[i])) - 1);
+      if (st.size() > 1) c |= 7;   // later gates' generators turn into the other two
+      A.rev_slot.push_back(A.n_acc);
+      A.rev_comps.push_back(c);
+      A.n_acc += __builtin_popcount(c);
+    }
+    for (size_t i = 0; i < A.fwd_sites.size(); i++) fwd_mat.push_back(4 * (int)i);
+    for (size_t i = 0; i < A.rev_sites.size(); i++) rev_mat.push_back(4 * (int)(A.fwd_sites.size() + i));
+    A.n_mats = (int)(A.fwd_sites.size() + A.rev_sites.size());
+  }
   std::vector<int> fwd_off(A.n_inst), rev_off(A.n_inst);
   for (int i = 0; i < A.n_inst; i++) {
     fwd_off[i] = 4 * i;
@@ -94,14 +144,15 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
   sv_status st = SV_OK;
   // forward
   {
-    std::vector<Block> blocks = fuse(gates, o1.fusion_k);
+    std::vector<Block> blocks = sites ? std::move(fwd_blocks) : fuse(gates, o1.fusion_k);
     int m = o1.tile_m, L = o1.L;
     if (!fit_tile(blocks, s->n, lmin(s->dt), mmax(s->dt, 1), m, L))
       return set_error(SV_EUNSUPPORTED, "a fused block does not fit a shared-memory tile");
     std::vector<PassPlan> passes = plan_passes(blocks, s->n, m, L, 256, 1 << 16);
     if (passes.empty() && !blocks.empty()) return set_error(SV_EINVAL, "internal: pass planning failed");
     BuildCtx b{s->dt, s->n, m, L, 1, 0};
-    append_passes(A.prog, A.op0s, passes, b, fwd_off, st);
+    b.site_mat = fwd_mat.data();
+    append_passes(A.prog, A.op0s, split_sites(passes), b, fwd_off, st);
   }
   // lambda = H psi
   {
@@ -132,7 +183,7 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     passes.front().ops.insert(passes.front().ops.begin(), zero);
     Block dot;
     dot.kind = TOP_DOT;
-    dot.slot = A.n_params;
+    dot.slot = A.n_acc;
     passes.back().ops.push_back(dot);
     for (size_t i = 0; i < passes.size() && st == SV_OK; i++) {
       BuildCtx b{s->dt, s->n, m, L, 2, (i == 0 ? 1u : 0u) | 2u};
@@ -143,7 +194,7 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
   {
     std::vector<Gate> rev;
     rev.reserve(2 * G);
-    for (int j = G - 1; j >= 0; j--) {
+    for (int j = G - 1; j >= 0 && !sites; j--) {
       const Gate &g = gates[j];
       if (g.param >= 0) {
         Gate probe;
@@ -156,18 +207,70 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
       u.U = adjoint_of(g.U, (int)g.targets.size());
       rev.push_back(u);
     }
-    std::vector<Block> blocks = fuse(rev, o2.fusion_k);
+    std::vector<Block> blocks = sites ? std::move(rev_blocks) : fuse(rev, o2.fusion_k);
     for (Block &b : blocks)
-      if (b.kind == TOP_DENSE) b.vmask = 3;
+      if (b.kind == TOP_DENSE || b.kind == TOP_SITES) b.vmask = 3;
     int m = o2.tile_m, L = o2.L;
     if (!fit_tile(blocks, s->n, lmin(s->dt), mmax(s->dt, 2), m, L))
       return set_error(SV_EUNSUPPORTED, "a fused block does not fit a shared-memory tile");
     std::vector<PassPlan> passes = plan_passes(blocks, s->n, m, L, 256, 1 << 16);
     if (passes.empty() && !blocks.empty()) return set_error(SV_EINVAL, "internal: pass planning failed");
     BuildCtx b{s->dt, s->n, m, L, 2, 0};
-    append_passes(A.prog, A.op0s, passes, b, rev_off, st);
+    b.site_mat = rev_mat.data();
+    b.site_slot = A.rev_slot.data();
+    b.site_comps = A.rev_comps.data();
+    append_passes(A.prog, A.op0s, split_sites(passes), b, rev_off, st);
   }
   return st;
+}
+
+// One matrix per site: the product of its gates' matrices (adjoints in the
+// reverse sweep), in FP64.
+static void put_site_mats(std::vector<uint8_t> &pool, const AdjointProgram &A, const double *theta) {
+  std::vector<cd> U;
+  for (int pass = 0; pass < 2; pass++)
+    for (const AdjSite &st : pass == 0 ? A.fwd_sites : A.rev_sites) {
+      cd M[4] = {1.0, 0.0, 0.0, 1.0};
+      for (int i : st) {
+        const double ang[3] = {theta[A.inst_param[i]], 0, 0};
+        gate_matrix(A.inst_gate[i], ang, U);
+        if (pass == 1) U = adjoint_of(U, 1);
+        const cd N[4] = {U[0] * M[0] + U[1] * M[2], U[0] * M[1] + U[1] * M[3], U[2] * M[0] + U[3] * M[2],
+                         U[2] * M[1] + U[3] * M[3]};
+        std::memcpy(M, N, sizeof(M));
+      }
+      put_pairs_c64(pool, M, 1);
+    }
+}
+
+// The gradients of a site from its components: p_G = Im <lambda| G |psi> at
+// the run's start.  Undoing U = exp(-i theta P / 2) on both vectors turns p_G
+// into Im <lambda| U G U^dagger |psi>, a rotation of (X, Y, Z) about P.
+static void site_grads(const AdjointProgram &A, const double *theta, const double *acc, double *grad) {
+  for (size_t k = 0; k < A.rev_sites.size(); k++) {
+    double p[3] = {0, 0, 0};   // X, Y, Z
+    int at = A.rev_slot[k];
+    for (int g = 0; g < 3; g++)
+      if ((A.rev_comps[k] >> g) & 1) p[g] = acc[at++];
+    for (int i : A.rev_sites[k]) {
+      const int gen = gate_generator(A.inst_gate[i]);
+      // PHASE's generator diag(0, -2) is Z - I, and <lambda|psi> = <psi|H|psi>
+      // has no imaginary part
+      grad[A.inst_param[i]] += p[std::min(gen, 3) - 1];
+      const double c = std::cos(theta[A.inst_param[i]]), s = std::sin(theta[A.inst_param[i]]);
+      const double x = p[0], y = p[1], z = p[2];
+      if (gen == 1) {
+        p[1] = c * y + s * z;
+        p[2] = c * z - s * y;
+      } else if (gen == 2) {
+        p[2] = c * z + s * x;
+        p[0] = c * x - s * z;
+      } else {
+        p[0] = c * x + s * y;
+        p[1] = c * y - s * x;
+      }
+    }
+  }
 }
 
 template <typename R>
@@ -220,7 +323,12 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
   // ansatz): fusion width 2 and 12-qubit tiles for both sweeps
   if (!opt || opt->fusion_k == 0) o1.fusion_k = o2.fusion_k = 2;
   if (!opt || opt->tile_m == 0) {
-    o1.tile_m = o2.tile_m = std::min(12, s->n);
+    // (12-qubit tiles; 10 for small states and few sets, whose tiles would
+    // not fill the GPU: one set of 16 qubits 441 -> 329 us, of 18 qubits
+    // 497 -> 398; at 20 qubits 700 -> 776)
+    int lb = 0;
+    while ((2 << lb) <= B) lb++;
+    o1.tile_m = o2.tile_m = std::min(s->dt == SV_C64 && s->n + lb <= 18 ? 10 : 12, s->n);
     o1.L = o2.L = std::min(o1.L, o1.tile_m);
   }
   // cache key: circuit structure, terms, options (parameters enter only the
@@ -232,20 +340,28 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
   k.val(o1);
   k.val(o2);
   k.val(s->dt);
+  // complex64 programs are made of sites (their accumulators, at most one and
+  // a half per parametric gate, fit the reduction area whenever the gates'
+  // matrices fit the program area); complex128 ones are bound by FP64
+  // arithmetic, which the probes of three components a site would add to
+  const bool sites = s->dt == SV_C64 && s->n >= 3 && o1.tile_m >= 3 && o2.tile_m >= 3;
+  const int np = c->n_params;
+  k.val((int)sites);
   const uint64_t kh = k.hash();
   std::shared_ptr<const AdjointProgram> Ap = g_adj_cache.find(s, k, kh);
   if (!Ap) {
     auto built = std::make_shared<AdjointProgram>();
-    SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, *built));
+    SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, sites, *built));
     built->serial = next_program_serial();
     Ap = g_adj_cache.insert(s, k, kh, std::move(built));
   }
   const AdjointProgram &A = *Ap;
-  const int np = c->n_params;
   // per-batch matrices, state pointer tables
   std::vector<uint8_t> pm;
+  pm.reserve((size_t)B * A.n_mats * 4 * (s->dt == SV_C64 ? 8 : 16));
   for (int b = 0; b < B; b++) {
-    if (s->dt == SV_C64) put_mats<float>(pm, A, params + (size_t)b * np);
+    if (A.sites) put_site_mats(pm, A, params + (size_t)b * np);
+    else if (s->dt == SV_C64) put_mats<float>(pm, A, params + (size_t)b * np);
     else put_mats<double>(pm, A, params + (size_t)b * np);
   }
   std::vector<void *> tbl(2 * (size_t)B);
@@ -261,7 +377,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
                        {tbl.data(), tbl.size() * sizeof(void *)},
                        {pm.data(), pm.size()}},
                       {L.ops_off, L.mats_off, L.coeffs_off, L.tbl_off, L.pmats_off}, L.end));
-  const size_t acc_stride = (size_t)np + 1;
+  const size_t acc_stride = (size_t)A.n_acc + 1;
   const size_t acc_bytes = acc_stride * B * sizeof(double);
   if (acc_bytes > red_bytes(s->n)) return set_error(SV_ENOMEM, "workspace too small for the gradient batch");
   double *acc = reinterpret_cast<double *>(s->ws + kWsRed);
@@ -271,7 +387,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
   E.tbl0 = reinterpret_cast<void *const *>(base + L.tbl_off);
   E.tbl1 = E.tbl0 + B;
   E.pmats = base + L.pmats_off;
-  E.pmats_stride = (uint64_t)8 * A.n_inst;
+  E.pmats_stride = (uint64_t)4 * A.n_mats;
   E.acc = acc;
   E.acc_stride = acc_stride;
   if (opt && opt->mode == SV_MODE_TILED_GRAPH) {
@@ -316,8 +432,14 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
   SV_CUDA(cudaMemcpyAsync(h.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, s->stream));
   SV_CUDA(cudaStreamSynchronize(s->stream));
   for (int b = 0; b < B; b++) {
-    ev_out[b] = h[(size_t)b * acc_stride + np];
-    for (int p = 0; p < np; p++) grad_out[(size_t)b * np + p] = h[(size_t)b * acc_stride + p];
+    const double *hb = h.data() + (size_t)b * acc_stride;
+    ev_out[b] = hb[A.n_acc];
+    if (A.sites) {
+      std::fill(grad_out + (size_t)b * np, grad_out + (size_t)(b + 1) * np, 0.0);
+      site_grads(A, params + (size_t)b * np, hb, grad_out + (size_t)b * np);
+    } else {
+      for (int p = 0; p < np; p++) grad_out[(size_t)b * np + p] = hb[p];
+    }
   }
   return SV_OK;
 }

@@ -360,6 +360,54 @@ static std::vector<int> tcp_first_targets(const std::vector<std::vector<int>> &T
   return c;
 }
 
+// A TOP_SITES op (complex64): its targets padded to three with the highest
+// tile positions not among them, its descriptor into the matrix pool.
+static sv_status emit_sites(DeviceProgram &prog, const Block &blk, const BuildCtx &b, const int *loc, int m,
+                            TileOp &op) {
+  if (b.dt != SV_C64 || m < 3 || !b.site_mat) return set_error(SV_EINVAL, "internal: sites op out of place");
+  int k = (int)blk.qubits.size();
+  uint32_t fixed = 0;
+  for (int j = 0; j < k; j++) fixed |= 1u << op.t[j];
+  for (int p = m - 1; k < 3; p--)
+    if (!((fixed >> p) & 1u)) {
+      op.t[k++] = (uint8_t)p;
+      fixed |= 1u << p;
+    }
+  op.k = 3;
+  SitesDesc d;
+  std::memset(&d, 0, sizeof(d));
+  // (swizzle of the complex64 tile, tile_ops.cuh)
+  auto slot = [](uint32_t l) { return (l ^ ((l >> 4) & 15u)) * (uint32_t)sizeof(float2); };
+  uint32_t off[8];
+  for (int y = 0; y < 8; y++) {
+    uint32_t l = 0;
+    for (int j = 0; j < 3; j++) l |= (uint32_t)((y >> j) & 1) << op.t[j];
+    off[y] = slot(l);
+  }
+  // the tables act on the block's own qubits; padding targets stay
+  const int mask = (1 << (int)blk.qubits.size()) - 1;
+  for (int y = 0; y < 8; y++) {
+    d.ld[(blk.pre[y & mask] & mask) | (y & ~mask)] = off[y];
+    d.st[y] = off[(blk.post[y & mask] & mask) | (y & ~mask)];
+  }
+  for (int j = 0; j < 3; j++) {
+    const int site = j < (int)blk.qubits.size() ? blk.site[j] : -1;
+    d.mat[j] = site >= 0 ? b.site_mat[site] : -1;
+    if (site < 0) continue;
+    d.any |= 1u << j;
+    if (b.site_slot) {
+      d.slot[j] = b.site_slot[site];
+      d.comps |= (uint32_t)b.site_comps[site] << (4 * j);
+    }
+  }
+  set_thread_positions(op, fixed, m, b.dt);
+  while (prog.mats.size() % 16) prog.mats.push_back(0);
+  op.mat = (uint32_t)(prog.mats.size() / 16);
+  const uint8_t *q = reinterpret_cast<const uint8_t *>(&d);
+  prog.mats.insert(prog.mats.end(), q, q + sizeof(d));
+  return SV_OK;
+}
+
 sv_status emit_pass(DeviceProgram &prog, const PassPlan &P, const BuildCtx &b,
                            std::vector<uint32_t> &op0s, const std::vector<int> &batch_mat_off) {
   TilePass tp;
@@ -434,6 +482,11 @@ sv_status emit_pass(DeviceProgram &prog, const PassPlan &P, const BuildCtx &b,
     for (int q : blk.controls) {
       if (loc[q] >= 0) op.lcmask |= 1u << loc[q];
       else gcm |= 1ull << q;
+    }
+    if (blk.kind == TOP_SITES) {
+      SV_TRY(emit_sites(prog, blk, b, loc, tp.m, op));
+      prog.ops.push_back(op);
+      continue;
     }
     if (blk.kind == TOP_DENSE && blk.diag) op.kind = TOP_DIAG;
     // 0/1 permutation blocks of complex128 states move amplitudes instead of

@@ -53,8 +53,22 @@ enum TileOpKind : uint8_t {
   TOP_DOT = 5,       // acc[slot] += Re <v0 | v1>
   TOP_TC = 6,        // 5-qubit dense block on the tensor cores (12-qubit tiles)
   TOP_PERM = 7,      // permutation block (k = 1..3): member y moves to member perm[y]; controls as TOP_DENSE
-  TOP_GRADU = 8      // TOP_GRAD then the 1-qubit matrix (per-batch pool) on both vectors, in one sweep
+  TOP_GRADU = 8,     // TOP_GRAD then the 1-qubit matrix (per-batch pool) on both vectors, in one sweep
+  TOP_SITES = 9      // up to 3 qubits: a permutation, per-batch 1-qubit matrices (with probes), a permutation
 };
+
+// Descriptor of a TOP_SITES op (matrix pool, 16-byte aligned): swizzled byte
+// offsets that member y (bits: the op's three targets) is loaded from and
+// stored to, and per target the matrix (per-batch pool, -1: none), the first
+// of its accumulators and which of Im <v1 | X, Y, Z | v0> it takes.
+struct SitesDesc {
+  uint32_t ld[8], st[8];
+  int32_t mat[3];
+  uint32_t any;        // targets with a matrix, as a bit mask
+  int32_t slot[3];
+  uint32_t comps;      // 4 bits per target
+};
+static_assert(sizeof(SitesDesc) == 96, "SitesDesc layout");
 
 // 32-byte op descriptor; matrices live in a separate pool.
 struct TileOp {
@@ -195,7 +209,15 @@ struct Block {
   int inst = -1;               // parametric instance (per-batch matrix)
   double coeff = 0;
   uint64_t xmask = 0, zmask = 0;
+  // TOP_SITES (at most 3 qubits): member moves before and after the sites
+  // (member y goes to pre[y] / post[y]) and the site of each qubit, -1 for none
+  uint8_t pre[8] = {0, 1, 2, 3, 4, 5, 6, 7}, post[8] = {0, 1, 2, 3, 4, 5, 6, 7};
+  int site[3] = {-1, -1, -1};
 };
+// A site of a gradient program: a run of parametric gates on one qubit with
+// nothing on that qubit between them.  All their generators' expectations
+// follow from those of X, Y and Z at the run's start.
+using AdjSite = std::vector<int>;   // parametric instances, in order
 
 // gates.cpp
 int gate_arity(int gate);                                    // -1 unknown
@@ -226,6 +248,11 @@ std::vector<PassPlan> plan_passes(const std::vector<Block> &blocks, int n, int m
 // Blocks of the planned passes in execution order, with blocks of a pass
 // merged where commuting lets them meet and the union has at most K qubits.
 std::vector<Block> merge_in_passes(const std::vector<PassPlan> &passes, int K);
+// Blocks of a sequence with parametric single-qubit gates (inst >= 0) for
+// gradient programs: parametric gates become sites, X, CNOT, SWAP, Toffoli and
+// other permutations of at most 3 qubits the moves around them (TOP_SITES ops
+// of at most 3 qubits), other gates dense blocks of at most K qubits.
+std::vector<Block> site_blocks(const std::vector<Gate> &gates, int K, std::vector<AdjSite> &sites);
 
 // ---------------------------------------------------------------------------
 // state handle
@@ -299,6 +326,9 @@ struct BuildCtx {
   uint32_t nvec;
   uint32_t flags;
   int prec = SV_PREC_PLAIN;   // mode of TOP_TC ops
+  // TOP_SITES: per site its matrix (per-batch pool), first accumulator slot
+  // and components (0: no probes)
+  const int *site_mat = nullptr, *site_slot = nullptr, *site_comps = nullptr;
 };
 sv_status emit_pass(DeviceProgram &prog, const PassPlan &P, const BuildCtx &b,
                     std::vector<uint32_t> &op0s, const std::vector<int> &batch_mat_off);
@@ -486,6 +516,11 @@ struct HostPass {
 sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStream_t stream,
                               const HostPass *host = nullptr);
 sv_status launch_tile_tc(sv_state *s, const TilePass &p, cudaStream_t stream);   // k_tile_tc.cu
+// a pass of TOP_SITES ops only, and its launch (k_tile_sites.cu); a pass never
+// mixes them with other kinds
+bool sites_pass_ok(const TilePass &p, const HostPass &h);
+sv_status launch_tile_sites(sv_state *s, const TilePass &p, int batch, int threads, cudaStream_t stream);
+constexpr int kMaxSitesOps = 40;   // ops of such a pass
 // pipelined split-BF16 tile pass (k_tile_tcp.cu): at most kTcpMaxBlocks
 // tensor-core blocks per pass, whose B operands stay in shared memory
 constexpr int kTcpMaxBlocks = 6;
