@@ -68,7 +68,12 @@ typedef enum { SV_C64 = 0, SV_C128 = 1 } sv_dtype;
  * kernel; blocks with controls stay on the CUDA cores.  Split-TF32 applies
  * dense 4- and 5-qubit blocks on the tensor cores (a 4-qubit block padded
  * with an idle qubit), as passes of their own unless tile_m is 12.
- * complex128 states always use FP64 CUDA-core arithmetic. */
+ * complex128 states always use FP64 arithmetic whatever the mode.  Their
+ * circuits of uncontrolled blocks run on the tensor cores from 14 qubits on
+ * where options are left at 0 (SV_PREC_PLAIN): products of exact integer
+ * digits of the FP64 numbers, joined and rounded to FP64 once per block.  The
+ * digits are relative to the largest number a block mixes: an amplitude
+ * keeps an absolute error below 2^-57 of it. */
 typedef enum {
   SV_PREC_PLAIN = 0,       /* FP32 FMA on CUDA cores */
   SV_PREC_TC_BF16X3 = 1,   /* tensor cores, split-BF16 (3 products), FP32 accumulate */

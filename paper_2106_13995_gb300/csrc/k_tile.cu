@@ -495,6 +495,10 @@ static sv_status launch_tile_tperm(sv_state *s, const TilePass &p, int batch, cu
 sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStream_t stream,
                               const HostPass *host) {
   if (p.flags & kPassTable) return launch_tile_tperm(s, p, batch, stream);
+  if (p.flags & kPassOz) {
+    if (!host || batch != 1) return set_error(SV_EINVAL, "internal: exact tensor-core pass without its host copy");
+    return launch_tile_oz(s, p, *host, stream);
+  }
   if (p.flags & kPassHasTC) {
     if (s->dt != SV_C64 || p.m != kTcTileM || batch != 1 || p.nvec != 1)
       return set_error(SV_EINVAL, "internal: tensor-core tile pass needs one complex64 vector and 12-qubit tiles");

@@ -6,6 +6,7 @@
 #include <map>
 #include <tuple>
 
+#include "oz_digits.cuh"
 #include "sv_internal.h"
 
 namespace sv {
@@ -83,6 +84,14 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   const bool explicit12 = o && o->tile_m == kTcTileM;
   const bool default_m = !(o && o->tile_m > 0);
   r.tc_in_tile = r.prec != SV_PREC_PLAIN && (explicit12 || (r.prec == SV_PREC_TC_BF16X3 && default_m));
+  // complex128 states of at least 14 qubits: 5-qubit blocks on the tensor
+  // cores, exactly (k_tile_oz), unless a fusion width or tile size is asked
+  // for.  Below, one or two 12-qubit tiles are a chain of blocks on one or two
+  // SMs (20 layers of U3 + CZ: 12 qubits 544 us against 463 in 7-qubit tiles
+  // of the CUDA cores, 14 qubits 506 against 570, 16 qubits 636 against 664;
+  // grid circuits of 17 qubits 254 against 480, of 23 qubits 7.2 ms against 28)
+  r.oz = s->dt == SV_C128 && s->n >= kOzMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
+         r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE;
   r.L = std::min(r.L, r.tile_m);
   if (s->dt == SV_C64 && r.L < 1) r.L = 1;
   return r;
@@ -705,8 +714,77 @@ static sv_status emit_tc_pass(CachedProgram &out, const Block &blk, int n, int p
   return SV_OK;
 }
 
+// A complex128 program of exact tensor-core passes, if every fused block of at
+// most 5 qubits qualifies: uncontrolled (wider or controlled ones stay on the
+// CUDA cores, and a program is all of one kind), digits within the exact range,
+// not all of them permutations (those move amplitudes in table passes), and the
+// operands fit the program area.  False leaves `out` empty.
+static bool build_oz_program(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
+  const int n = s->n, m = kTcTileM, L = o.L;
+  std::vector<Block> blocks = fuse(gates, 5);
+  if (m < n) {
+    const std::vector<PassPlan> first = plan_passes(blocks, n, m, L, kOzMaxBlocks, kMaxMatPerPass);
+    if (first.empty()) return false;
+    std::vector<Block> merged = merge_in_passes(first, 5);
+    if (merged.size() < blocks.size()) blocks = std::move(merged);
+  }
+  bool moves = true;
+  int perm[64];
+  for (Block &b : blocks) {
+    if (b.kind != TOP_DENSE || !b.controls.empty() || b.qubits.size() > 5) return false;
+    moves = moves && permutation_of(b.U, (int)b.qubits.size(), perm);
+    b.kind = TOP_TC;
+  }
+  if (moves || blocks.size() * kOzDigits * 64 * 64 * 2 + (64 << 10) > kWsProgBytes) return false;
+  std::vector<PassPlan> passes = plan_passes(blocks, n, m, L, kOzMaxBlocks, kOzMaxBlocks * 1024 + 1023);
+  if (passes.empty()) return false;
+  CachedProgram prog;
+  for (PassPlan &P : passes) {
+    TilePass tp;
+    std::memset(&tp, 0, sizeof(tp));
+    tp.n = n;
+    tp.m = m;
+    tp.L = std::min(L, m);
+    tp.nvec = 1;
+    tp.flags = kPassOz;
+    int loc[64];
+    std::fill(loc, loc + 64, -1);
+    for (size_t i = 0; i < P.S.size(); i++) loc[P.S[i]] = (int)i;
+    for (int j = tp.L; j < m; j++) tp.hi_pos[j - tp.L] = (int8_t)P.S[j];
+    int no = 0;
+    for (int q = 0; q < n; q++)
+      if (loc[q] < 0) tp.out_pos[no++] = (int8_t)q;
+    tp.nops = (int)P.ops.size();
+    prog.op0s.push_back((uint32_t)prog.prog.ops.size());
+    for (Block &b : P.ops) {
+      if (b.qubits.size() < 5) pad_in_tile(b, P.S);
+      TileOp op;
+      std::memset(&op, 0, sizeof(op));
+      op.kind = TOP_TC;
+      op.k = 5;
+      op.vmask = 1;
+      for (int j = 0; j < 5; j++) op.t[j] = (uint8_t)loc[b.qubits[j]];
+      std::vector<uint16_t> packed;
+      int eu = 0;
+      if (!oz_pack_matrix(b.U, packed, eu) || eu < -1000 || eu > 1000) return false;
+      op.slot = (int16_t)eu;
+      op.mat = (uint32_t)(prog.prog.mats.size() / 16);
+      const uint8_t *q = reinterpret_cast<const uint8_t *>(packed.data());
+      prog.prog.mats.insert(prog.prog.mats.end(), q, q + packed.size() * 2);
+      prog.prog.ops.push_back(op);
+    }
+    prog.prog.passes.push_back(tp);
+  }
+  prog.blocks = std::move(blocks);
+  prog.lay = layout_of(prog.prog, 0, 0);
+  if (prog.lay.end > kWsProgBytes) return false;
+  out = std::move(prog);
+  return true;
+}
+
 static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gates, const Opts &o,
                                        CachedProgram &out) {
+  if (o.oz && build_oz_program(s, gates, o, out)) return SV_OK;
   out.blocks = fuse(gates, o.fusion_k);
   if (o.mode == SV_MODE_PER_GATE) return SV_OK;
   int m = o.tile_m, L = o.L;
@@ -856,6 +934,7 @@ sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, co
   k.val(o.mode);
   k.val(o.prec);
   k.val(o.tc_in_tile);
+  k.val(o.oz);
   k.val((int)s->dt);
   if (params && c->n_params > 0) k.bytes(params, sizeof(double) * c->n_params);
   const uint64_t h = k.hash();

@@ -126,7 +126,7 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
     bool has_tc = false;
     // (tensor-core and permutation passes have kernels of their own, which
     // the persistent queue does not run)
-    for (const TilePass &tp : cps[b]->prog.passes) has_tc |= (tp.flags & (kPassTC | kPassHasTC | kPassTable)) != 0;
+    for (const TilePass &tp : cps[b]->prog.passes) has_tc |= (tp.flags & (kPassTC | kPassHasTC | kPassTable | kPassOz)) != 0;
     wide[b] = !cps[b]->prog.passes.empty() && (has_tc || states[b]->n >= wide_n);
   }
   // descriptors in wave order: pass 0 of every state, then pass 1, ...

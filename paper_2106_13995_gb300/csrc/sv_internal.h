@@ -136,6 +136,10 @@ constexpr uint32_t kPassHasTC = 0x8;
 // moves by a gather table (16-byte index mat0 of its block in the matrix
 // pool; k_tile_tperm)
 constexpr uint32_t kPassTable = 0x800;
+// TilePass.flags: a pass of 5-qubit blocks of a complex128 state on the tensor
+// cores (k_tile_oz): op i's targets t[], packed operand mat (16-byte index) and
+// matrix exponent in slot
+constexpr uint32_t kPassOz = 0x1000;
 constexpr int kTcTileM = 12;          // tile size that gives M = 128 groups for a 5-qubit block
 size_t tc_tile_smem(sv_prec mode);    // shared memory of a 12-qubit tile pass with TOP_TC ops
 struct TilePass {
@@ -355,6 +359,7 @@ sv_status launch_program(sv_state *s, const DeviceProgram &p, const ProgLayout &
 struct Opts {   // all int: hashed as key bytes, so no padding
   int fusion_k, tile_m, L, prec, mode;
   int tc_in_tile = 0;
+  int oz = 0;   // complex128: blocks of 5 qubits on the tensor cores where they all qualify
 };
 constexpr int kSmall128 = 17;   // widest complex128 state with the small-state plan
 Opts resolve(const sv_state *s, const sv_options *o, int nvec);
@@ -543,6 +548,11 @@ void tcp_row_positions(TileOp &op, int pair_gather, int pair_scatter);
 // host replay of a pipelined pass's shared-memory addressing; "" when sound
 std::string tcp_layout_selftest(const TilePass &p, const HostPass &host, int *pair_gathers = nullptr,
                                 int *pair_scatters = nullptr);
+// exact tensor-core passes of complex128 states (k_tile_oz.cu)
+constexpr int kOzMaxBlocks = 12;
+constexpr int kOzMinQubits = 14;
+bool oz_pack_matrix(const std::vector<cd> &U, std::vector<uint16_t> &out, int &eu);
+sv_status launch_tile_oz(sv_state *s, const TilePass &p, const HostPass &host, cudaStream_t stream);
 // tensor-core 5-qubit block (k_tc.cu)
 size_t tc_matrix_words(sv_prec mode, int k);
 void tc_pack_matrix(const std::vector<cd> &U, sv_prec mode, std::vector<uint32_t> &out);
