@@ -19,11 +19,15 @@
 // first half is joined and scattered while they run.  The B operands (56 KB a
 // block) are copied from L2 into two buffers in turn.
 //
-// Bound (21 qubits, 13 us per tile and block): the chain gather - digits - MMA
-// - join of one tile.  The MMAs take 0.42 of it (N = 32 runs at half the rate
-// of N = 64, whose sums would not fit TMEM next to the digits), the join 0.19;
-// integer ALU pipe 36%, tensor pipe 13%, HBM 6%.  A 23-qubit grid circuit of
-// 20 cycles: 27 ms in FP64 arithmetic, 7.2 ms here.
+// An MMA of M = 128 and K = 16 with A in TMEM takes about 50 clocks up to N =
+// 64, so digit i of A meets all its digits of B in one of N = 32 (7 - i): 56
+// MMAs per tile and block.  One MMA of N = 32 per digit product (224) took 0.42
+// of the time: 1.78 ms against 1.24 for 33 blocks of 21 qubits.
+//
+// Bound (21 qubits, 9.3 us per tile and block): the chain gather - digits - MMA
+// - join of one tile; without the join 0.28 less, with a seventh of the MMAs
+// 0.13 less.  A 23-qubit grid circuit of 20 cycles: 27.2 ms in FP64 arithmetic,
+// 4.4 ms here.
 //
 // Every wait is bounded, as in K9.
 #include <algorithm>
@@ -40,8 +44,8 @@ namespace sv {
 
 constexpr int kOzThreads = 512;
 constexpr uint32_t kOzTileBytes = (1u << kTcTileM) * 16;     // 64 KB
-constexpr uint32_t kOzDigitBytes = 64 * 64 * 2;               // one digit of B: 8 KB
-constexpr uint32_t kOzBBytes = kOzDigits * kOzDigitBytes;     // 56 KB
+constexpr uint32_t kOzBRows = kOzDigits * 64;                 // of B: half of the columns, digit, 32 columns
+constexpr uint32_t kOzBBytes = kOzBRows * 64 * 2;             // 56 KB
 constexpr uint32_t kOzSmB = kOzTileBytes, kOzSmExp = kOzSmB + 2 * kOzBBytes, kOzSmBar = kOzSmExp + 4 * 128 * 4;
 constexpr uint32_t kOzSmem = kOzSmBar + 8 * 3 + 8;
 static_assert(kOzSmem <= 227u * 1024u, "shared memory of a CTA");
@@ -84,19 +88,18 @@ __device__ __forceinline__ void oz_commit(uint32_t bar) {
 }
 
 // (one thread) result columns 32 h .. 32 h + 31: every digit product of weight
-// at most 6 into the sum of its weight
+// at most 6 into the sum of its weight.  Digit i of A meets digits 0 .. 6 - i
+// of B in one MMA: their operands follow each other by 32 rows, as the sums of
+// weight i and up do by 32 columns.
 __device__ __forceinline__ void oz_issue(uint32_t tmem, uint32_t bs, int h) {
-  const uint32_t idesc = instr_desc(0u, 128, 32);   // FP16 A and B, FP32 D
   // descriptors differ in their address field alone (16-byte units)
-  const uint64_t b0 = smem_desc(bs + (uint32_t)h * 512, 1024, 128);
+  const uint64_t b0 = smem_desc(bs + (uint32_t)h * (kOzBRows / 2) * 16, kOzBRows * 16, 128);
 #pragma unroll
   for (uint32_t k = 0; k < 4; k++)
 #pragma unroll
-    for (int i = 0; i < kOzDigits; i++)
-#pragma unroll
-      for (int j = 0; i + j < kOzDigits; j++)
-        oz_mma(tmem + kOzTmemD + 32 * (i + j), tmem + 32 * i + 8 * k, b0 + (j * kOzDigitBytes + k * 2048) / 16, idesc,
-               (i > 0 || k > 0) ? 1u : 0u);
+    for (uint32_t i = 0; i < kOzDigits; i++)
+      oz_mma(tmem + kOzTmemD + 32 * i, tmem + 32 * i + 8 * k, b0 + (uint64_t)(2 * k * kOzBRows),
+             instr_desc(0u, 128, (kOzDigits - i) * 32), (i > 0 || k > 0) ? 1u : 0u);   // FP16 A and B, FP32 D
 }
 
 // A denormal, infinite or zero result.  Out of line: inlined, its FP64
@@ -313,8 +316,8 @@ static std::pair<uint32_t, uint32_t> oz_words(double v) {
   return {(uint32_t)(b >> 32), (uint32_t)b};
 }
 
-// U (32 x 32) as FP16 digits of its real embedding, digit by digit in the
-// canonical no-swizzle K-major layout of 64 rows; eu: |entries| < 2^eu.  False
+// U (32 x 32) as FP16 digits of its real embedding in the canonical no-swizzle
+// K-major layout: row 224 h + 32 i + c is digit i of result column 32 h + c; eu: |entries| < 2^eu.  False
 // when a sum of weight at most 4 could pass 2^24 for some input (row sums of
 // the digits' magnitudes; the weights beyond may: an FP32 rounding there is
 // 2^-57 of a result), when the first weight's could pass 15/16 of 2^20 (the
@@ -367,14 +370,15 @@ static bool oz_pack_digits(const std::vector<cd> &U, std::vector<uint16_t> &out,
         const uint64_t w = oz_fields(hi, lo, E);
         // Re at (2r, 2q) and (2r + 1, 2q + 1); Im at (2r + 1, 2q), -Im at (2r, 2q + 1)
         auto at = [](int n, int k) {
-          return (size_t)(cm_offset((uint32_t)n, (uint32_t)k / 8, 64) / 2) + (size_t)(k % 8);
+          return (size_t)(cm_offset((uint32_t)(n / 32) * (kOzBRows / 2) + (uint32_t)(n % 32), (uint32_t)k / 8, kOzBRows) / 2) +
+                 (size_t)(k % 8);
         };
         const size_t at0 = at(2 * r + part, 2 * q), at1 = at(2 * r + 1 - part, 2 * q + 1);
         for (int i = 0; i < kOzDigits; i++) {
           const int d = oz_digit(w, i);
           mag[(size_t)r * kOzDigits + i] += (uint32_t)(d < 0 ? -d : d);
-          out[at0 + (size_t)i * 64 * 64] = halves.of[256 + d];
-          out[at1 + (size_t)i * 64 * 64] = halves.of[256 + (part ? -d : d)];
+          out[at0 + (size_t)i * 32 * 8] = halves.of[256 + d];
+          out[at1 + (size_t)i * 32 * 8] = halves.of[256 + (part ? -d : d)];
         }
       }
   for (int r = 0; r < 32; r++) {

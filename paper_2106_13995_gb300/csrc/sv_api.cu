@@ -86,10 +86,11 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   r.tc_in_tile = r.prec != SV_PREC_PLAIN && (explicit12 || (r.prec == SV_PREC_TC_BF16X3 && default_m));
   // complex128 states of at least 14 qubits: 5-qubit blocks on the tensor
   // cores, exactly (k_tile_oz), unless a fusion width or tile size is asked
-  // for.  Below, one or two 12-qubit tiles are a chain of blocks on one or two
-  // SMs (20 layers of U3 + CZ: 12 qubits 544 us against 463 in 7-qubit tiles
-  // of the CUDA cores, 14 qubits 506 against 570, 16 qubits 636 against 664;
-  // grid circuits of 17 qubits 254 against 480, of 23 qubits 7.2 ms against 28)
+  // for (20 layers of U3 + CZ, against 7-qubit tiles of the CUDA cores: 14
+  // qubits 357 us against 569, 16 qubits 457 against 669; grid circuits of 17
+  // qubits 181 against 480, of 23 qubits 5.0 ms against 30).  Below, one or two
+  // SMs run all blocks in turn, and what preparing the operands adds to a
+  // circuit's first run (30 us a block) is more than its blocks save
   r.oz = s->dt == SV_C128 && s->n >= kOzMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
          r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE;
   r.L = std::min(r.L, r.tile_m);

@@ -51,8 +51,9 @@ extern "C" int oz_block(const double *u, const double *x, double *out, double *w
       int64_t sum = 0;
       for (int i = 0; i <= s; i++)
         for (int k = 0; k < 64; k++) {
-          // canonical layout: 8-element chunks along K, 64 rows
-          const size_t at = (size_t)(s - i) * 4096 + (size_t)(k / 8) * 512 + (size_t)(n / 8) * 64 + (size_t)(n % 8) * 8 + (size_t)(k % 8);
+          // canonical layout: 8-element chunks along K, 448 rows (column half, digit, column)
+          const size_t row = (size_t)(n / 32) * 224 + (size_t)(s - i) * 32 + (size_t)(n % 32);
+          const size_t at = (size_t)(k / 8) * 448 * 8 + row * 8 + (size_t)(k % 8);
           sum += (int64_t)half_value(B[at]) * oz_digit(w[k], i);
         }
       if (s <= 4) worst[1] = std::max(worst[1], (double)std::llabs(sum));
