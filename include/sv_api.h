@@ -142,8 +142,10 @@ typedef struct sv_state sv_state;
  * State handles (Sec. I-A: the state is the vector of 2^n amplitudes)
  * ------------------------------------------------------------------------- */
 
-/* Workspace bytes a state of this size needs for reductions, sampling and
- * uploaded gate programs. */
+/* Workspace bytes for a state of this size: reductions, sampling, uploaded gate
+ * programs, and from 15 qubits on the scratch of permutation runs (a quarter of
+ * the state, at most 64 MB).  sv_create also takes a workspace without that
+ * scratch; permutation gates then run as tile passes. */
 size_t sv_workspace_bytes(int n_qubits, sv_dtype dtype);
 
 /* Wrap caller-owned device memory as a state.

@@ -93,6 +93,9 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   // circuit's first run (30 us a block) is more than its blocks save
   r.oz = s->dt == SV_C128 && s->n >= kOzMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
          r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE;
+  r.moves = s->n >= kMovesMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
+            r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE &&
+            s->ws_bytes >= moves_off(s->n) + moves_bytes(s->n, s->dt);
   r.L = std::min(r.L, r.tile_m);
   if (s->dt == SV_C64 && r.L < 1) r.L = 1;
   return r;
@@ -715,12 +718,12 @@ static sv_status emit_tc_pass(CachedProgram &out, const Block &blk, int n, int p
   return SV_OK;
 }
 
-// A complex128 program of exact tensor-core passes, if every fused block of at
+// Append a complex128 program of exact tensor-core passes, if every fused block of at
 // most 5 qubits qualifies: uncontrolled (wider or controlled ones stay on the
 // CUDA cores, and a program is all of one kind), digits within the exact range,
 // not all of them permutations (those move amplitudes in table passes), and the
-// operands fit the program area.  False leaves `out` empty.
-static bool build_oz_program(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
+// operands fit the program area.  False leaves `out` as it was.
+static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
   const int n = s->n, m = kTcTileM, L = o.L;
   std::vector<Block> blocks = fuse(gates, 5);
   if (m < n) {
@@ -736,7 +739,7 @@ static bool build_oz_program(const sv_state *s, const std::vector<Gate> &gates, 
     moves = moves && permutation_of(b.U, (int)b.qubits.size(), perm);
     b.kind = TOP_TC;
   }
-  if (moves || blocks.size() * kOzDigits * 64 * 64 * 2 + (64 << 10) > kWsProgBytes) return false;
+  if (moves || out.prog.mats.size() + blocks.size() * kOzDigits * 64 * 64 * 2 + (64 << 10) > kWsProgBytes) return false;
   std::vector<PassPlan> passes = plan_passes(blocks, n, m, L, kOzMaxBlocks, kOzMaxBlocks * 1024 + 1023);
   if (passes.empty()) return false;
   CachedProgram prog;
@@ -776,29 +779,39 @@ static bool build_oz_program(const sv_state *s, const std::vector<Gate> &gates, 
     }
     prog.prog.passes.push_back(tp);
   }
-  prog.blocks = std::move(blocks);
-  prog.lay = layout_of(prog.prog, 0, 0);
-  if (prog.lay.end > kWsProgBytes) return false;
-  out = std::move(prog);
+  // behind what `out` holds
+  DeviceProgram &to = out.prog;
+  while (to.mats.size() % 16) to.mats.push_back(0);
+  const uint32_t op0 = (uint32_t)to.ops.size(), mat0 = (uint32_t)(to.mats.size() / 16);
+  for (TileOp &op : prog.prog.ops) op.mat += mat0;
+  for (uint32_t x : prog.op0s) out.op0s.push_back(x + op0);
+  to.ops.insert(to.ops.end(), prog.prog.ops.begin(), prog.prog.ops.end());
+  to.mats.insert(to.mats.end(), prog.prog.mats.begin(), prog.prog.mats.end());
+  to.passes.insert(to.passes.end(), prog.prog.passes.begin(), prog.prog.passes.end());
+  out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
   return true;
 }
 
-static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gates, const Opts &o,
-                                       CachedProgram &out) {
-  if (o.oz && build_oz_program(s, gates, o, out)) return SV_OK;
-  out.blocks = fuse(gates, o.fusion_k);
-  if (o.mode == SV_MODE_PER_GATE) return SV_OK;
+// Append a program of tile passes for `gates` to `out` (its layout is left to
+// the caller).
+static sv_status append_gates(sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
+  if (o.oz && append_oz_program(s, gates, o, out)) return SV_OK;
+  std::vector<Block> blocks = fuse(gates, o.fusion_k);
+  if (o.mode == SV_MODE_PER_GATE) {
+    out.blocks = std::move(blocks);
+    return SV_OK;
+  }
   int m = o.tile_m, L = o.L;
-  if (!fit_tile(out.blocks, s->n, lmin(s->dt), mmax(s->dt, 1), m, L))
+  if (!fit_tile(blocks, s->n, lmin(s->dt), mmax(s->dt, 1), m, L))
     return set_error(SV_EUNSUPPORTED, "a fused block does not fit a shared-memory tile");
   if (o.fusion_k >= 2 && m < s->n) {
     // blocks that meet inside a pass merge (one pass-sized op instead of two)
-    const std::vector<PassPlan> first = plan_passes(out.blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass);
+    const std::vector<PassPlan> first = plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass);
     if (!first.empty()) {
       std::vector<Block> merged = merge_in_passes(first, o.fusion_k);
       int m2 = m, L2 = L;
-      if (merged.size() < out.blocks.size() && fit_tile(merged, s->n, lmin(s->dt), mmax(s->dt, 1), m2, L2)) {
-        out.blocks = std::move(merged);
+      if (merged.size() < blocks.size() && fit_tile(merged, s->n, lmin(s->dt), mmax(s->dt, 1), m2, L2)) {
+        blocks = std::move(merged);
         m = m2;
         L = L2;
       }
@@ -830,7 +843,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
     // whose operands stay in shared memory (each counts 1024 entries).
     // Split-TF32: dense 4- and 5-qubit blocks only.
     const bool bf16 = o.prec == SV_PREC_TC_BF16X3;
-    for (Block &blk : out.blocks) {
+    for (Block &blk : blocks) {
       if (bf16) {
         if (blk.kind == TOP_DENSE && blk.controls.empty() && blk.qubits.size() <= 5) blk.kind = TOP_TC;
       } else {
@@ -852,7 +865,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
       seg.clear();
       return SV_OK;
     };
-    for (const Block &blk : out.blocks) {
+    for (const Block &blk : blocks) {
       // split-BF16: an uncontrolled dense 6-qubit block (fusion width 6) is
       // a tensor-core pass of its own, between the tile passes
       const bool six = bf16 && s->n >= 13 && blk.kind == TOP_DENSE && blk.qubits.size() == 6 &&
@@ -865,7 +878,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
       SV_TRY(emit_tc_pass(out, blk, s->n, o.prec));
     }
     SV_TRY(flush_tc());
-    out.lay = layout_of(out.prog, 0, 0);
+    out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
     return SV_OK;
   }
   std::vector<Block> seg;
@@ -877,7 +890,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
     seg.clear();
     return SV_OK;
   };
-  for (const Block &blk0 : out.blocks) {
+  for (const Block &blk0 : blocks) {
     Block blk = blk0;
     if (tc) pad4(blk);
     const bool is_tc = tc && blk.kind == TOP_DENSE && blk.qubits.size() == 5 && blk.controls.empty() && !blk.diag;
@@ -889,6 +902,55 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
     SV_TRY(emit_tc_pass(out, blk, s->n, o.prec));
   }
   SV_TRY(flush());
+  out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
+  return SV_OK;
+}
+
+// A run of at least kMovesMinGates permutation gates becomes moves where it would
+// take at least moves_worth tile passes for each of its move passes.  At 29
+// qubits a move pass takes 4.7 ms and a table pass 1.6; up to 20 qubits, where
+// launches count, about 28 and 8 us (random X, CNOT and Toffoli: 240 gates on 28
+// qubits 10.3 ms against 25.5 in tables, on 18 qubits 186 us against 180).
+constexpr size_t kMovesMinGates = 12;
+static size_t moves_worth(int n) { return n <= 20 ? 4 : 3; }
+// Passes a run of permutation gates takes as tile passes.
+static size_t count_passes(const sv_state *s, const std::vector<Gate> &gates, const Opts &o) {
+  std::vector<Block> blocks = fuse(gates, o.fusion_k);
+  int m = o.tile_m, L = o.L;
+  if (!fit_tile(blocks, s->n, lmin(s->dt), mmax(s->dt, 1), m, L)) return 0;
+  return plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass).size();
+}
+
+static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gates, const Opts &o,
+                                       CachedProgram &out) {
+  std::vector<Gate> rest;   // gates not yet in the program
+  size_t i = 0;
+  const int m = moves_m(s->n, s->dt);
+  while (o.moves && i < gates.size()) {
+    std::vector<Move> moves;
+    size_t e = i;
+    while (e < gates.size() && gate_moves(gates[e], moves)) e++;
+    if (e - i >= kMovesMinGates) {
+      const std::vector<Gate> run(gates.begin() + i, gates.begin() + e);
+      const std::vector<std::vector<Move>> passes = plan_moves(moves, m);
+      // (at most 9 ops of 16 bytes a move, 8 of them for many controls)
+      const bool fits = out.prog.mats.size() + 9 * 16 * moves.size() + 256 * passes.size() <= kWsProgBytes / 2;
+      if (fits && count_passes(s, run, o) >= moves_worth(s->n) * passes.size()) {
+        if (!rest.empty()) SV_TRY(append_gates(s, rest, o, out));
+        rest.clear();
+        for (const std::vector<Move> &p : passes) emit_moves(out.prog, p, s->n, m, out.op0s);
+        const std::vector<Block> blocks = fuse(run, o.fusion_k);
+        out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
+        i = e;
+        continue;
+      }
+    }
+    e = std::max(e, i + 1);
+    rest.insert(rest.end(), gates.begin() + i, gates.begin() + e);
+    i = e;
+  }
+  if (!o.moves) SV_TRY(append_gates(s, gates, o, out));
+  else if (!rest.empty()) SV_TRY(append_gates(s, rest, o, out));
   out.lay = layout_of(out.prog, 0, 0);
   return SV_OK;
 }
@@ -936,6 +998,7 @@ sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, co
   k.val(o.prec);
   k.val(o.tc_in_tile);
   k.val(o.oz);
+  k.val(o.moves);
   k.val((int)s->dt);
   if (params && c->n_params > 0) k.bytes(params, sizeof(double) * c->n_params);
   const uint64_t h = k.hash();
@@ -986,9 +1049,8 @@ int64_t sv_program_cache_limit(int64_t max_programs) {
 }
 
 size_t sv_workspace_bytes(int n, sv_dtype dt) {
-  (void)dt;
-  if (n < 1 || n > 34) return 0;
-  return kWsRed + red_bytes(n);
+  if (n < 1 || n > 34 || (dt != SV_C64 && dt != SV_C128)) return 0;
+  return moves_off(n) + moves_bytes(n, dt);
 }
 
 sv_status sv_create(int n, sv_dtype dt, void *amps, size_t amps_bytes, void *ws, size_t ws_bytes,
@@ -1001,7 +1063,9 @@ sv_status sv_create(int n, sv_dtype dt, void *amps, size_t amps_bytes, void *ws,
   if (((uintptr_t)amps & 255) || ((uintptr_t)ws & 255))
     return set_error(SV_EINVAL, "device buffers must be 256-byte aligned");
   if (amps_bytes < ((size_t)1 << n) * amp_bytes(dt)) return set_error(SV_EINVAL, "amplitude buffer too small");
-  if (ws_bytes < sv_workspace_bytes(n, dt))
+  // (without the permutation runs' scratch behind it, their gates take table
+  // passes)
+  if (ws_bytes < kWsRed + red_bytes(n))
     return set_error(SV_ENOMEM, "workspace smaller than sv_workspace_bytes()");
   cudaPointerAttributes attr;
   SV_CUDA(cudaPointerGetAttributes(&attr, amps));

@@ -76,6 +76,7 @@ void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt
   tune_load_locked();
   auto it = g_tune.find(tune_key(s->n, s->dt, c));
   if (it == g_tune.end() || it->second.first == 0) return;   // not tuned, or the defaults were fastest
+  o.oz = o.moves = 0;   // the pair was timed on the CUDA cores' tile passes
   if (want_k) o.fusion_k = it->second.first;
   if (want_m) o.tile_m = std::min(it->second.second, s->n);
 }
@@ -108,7 +109,6 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
     SV_TRY(get_program(states[b], circs[b], params ? params[b] : nullptr, opt, &cps[b], &os[b]));
     if (os[b].mode == SV_MODE_PER_GATE) return set_error(SV_EINVAL, "per-gate mode has no batched form");
     maxP = std::max(maxP, (int)cps[b]->prog.passes.size());
-    for (const TilePass &tp : cps[b]->prog.passes) m_max = std::max(m_max, tp.m);
   }
   for (int b = 0; b < B; b++) SV_TRY(upload_program(states[b], *cps[b]));
   // Wide states run as one ordinary launch per pass, spread over the fan-out
@@ -126,8 +126,10 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
     bool has_tc = false;
     // (tensor-core and permutation passes have kernels of their own, which
     // the persistent queue does not run)
-    for (const TilePass &tp : cps[b]->prog.passes) has_tc |= (tp.flags & (kPassTC | kPassHasTC | kPassTable | kPassOz)) != 0;
+    for (const TilePass &tp : cps[b]->prog.passes) has_tc |= (tp.flags & (kPassTC | kPassHasTC | kPassTable | kPassOz | kPassMoves)) != 0;
     wide[b] = !cps[b]->prog.passes.empty() && (has_tc || states[b]->n >= wide_n);
+    if (!wide[b])
+      for (const TilePass &tp : cps[b]->prog.passes) m_max = std::max(m_max, tp.m);
   }
   // descriptors in wave order: pass 0 of every state, then pass 1, ...
   std::vector<TilePass> desc;

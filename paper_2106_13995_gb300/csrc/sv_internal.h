@@ -140,6 +140,10 @@ constexpr uint32_t kPassTable = 0x800;
 // cores (k_tile_oz): op i's targets t[], packed operand mat (16-byte index) and
 // matrix exponent in slot
 constexpr uint32_t kPassOz = 0x1000;
+// TilePass.flags: a run of permutation gates as one move within chunks of 2^m
+// amplitudes (qubits hi_pos[0..m)); mat0: 16-byte index of its MoveDesc
+// (k_moves.cu)
+constexpr uint32_t kPassMoves = 0x2000;
 constexpr int kTcTileM = 12;          // tile size that gives M = 128 groups for a 5-qubit block
 size_t tc_tile_smem(sv_prec mode);    // shared memory of a 12-qubit tile pass with TOP_TC ops
 struct TilePass {
@@ -312,6 +316,14 @@ constexpr size_t kWsProg = kWsCtrlBytes;         // uploaded programs
 constexpr size_t kWsProgBytes = 8 << 20;
 constexpr size_t kWsRed = kWsProg + kWsProgBytes;  // reduction / sampling area
 size_t red_bytes(int n);
+// scratch of the permutation runs, behind the reduction area: two chunks of
+// 2^moves_m amplitudes, a quarter of the state up to 64 MB
+constexpr int kMovesMinQubits = 15;
+inline size_t moves_off(int n) { return (kWsRed + red_bytes(n) + 255) & ~(size_t)255; }
+inline int moves_m(int n, sv_dtype dt) { return n - 3 < (dt == SV_C64 ? 22 : 21) ? n - 3 : (dt == SV_C64 ? 22 : 21); }
+inline size_t moves_bytes(int n, sv_dtype dt) {
+  return n < kMovesMinQubits ? 0 : (size_t)(dt == SV_C64 ? 16 : 32) << moves_m(n, dt);
+}
 constexpr size_t kPinnedBytes = kWsProgBytes + kWsCtrlBytes;
 
 size_t amp_bytes(sv_dtype dt);
@@ -360,6 +372,7 @@ struct Opts {   // all int: hashed as key bytes, so no padding
   int fusion_k, tile_m, L, prec, mode;
   int tc_in_tile = 0;
   int oz = 0;   // complex128: blocks of 5 qubits on the tensor cores where they all qualify
+  int moves = 0;   // runs of permutation gates as moves (k_moves.cu)
 };
 constexpr int kSmall128 = 17;   // widest complex128 state with the small-state plan
 Opts resolve(const sv_state *s, const sv_options *o, int nvec);
@@ -367,6 +380,17 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec);
 // cache for this circuit's shape (sv_batch.cu), if a pair in it beat the
 // defaults.
 void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt, Opts &o);
+// permutation runs (k_moves.cu)
+struct Move {             // X on `target` where all of `controls` are 1
+  uint64_t controls;
+  int target;
+};
+// Append a gate as moves if it is a fixed permutation of at most 3 targets.
+bool gate_moves(const Gate &g, std::vector<Move> &out);
+std::vector<std::vector<Move>> plan_moves(const std::vector<Move> &moves, int m);
+void emit_moves(DeviceProgram &prog, const std::vector<Move> &moves, int n, int m, std::vector<uint32_t> &op0s);
+sv_status launch_moves(sv_state *s, const TilePass &p, cudaStream_t stream);
+
 // ---------------------------------------------------------------------------
 // program caches
 // ---------------------------------------------------------------------------
