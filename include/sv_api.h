@@ -259,8 +259,8 @@ sv_status sv_plan_fmas(sv_state *s, const sv_circuit *c, const double *params, c
  * bounded by opt->timeout_cycles polls (~128 ns each; 0 = about 1 s); a wait
  * that runs out stops the launch and the next sv_synchronize on states[0]
  * returns SV_ETIMEOUT.  With opt->mode == SV_MODE_TILED_GRAPH the counter
- * reset and the launch are captured once per batch layout and replayed as a
- * CUDA graph.  fusion_k / tile_m left at 0 take the autotuner's cached
+ * reset and the launches are captured when a batch layout comes a second time
+ * and replayed as a CUDA graph from then on.  fusion_k / tile_m left at 0 take the autotuner's cached
  * choice for the circuit's shape, if any.  All states must be distinct and
  * share one stream and device; the first state's workspace holds the batch
  * tables.  Enqueues only (no synchronisation).  Errors: SV_EINVAL (arguments,

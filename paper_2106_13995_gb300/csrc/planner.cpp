@@ -165,7 +165,7 @@ bool fit_tile(const std::vector<Block> &blocks, int n, int lmin, int mmax, int &
   return L >= lmin;
 }
 
-std::vector<PassPlan> plan_passes(const std::vector<Block> &blocks, int n, int m, int L,
+std::vector<PassPlan> plan_passes(std::vector<Block> blocks, int n, int m, int L,
                                   int max_ops, int max_mat_entries) {
   std::vector<PassPlan> passes;
   m = std::min(m, n);
@@ -183,7 +183,7 @@ std::vector<PassPlan> plan_passes(const std::vector<Block> &blocks, int n, int m
     PassPlan P;
     for (size_t i = first; i < blocks.size(); i++) {
       if (done[i]) continue;
-      const Block &b = blocks[i];
+      Block &b = blocks[i];
       const uint64_t need = qmask(b.qubits);
       const uint64_t touch = need | qmask(b.controls) | b.xmask;
       if (touch & blocked) {
@@ -193,7 +193,7 @@ std::vector<PassPlan> plan_passes(const std::vector<Block> &blocks, int n, int m
         S |= need;
         nops++;
         nmat += mat_entries(b);
-        P.ops.push_back(b);
+        P.ops.push_back(std::move(b));
         done[i] = 1;
         remaining--;
       } else {
@@ -219,10 +219,10 @@ std::vector<PassPlan> plan_passes(const std::vector<Block> &blocks, int n, int m
 static bool mergeable(const Block &b) {
   return b.kind == TOP_DENSE && b.controls.empty() && b.param < 0 && b.inst < 0 && b.fusable;
 }
-std::vector<Block> merge_in_passes(const std::vector<PassPlan> &passes, int K) {
+std::vector<Block> merge_in_passes(std::vector<PassPlan> passes, int K) {
   std::vector<Block> out;
-  for (const PassPlan &P : passes) {
-    std::vector<Block> ops = P.ops;
+  for (PassPlan &P : passes) {
+    std::vector<Block> &ops = P.ops;
     std::vector<char> alive(ops.size(), 1);
     for (size_t j = 0; j < ops.size(); j++) {
       if (!mergeable(ops[j])) continue;

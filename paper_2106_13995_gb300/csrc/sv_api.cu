@@ -718,6 +718,10 @@ static sv_status emit_tc_pass(CachedProgram &out, const Block &blk, int n, int p
   return SV_OK;
 }
 
+static void move_to_end(std::vector<Block> &from, std::vector<Block> &to) {
+  to.insert(to.end(), std::make_move_iterator(from.begin()), std::make_move_iterator(from.end()));
+}
+
 // Append a complex128 program of exact tensor-core passes, if every fused block of at
 // most 5 qubits qualifies: uncontrolled (wider or controlled ones stay on the
 // CUDA cores, and a program is all of one kind), digits within the exact range,
@@ -727,9 +731,9 @@ static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates,
   const int n = s->n, m = kTcTileM, L = o.L;
   std::vector<Block> blocks = fuse(gates, 5);
   if (m < n) {
-    const std::vector<PassPlan> first = plan_passes(blocks, n, m, L, kOzMaxBlocks, kMaxMatPerPass);
+    std::vector<PassPlan> first = plan_passes(blocks, n, m, L, kOzMaxBlocks, kMaxMatPerPass);
     if (first.empty()) return false;
-    std::vector<Block> merged = merge_in_passes(first, 5);
+    std::vector<Block> merged = merge_in_passes(std::move(first), 5);
     if (merged.size() < blocks.size()) blocks = std::move(merged);
   }
   bool moves = true;
@@ -788,7 +792,7 @@ static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates,
   to.ops.insert(to.ops.end(), prog.prog.ops.begin(), prog.prog.ops.end());
   to.mats.insert(to.mats.end(), prog.prog.mats.begin(), prog.prog.mats.end());
   to.passes.insert(to.passes.end(), prog.prog.passes.begin(), prog.prog.passes.end());
-  out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
+  move_to_end(blocks, out.blocks);
   return true;
 }
 
@@ -806,9 +810,9 @@ static sv_status append_gates(sv_state *s, const std::vector<Gate> &gates, const
     return set_error(SV_EUNSUPPORTED, "a fused block does not fit a shared-memory tile");
   if (o.fusion_k >= 2 && m < s->n) {
     // blocks that meet inside a pass merge (one pass-sized op instead of two)
-    const std::vector<PassPlan> first = plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass);
+    std::vector<PassPlan> first = plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass);
     if (!first.empty()) {
-      std::vector<Block> merged = merge_in_passes(first, o.fusion_k);
+      std::vector<Block> merged = merge_in_passes(std::move(first), o.fusion_k);
       int m2 = m, L2 = L;
       if (merged.size() < blocks.size() && fit_tile(merged, s->n, lmin(s->dt), mmax(s->dt, 1), m2, L2)) {
         blocks = std::move(merged);
@@ -855,7 +859,7 @@ static sv_status append_gates(sv_state *s, const std::vector<Gate> &gates, const
     std::vector<Block> seg;
     auto flush_tc = [&]() -> sv_status {
       if (seg.empty()) return SV_OK;
-      std::vector<PassPlan> passes = plan_passes(seg, s->n, m, L, kMaxOpsPerPass, mat_cap);
+      std::vector<PassPlan> passes = plan_passes(std::move(seg), s->n, m, L, kMaxOpsPerPass, mat_cap);
       if (passes.empty()) return set_error(SV_EINVAL, "internal: pass planning failed");
       for (PassPlan &P : passes) {
         for (Block &blk : P.ops)
@@ -878,13 +882,13 @@ static sv_status append_gates(sv_state *s, const std::vector<Gate> &gates, const
       SV_TRY(emit_tc_pass(out, blk, s->n, o.prec));
     }
     SV_TRY(flush_tc());
-    out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
+    move_to_end(blocks, out.blocks);
     return SV_OK;
   }
   std::vector<Block> seg;
   auto flush = [&]() -> sv_status {
     if (seg.empty()) return SV_OK;
-    std::vector<PassPlan> passes = plan_passes(seg, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass);
+    std::vector<PassPlan> passes = plan_passes(std::move(seg), s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass);
     if (passes.empty()) return set_error(SV_EINVAL, "internal: pass planning failed");
     for (const PassPlan &P : passes) SV_TRY(emit_pass(out.prog, P, b, out.op0s, {}));
     seg.clear();
@@ -895,14 +899,14 @@ static sv_status append_gates(sv_state *s, const std::vector<Gate> &gates, const
     if (tc) pad4(blk);
     const bool is_tc = tc && blk.kind == TOP_DENSE && blk.qubits.size() == 5 && blk.controls.empty() && !blk.diag;
     if (!is_tc) {
-      seg.push_back(blk);
+      seg.push_back(std::move(blk));
       continue;
     }
     SV_TRY(flush());
     SV_TRY(emit_tc_pass(out, blk, s->n, o.prec));
   }
   SV_TRY(flush());
-  out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
+  move_to_end(blocks, out.blocks);
   return SV_OK;
 }
 
@@ -939,8 +943,8 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
         if (!rest.empty()) SV_TRY(append_gates(s, rest, o, out));
         rest.clear();
         for (const std::vector<Move> &p : passes) emit_moves(out.prog, p, s->n, m, out.op0s);
-        const std::vector<Block> blocks = fuse(run, o.fusion_k);
-        out.blocks.insert(out.blocks.end(), blocks.begin(), blocks.end());
+        std::vector<Block> blocks = fuse(run, o.fusion_k);
+        move_to_end(blocks, out.blocks);
         i = e;
         continue;
       }

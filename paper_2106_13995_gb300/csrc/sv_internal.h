@@ -251,11 +251,11 @@ int max_targets(const std::vector<Block> &blocks);
 bool fit_tile(const std::vector<Block> &blocks, int n, int lmin, int mmax, int &m, int &L);
 // Empty result when some block cannot fit a tile of m qubits with L fixed low
 // qubits (callers size m and L with fit_tile first).
-std::vector<PassPlan> plan_passes(const std::vector<Block> &blocks, int n, int m, int L,
+std::vector<PassPlan> plan_passes(std::vector<Block> blocks, int n, int m, int L,
                                   int max_ops, int max_mat_entries);
 // Blocks of the planned passes in execution order, with blocks of a pass
 // merged where commuting lets them meet and the union has at most K qubits.
-std::vector<Block> merge_in_passes(const std::vector<PassPlan> &passes, int K);
+std::vector<Block> merge_in_passes(std::vector<PassPlan> passes, int K);
 // Blocks of a sequence with parametric single-qubit gates (inst >= 0) for
 // gradient programs: parametric gates become sites, X, CNOT, SWAP, Toffoli and
 // other permutations of at most 3 qubits the moves around them (TOP_SITES ops
