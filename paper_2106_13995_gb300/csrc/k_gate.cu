@@ -171,20 +171,88 @@ __global__ void k_dense(typename Cx<R>::T *__restrict__ a, uint64_t ngroups, uin
   }
 }
 
+// complex64 and K <= 2 with qubit 0 neither a target nor a control: two groups a
+// unit, 16-byte accesses, several units per trip (as K3; the same sums in the
+// same order).  On 26 qubits a 2-qubit unitary 174 us by single amplitudes and
+// 159 so, a CNOT 85 and 75, a Toffoli 51 and 40; 3 targets load as much at a
+// time either way (160 and 161).
+template <int K>
+__global__ void k_dense_pairs(float2 *__restrict__ a, uint64_t nunits, uint64_t fixed, uint64_t cmask,
+                              const __grid_constant__ DenseArgs<float, K> A) {
+  constexpr int D = 1 << K, UN = K == 1 ? 4 : 2;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < nunits; u0 += UN * stride) {
+    float4 x[UN][D];
+    uint64_t i0[UN];
+#pragma unroll
+    for (int j = 0; j < UN; j++) {
+      const uint64_t u = u0 + j * stride;
+      i0[j] = ins0_mask64(2 * u, fixed) | cmask;
+      if (u < nunits) {
+#pragma unroll
+        for (int y = 0; y < D; y++) x[j][y] = __ldcs(reinterpret_cast<const float4 *>(a + i0[j] + A.off[y]));
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < UN; j++) {
+      if (u0 + j * stride >= nunits) break;
+#pragma unroll
+      for (int r = 0; r < D; r++) {
+        float2 p = czero<float2>(), q = czero<float2>();
+#pragma unroll
+        for (int y = 0; y < D; y++) {
+          p = cfma(A.u[r * D + y], make_float2(x[j][y].x, x[j][y].y), p);
+          q = cfma(A.u[r * D + y], make_float2(x[j][y].z, x[j][y].w), q);
+        }
+        __stcs(reinterpret_cast<float4 *>(a + i0[j] + A.off[r]), make_float4(p.x, p.y, q.x, q.y));
+      }
+    }
+  }
+}
+
 // ---- K4: diagonal gate (targets and controls folded into one table) ------
+// Qubits whose 0 leaves an amplitude alone (controls, and the targets of Z, S, T
+// and phase gates) are fixed at 1, so a phase gate moves half of the state and a
+// controlled one a quarter.  Four 16-byte units per thread and trip, the table
+// in shared memory (each thread reads an entry of its own).  HBM-bound: a
+// controlled phase on 26 qubits 192 us when every amplitude passed through, 36
+// now.
 template <typename R> struct DiagArgs {
   int npos;
-  int pos[14];                  // qubit of table bit j
-  typename Cx<R>::T d[256];     // 2^npos entries, 1 where controls are not all set
+  uint32_t q0;                  // table bit of qubit 0 (complex64 units hold both of its values), or 0
+  uint64_t fixed;               // qubits fixed at 1
+  int pos[8];                   // qubit of table bit j
+  typename Cx<R>::T d[256];     // 2^npos entries
 };
 
 template <typename R>
-__global__ void k_diag(typename Cx<R>::T *__restrict__ a, uint64_t namps, const __grid_constant__ DiagArgs<R> A) {
+__global__ void __launch_bounds__(256) k_diag(typename Cx<R>::T *__restrict__ a, uint64_t nunits,
+                                              const __grid_constant__ DiagArgs<R> A) {
+  using C = typename Cx<R>::T;
+  constexpr int APU = 16 / (int)sizeof(C), UN = 4;
+  __shared__ C tab[256];
+  for (int r = threadIdx.x; r < 1 << A.npos; r += blockDim.x) tab[r] = A.d[r];
+  __syncthreads();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < namps; x += stride) {
-    uint32_t r = 0;
-    for (int j = 0; j < A.npos; j++) r |= (uint32_t)((x >> A.pos[j]) & 1ull) << j;
-    a[x] = cmul(A.d[r], a[x]);
+  for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < nunits; u0 += UN * stride) {
+    int4 x[UN];
+    uint64_t i0[UN];
+#pragma unroll
+    for (int j = 0; j < UN; j++) {
+      const uint64_t u = u0 + j * stride;
+      i0[j] = ins0_mask64(u * APU, A.fixed) | A.fixed;
+      if (u < nunits) x[j] = __ldcs(reinterpret_cast<const int4 *>(a + i0[j]));
+    }
+#pragma unroll
+    for (int j = 0; j < UN; j++) {
+      if (u0 + j * stride >= nunits) break;
+      uint32_t r = 0;
+      for (int k = 0; k < A.npos; k++) r |= (uint32_t)((i0[j] >> A.pos[k]) & 1ull) << k;
+      C *v = reinterpret_cast<C *>(&x[j]);
+      v[0] = cmul(tab[r], v[0]);
+      if (APU == 2) v[APU - 1] = cmul(tab[r | A.q0], v[APU - 1]);
+      __stcs(reinterpret_cast<int4 *>(a + i0[j]), x[j]);
+    }
   }
 }
 
@@ -235,6 +303,16 @@ static sv_status dense_k(sv_state *s, const std::vector<int> &t, const std::vect
   }
   const uint64_t ngroups = 1ull << (s->n - __builtin_popcountll(fixed));
   const int threads = 256;
+  if constexpr (K <= 2 && sizeof(R) == 4) {
+    if (!(fixed & 1) && ngroups >= 2) {
+      constexpr int UN = K == 1 ? 4 : 2;
+      k_dense_pairs<K><<<grid_for(s, (ngroups / 2 + UN - 1) / UN, threads), threads, 0, s->stream>>>(
+          reinterpret_cast<float2 *>(s->amps), ngroups / 2, fixed, cmask, A);
+      g_launches++;
+      SV_CUDA(cudaGetLastError());
+      return SV_OK;
+    }
+  }
   k_dense<R, K><<<grid_for(s, ngroups, threads), threads, 0, s->stream>>>(
       reinterpret_cast<typename Cx<R>::T *>(s->amps), ngroups, fixed, cmask, A);
   g_launches++;
@@ -301,21 +379,39 @@ template <typename R>
 static sv_status diag_launch(sv_state *s, const std::vector<int> &t, const std::vector<int> &c,
                              const std::vector<cd> &d) {
   DiagArgs<R> A{};
-  const int k = (int)t.size(), nc = (int)c.size();
-  A.npos = k + nc;
-  if (A.npos > 8) return set_error(SV_EUNSUPPORTED, "diagonal gate with more than 8 qubits");
-  for (int j = 0; j < k; j++) A.pos[j] = t[j];
-  for (int j = 0; j < nc; j++) A.pos[k + j] = c[j];
-  const int cm = ((1 << nc) - 1) << k;
+  std::vector<int> q = t;
+  q.insert(q.end(), c.begin(), c.end());
+  const int k = (int)t.size(), nq = (int)q.size(), cm = ((1 << c.size()) - 1) << k;
+  if (nq > 8) return set_error(SV_EUNSUPPORTED, "diagonal gate with more than 8 qubits");
+  auto entry = [&](int r) { return (r & cm) == cm ? d[r & ((1 << k) - 1)] : cd(1.0); };
+  // units of 16 bytes keep both values of qubit 0 (complex64)
+  const int apu = s->dt == SV_C64 && s->n >= 1 ? 2 : 1;
+  int on = 0;             // table bits fixed at 1
+  std::vector<int> free;  // the others, qubit 0 first
+  for (int j = 0; j < nq; j++) {
+    bool idle = !(apu == 2 && q[j] == 0);
+    for (int r = 0; r < (1 << nq) && idle; r++) idle = ((r >> j) & 1) || entry(r) == cd(1.0);
+    if (idle) {
+      on |= 1 << j;
+      A.fixed |= 1ull << q[j];
+    } else {
+      free.insert(q[j] == 0 ? free.begin() : free.end(), j);
+    }
+  }
+  A.npos = (int)free.size();
+  for (int j = 0; j < A.npos; j++) A.pos[j] = q[free[j]];
+  A.q0 = apu == 2 && A.npos > 0 && A.pos[0] == 0 ? 1u : 0u;
   for (int r = 0; r < (1 << A.npos); r++) {
-    cd v = ((r & cm) == cm) ? d[r & ((1 << k) - 1)] : cd(1.0);
+    int full = on;
+    for (int j = 0; j < A.npos; j++) full |= ((r >> j) & 1) << free[j];
+    const cd v = entry(full);
     A.d[r].x = (R)v.real();
     A.d[r].y = (R)v.imag();
   }
-  const uint64_t na = 1ull << s->n;
+  const uint64_t nunits = (1ull << (s->n - __builtin_popcountll(A.fixed))) / apu;
   const int threads = 256;
-  k_diag<R><<<grid_for(s, na, threads), threads, 0, s->stream>>>(
-      reinterpret_cast<typename Cx<R>::T *>(s->amps), na, A);
+  k_diag<R><<<grid_for(s, (nunits + 3) / 4, threads), threads, 0, s->stream>>>(
+      reinterpret_cast<typename Cx<R>::T *>(s->amps), nunits, A);
   g_launches++;
   SV_CUDA(cudaGetLastError());
   return SV_OK;
