@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(kMoveThreads, 7) k_moves(const __grid_constant
   const bool copies = blockIdx.x >= A.fill;
   const uint32_t tile = copies ? blockIdx.x - A.fill : blockIdx.x;
   C *amps = reinterpret_cast<C *>(P.v0);
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  pass_start();
   if (copies) {
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    pass_wait();
     constexpr uint32_t APU = 16 / sizeof(C), kUnits = (1u << kMoveBits) / APU / kMoveThreads, kBatch = 8;
     if (tid < kUnits) off[tid] = move_spread(P, tid * kMoveThreads * APU);
     const uint64_t base = A.cbase | move_spread(P, (tile << kMoveBits) | (tid * APU));
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kMoveThreads, 7) k_moves(const __grid_constant
   const uint32_t rest = loc & ~pmask;
   const C *src = static_cast<const C *>(A.src);
   C *dst = amps + (A.gbase | move_spread(P, loc));
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");   // (the indices needed no memory of the last launch)
+  pass_wait();   // (the indices needed no memory of the last launch)
   constexpr int kBatch = 128 / sizeof(C);   // 32 registers of loads in flight
 #pragma unroll
   for (int i0 = 0; i0 < 32; i0 += kBatch) {
@@ -173,16 +173,8 @@ sv_status launch_moves(sv_state *s, const TilePass &p, cudaStream_t stream) {
     A.gbase = j > 0 ? base_of(j - 1) : 0;
     A.dst = scratch + (j & 1) * chunk;
     A.src = scratch + ((j + 1) & 1) * chunk;
-    cudaLaunchAttribute early;
-    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    early.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(A.copy + A.fill);
-    cfg.blockDim = dim3(kMoveThreads);
-    cfg.stream = stream;
-    cfg.attrs = &early;
-    cfg.numAttrs = j > 0 ? 1 : 0;
-    SV_CUDA(s->dt == SV_C64 ? cudaLaunchKernelEx(&cfg, k_moves<float2>, p, A) : cudaLaunchKernelEx(&cfg, k_moves<double2>, p, A));
+    SV_CUDA(launch_early(s->dt == SV_C64 ? k_moves<float2> : k_moves<double2>, dim3(A.copy + A.fill), kMoveThreads, 0,
+                         stream, p, A));
     g_launches++;
   }
   return SV_OK;

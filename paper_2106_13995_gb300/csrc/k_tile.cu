@@ -212,6 +212,8 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
 template <typename R>
 __global__ void __launch_bounds__(kTilePassThreads, kTilePassMinBlocks) k_tile(const __grid_constant__ TilePass P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_start();
+  pass_wait();
   tile_body<R, false>(P, blockIdx.x, blockIdx.y, smem_raw);
 }
 
@@ -377,6 +379,8 @@ static bool launch_inl(sv_state *s, const TilePass &p, const HostPass &h, dim3 g
   Inl inl;   // copied into the launch
   if (!build_inline(p, h, inl, threads)) return false;
   st = func_attr_once((const void *)k_tile_inl<Inl>, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10);
+  // (not launch_early: with a parameter block of several KB that costs more than
+  // it hides, 18 qubits of U3 + CZ 368 us and 436)
   if (st == SV_OK) k_tile_inl<Inl><<<grid, threads, smem, stream>>>(p, inl);
   return true;
 }
@@ -420,6 +424,8 @@ __global__ void __launch_bounds__(kTilePassThreads) k_tile_tperm(const __grid_co
   using UN = Unit<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *v = reinterpret_cast<C *>(smem_raw);
+  pass_start();
+  pass_wait();
   const uint32_t TS = 1u << P.m;
   const uint64_t base = tile_base(P, blockIdx.x);
   C *g0 = reinterpret_cast<C *>(P.tbl0 ? P.tbl0[blockIdx.y] : P.v0);
@@ -484,11 +490,10 @@ static sv_status launch_tile_tperm(sv_state *s, const TilePass &p, int batch, cu
   dim3 grid((unsigned)(1ull << (p.n - p.m)), (unsigned)batch);
   const int threads = tile_threads(p.m, s->dt);
   if (s->dt == SV_C64)
-    k_tile_tperm<float><<<grid, threads, smem, stream>>>(p);
+    SV_CUDA(launch_early(k_tile_tperm<float>, grid, threads, smem, stream, p));
   else
-    k_tile_tperm<double><<<grid, threads, smem, stream>>>(p);
+    SV_CUDA(launch_early(k_tile_tperm<double>, grid, threads, smem, stream, p));
   g_launches++;
-  SV_CUDA(cudaGetLastError());
   return SV_OK;
 }
 
@@ -529,11 +534,10 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
                   launch_inl<TileInline>(s, p, *host, grid, threads, smem, stream, st)))
     SV_TRY(st);
   else if (s->dt == SV_C64)
-    k_tile<float><<<grid, threads, smem, stream>>>(p);
+    SV_CUDA(launch_early(k_tile<float>, grid, threads, smem, stream, p));
   else
-    k_tile<double><<<grid, threads, smem, stream>>>(p);
+    SV_CUDA(launch_early(k_tile<double>, grid, threads, smem, stream, p));
   g_launches++;
-  SV_CUDA(cudaGetLastError());
   return SV_OK;
 }
 

@@ -166,6 +166,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   uint64_t copied = 0, c = 0;
   if (tid == 0)
     for (; copied < 2 && copied < total; copied++) copy_b(copied);
+  pass_start();
+  pass_wait();
   uint64_t thr = tid & segmask;
   for (uint32_t x = tid >> P.L; x; x &= x - 1) thr |= 1ull << P.hi_pos[__ffs(x) - 1];
   double2 *amps = reinterpret_cast<double2 *>(P.v0);
@@ -430,9 +432,8 @@ sv_status launch_tile_oz(sv_state *s, const TilePass &p, const HostPass &host, c
   }
   const uint64_t ntiles = 1ull << (p.n - p.m);
   const int grid = (int)std::min<uint64_t>(ntiles, (uint64_t)s->sm_count);
-  k_tile_oz<<<grid, kOzThreads, kOzSmem, stream>>>(p, T);
+  SV_CUDA(launch_early(k_tile_oz, dim3((unsigned)grid), kOzThreads, kOzSmem, stream, p, T));
   g_launches++;
-  SV_CUDA(cudaGetLastError());
   return SV_OK;
 }
 

@@ -170,18 +170,10 @@ __global__ void __launch_bounds__(kSitesThreads, 3) k_tile_sites(const __grid_co
   auto copy8 = [](uint32_t dst, const float2 *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
   };
-  for (uint32_t i = 0; i * T + threadIdx.x < nunits; i++) {
-    const uint64_t g = goff(i);
-    const uint32_t l = (i * T + threadIdx.x) * 2, a = swb<float>(l), b = swb<float>(l + 1);
-    copy8(vs0 + a, &g0[g]);
-    copy8(vs0 + b, &g0[g + 1]);
-    if (TWO) {
-      copy8(vs1 + a, &g1[g]);
-      copy8(vs1 + b, &g1[g + 1]);
-    }
-  }
   // the pass's ops, descriptors and this set's matrices next to the tile: read
-  // from global memory op by op they were a chain of three latencies each
+  // from global memory op by op they were a chain of three latencies each (and
+  // they were uploaded before the call's first pass)
+  pass_start();
   for (uint32_t k = threadIdx.x; k < (uint32_t)P.nops * kSitesEntry; k += T) {
     const uint32_t oi = k / kSitesEntry, w = k % kSitesEntry;
     const uint4 *op = reinterpret_cast<const uint4 *>(P.ops + oi);
@@ -195,6 +187,17 @@ __global__ void __launch_bounds__(kSitesThreads, 3) k_tile_sites(const __grid_co
     } else {
       const int mat = reinterpret_cast<const int *>(d + 4)[(w - 8) / 2];
       if (mat >= 0) ent[k] = __ldg(reinterpret_cast<const uint4 *>(pm + mat) + (w & 1));
+    }
+  }
+  pass_wait();
+  for (uint32_t i = 0; i * T + threadIdx.x < nunits; i++) {
+    const uint64_t g = goff(i);
+    const uint32_t l = (i * T + threadIdx.x) * 2, a = swb<float>(l), b = swb<float>(l + 1);
+    copy8(vs0 + a, &g0[g]);
+    copy8(vs0 + b, &g0[g + 1]);
+    if (TWO) {
+      copy8(vs1 + a, &g1[g]);
+      copy8(vs1 + b, &g1[g + 1]);
     }
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -228,10 +231,8 @@ sv_status launch_tile_sites(sv_state *s, const TilePass &p, int batch, int threa
   const dim3 grid((unsigned)(1ull << (p.n - p.m)), (unsigned)batch);
   const void *fn = p.nvec > 1 ? (const void *)k_tile_sites<true> : (const void *)k_tile_sites<false>;
   SV_TRY(func_attr_once(fn, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 << 10));
-  if (p.nvec > 1) k_tile_sites<true><<<grid, threads, smem, stream>>>(p);
-  else k_tile_sites<false><<<grid, threads, smem, stream>>>(p);
+  SV_CUDA(launch_early(p.nvec > 1 ? k_tile_sites<true> : k_tile_sites<false>, grid, threads, smem, stream, p));
   g_launches++;
-  SV_CUDA(cudaGetLastError());
   return SV_OK;
 }
 

@@ -14,6 +14,7 @@
 #include <mutex>
 #include <string>
 #include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include "../../include/sv_api.h"
@@ -380,6 +381,23 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec);
 // cache for this circuit's shape (sv_batch.cu), if a pair in it beat the
 // defaults.
 void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt, Opts &o);
+// Launch a kernel whose every CTA calls pass_wait() before it reads or writes
+// what the kernel before it in the stream wrote or read.
+template <typename... P, typename... A>
+cudaError_t launch_early(void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A &&...args) {
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, std::forward<A>(args)...);
+}
+
 // permutation runs (k_moves.cu)
 struct Move {             // X on `target` where all of `controls` are 1
   uint64_t controls;
