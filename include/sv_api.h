@@ -216,9 +216,13 @@ sv_status sv_apply_gate(sv_state *s, const int32_t *targets, int k, const int32_
  * their products) only move amplitudes inside the tile: a pass made only of
  * such blocks is composed on the host into one gather table per setting of
  * its global control qubits (at most 5 of them, tables within half the
- * program area) and moves each amplitude once, exactly; a state known to be
- * a basis state (see sv_set_basis) takes no pass at all when every gate
- * maps basis states to basis states.
+ * program area) and moves each amplitude once, exactly.  From 15 qubits on and
+ * with fusion_k and tile_m left at 0, a long run of such gates is one move of
+ * every amplitude within chunks of 2^22 (see sv_workspace_bytes).  A state
+ * known to be a basis state (see sv_set_basis) takes no pass at all when every
+ * gate maps basis states to basis states; single-qubit gates on it in front of
+ * such a run are written as the product state they make (not while the stream
+ * is being captured).
  * Errors: SV_EINVAL (malformed op, width mismatch), SV_ENOMEM (program does
  * not fit the workspace). */
 sv_status sv_apply_circuit(sv_state *s, const sv_circuit *c, const double *params,

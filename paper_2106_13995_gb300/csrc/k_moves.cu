@@ -21,10 +21,10 @@
 //
 // Bound: the load-store pipe.  The gather reads 8 bytes from each of 32 lines a
 // warp (one line a clock: 14 us a chunk), the words of a 222-gate run add 8 us;
-// a chunk of 32 MB takes 37 us, 10 of them HBM.  The 7-bit multiplier on 29
-// qubits: 28.8 ms in tables, 8.8 ms here, of which the moves are 4.7 (10.6 with
-// the launches one after the other, 10.1 with copying CTAs first; chunks of
-// 2^23 9.0, of 2^20 23 in two passes).
+// a chunk of 32 MB takes 36 us, 10 of them HBM.  The 7-bit multiplier on 29
+// qubits took 15 table passes of 1.6 ms; its moves take 4.6 ms (6.4 with the
+// launches one after the other, 5.9 with the copying CTAs first, 4.8 in chunks
+// of 2^23).
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -313,6 +313,106 @@ void emit_moves(DeviceProgram &prog, const std::vector<Move> &moves, int n, int 
   prog.mats.insert(prog.mats.end(), q, q + ops.size() * sizeof(MoveOp));
   op0s.push_back((uint32_t)prog.ops.size());
   prog.passes.push_back(tp);
+}
+
+// ---------------------------------------------------------------------------
+// product states
+// ---------------------------------------------------------------------------
+// K16: amplitude x = product over q of v[q][bit q of x], written once.  Factors
+// of six bits at a time come from tables (FP64, built once per persistent CTA);
+// a chunk of 2^12 amplitudes multiplies its upper factors into one table in
+// FP64, and an amplitude is one product of two entries in the state's type (one
+// FP64 product each would be bound by the FP64 pipe).  The Hadamards in front of
+// the 29-qubit multiplier took a tile pass of 3.4 ms (FP32-bound, 128
+// multiply-adds an amplitude), the product 0.7 ms.
+constexpr int kProdTables = 6;   // of six bits: 36 >= 34 qubits
+struct ProductArgs {
+  double2 v[6 * kProdTables][2];
+};
+template <typename R>
+__global__ void __launch_bounds__(256) k_product(typename Cx<R>::T *__restrict__ a, uint64_t nchunks,
+                                                 const __grid_constant__ ProductArgs A) {
+  using C = typename Cx<R>::T;
+  __shared__ double2 tab[kProdTables][64];
+  __shared__ __align__(16) C low[64], up[2][64];
+  const uint32_t tid = threadIdx.x;
+  for (uint32_t e = tid; e < kProdTables * 64; e += 256) {
+    double2 p = make_double2(1.0, 0.0);
+    for (uint32_t b = 0; b < 6; b++) p = cmul(A.v[6 * (e >> 6) + b][(e >> b) & 1u], p);
+    tab[e >> 6][e & 63u] = p;
+  }
+  __syncthreads();
+  auto cast = [](double2 p) {
+    C c;
+    c.x = (R)p.x;
+    c.y = (R)p.y;
+    return c;
+  };
+  if (tid < 64) low[tid] = cast(tab[0][tid]);
+  int turn = 0;
+  for (uint64_t c = blockIdx.x; c < nchunks; c += gridDim.x, turn ^= 1) {
+    if (tid < 64) {
+      double2 p = tab[1][tid];
+      for (int k = 2; k < kProdTables; k++) p = cmul(tab[k][(c >> (6 * (k - 2))) & 63u], p);
+      up[turn][tid] = cast(p);
+    }
+    __syncthreads();   // (the table of the chunk before last has been read)
+    constexpr uint32_t APU = 16 / sizeof(C), kTrips = 4096 / APU / 256;
+#pragma unroll
+    for (uint32_t i = 0; i < kTrips; i++) {
+      const uint32_t x = (tid + 256 * i) * APU;
+      __align__(16) C o[APU];
+#pragma unroll
+      for (uint32_t j = 0; j < APU; j++) o[j] = cmul(up[turn][x >> 6], low[(x & 63u) + j]);
+      __stcs(reinterpret_cast<int4 *>(a + (c << 12) + x), *reinterpret_cast<const int4 *>(o));
+    }
+  }
+}
+
+bool product_of(const std::vector<Gate> &gates, int n, std::vector<cd> &U) {
+  U.assign(4 * (size_t)n, cd(0.0));
+  for (int q = 0; q < n; q++) U[4 * q] = U[4 * q + 3] = 1.0;
+  for (const Gate &g : gates) {
+    if (g.targets.size() != 1 || !g.controls.empty() || g.inst >= 0 || g.param >= 0 || g.grad_gen > 0 ||
+        g.fixed_structure)
+      return false;
+    cd *u = &U[4 * (size_t)g.targets[0]];
+    const cd a = u[0], b = u[1], c = u[2], d = u[3];
+    u[0] = g.U[0] * a + g.U[1] * c;
+    u[1] = g.U[0] * b + g.U[1] * d;
+    u[2] = g.U[2] * a + g.U[3] * c;
+    u[3] = g.U[2] * b + g.U[3] * d;
+  }
+  return true;
+}
+
+sv_status launch_product(sv_state *s, const TilePass &p, const HostPass &host, cudaStream_t stream) {
+  if (!s->basis_known || s->n < 12) return set_error(SV_EINVAL, "internal: product pass on an unknown state");
+  ProductArgs A;
+  const double *u = reinterpret_cast<const double *>(host.mats + 16 * (size_t)p.mat0);
+  for (int q = 0; q < 6 * kProdTables; q++)
+    for (int r = 0; r < 2; r++) {
+      if (q < s->n) {
+        const double *e = u + 8 * q + 4 * r + 2 * ((s->basis_index >> q) & 1);   // row r, column: the basis bit
+        A.v[q][r] = make_double2(e[0], e[1]);
+      } else {
+        A.v[q][r] = make_double2(1.0, 0.0);
+      }
+    }
+  // the basis state's own phase, into a qubit's two factors
+  for (int r = 0; r < 2; r++) {
+    const cd v = cd(A.v[0][r].x, A.v[0][r].y) * s->basis_amp;
+    A.v[0][r] = make_double2(v.real(), v.imag());
+  }
+  const uint64_t chunks = 1ull << (s->n - 12);
+  const unsigned grid = (unsigned)std::min<uint64_t>(chunks, (uint64_t)s->sm_count * 8);
+  if (s->dt == SV_C64)
+    k_product<float><<<grid, 256, 0, stream>>>(reinterpret_cast<float2 *>(p.v0), chunks, A);
+  else
+    k_product<double><<<grid, 256, 0, stream>>>(reinterpret_cast<double2 *>(p.v0), chunks, A);
+  g_launches++;
+  SV_CUDA(cudaGetLastError());
+  return SV_OK;
 }
 
 }  // namespace sv

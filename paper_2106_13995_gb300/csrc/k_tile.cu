@@ -500,6 +500,10 @@ static sv_status launch_tile_tperm(sv_state *s, const TilePass &p, int batch, cu
 sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStream_t stream,
                               const HostPass *host) {
   if (p.flags & kPassTable) return launch_tile_tperm(s, p, batch, stream);
+  if (p.flags & kPassProduct) {
+    if (batch != 1 || !host) return set_error(SV_EINVAL, "internal: product pass over a batch");
+    return launch_product(s, p, *host, stream);
+  }
   if (p.flags & kPassMoves) {
     if (batch != 1) return set_error(SV_EINVAL, "internal: permutation run over a batch");
     return launch_moves(s, p, stream);

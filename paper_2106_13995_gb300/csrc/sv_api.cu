@@ -925,6 +925,28 @@ static size_t count_passes(const sv_state *s, const std::vector<Gate> &gates, co
   return plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass).size();
 }
 
+// Single-qubit gates in front of everything else, on a known basis state, as a
+// product pass; false: nothing appended.
+static bool append_product(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
+  std::vector<cd> U;
+  if (!o.product || !out.prog.passes.empty() || !product_of(gates, s->n, U)) return false;
+  TilePass tp;
+  std::memset(&tp, 0, sizeof(tp));
+  tp.n = s->n;
+  tp.m = s->n;
+  tp.nvec = 1;
+  tp.flags = kPassProduct;
+  while (out.prog.mats.size() % 16) out.prog.mats.push_back(0);
+  tp.mat0 = (uint32_t)(out.prog.mats.size() / 16);
+  const uint8_t *u = reinterpret_cast<const uint8_t *>(U.data());
+  out.prog.mats.insert(out.prog.mats.end(), u, u + U.size() * sizeof(cd));
+  out.op0s.push_back((uint32_t)out.prog.ops.size());
+  out.prog.passes.push_back(tp);
+  std::vector<Block> blocks = fuse(gates, o.fusion_k);
+  move_to_end(blocks, out.blocks);
+  return true;
+}
+
 static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gates, const Opts &o,
                                        CachedProgram &out) {
   std::vector<Gate> rest;   // gates not yet in the program
@@ -933,14 +955,33 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
   while (o.moves && i < gates.size()) {
     std::vector<Move> moves;
     size_t e = i;
-    while (e < gates.size() && gate_moves(gates[e], moves)) e++;
-    if (e - i >= kMovesMinGates) {
-      const std::vector<Gate> run(gates.begin() + i, gates.begin() + e);
+    // (a plain X that comes first on its qubit goes with the gates before the
+    // run: it would only add a qubit to those the run moves)
+    std::vector<Gate> run, before;
+    uint64_t touched = 0;
+    for (; e < gates.size(); e++) {
+      const Gate &g = gates[e];
+      uint64_t q = 0;
+      for (int t : g.targets) q |= 1ull << t;
+      for (int t : g.controls) q |= 1ull << t;
+      std::vector<Move> mv;
+      if (!gate_moves(g, mv)) break;
+      const bool first = g.targets.size() == 1 && g.controls.empty() && !(q & touched) && !rest.empty();
+      if (first) {
+        before.push_back(g);
+      } else {
+        run.push_back(g);
+        moves.insert(moves.end(), mv.begin(), mv.end());
+        touched |= q;
+      }
+    }
+    if (run.size() >= kMovesMinGates) {
       const std::vector<std::vector<Move>> passes = plan_moves(moves, m);
       // (at most 9 ops of 16 bytes a move, 8 of them for many controls)
       const bool fits = out.prog.mats.size() + 9 * 16 * moves.size() + 256 * passes.size() <= kWsProgBytes / 2;
       if (fits && count_passes(s, run, o) >= moves_worth(s->n) * passes.size()) {
-        if (!rest.empty()) SV_TRY(append_gates(s, rest, o, out));
+        rest.insert(rest.end(), before.begin(), before.end());
+        if (!rest.empty() && !append_product(s, rest, o, out)) SV_TRY(append_gates(s, rest, o, out));
         rest.clear();
         for (const std::vector<Move> &p : passes) emit_moves(out.prog, p, s->n, m, out.op0s);
         std::vector<Block> blocks = fuse(run, o.fusion_k);
@@ -987,11 +1028,12 @@ sv_status upload_program(sv_state *s, const CachedProgram &cp) {
 }
 
 sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,
-                      ProgramRef *out, Opts *o_out) {
+                      ProgramRef *out, Opts *o_out, bool basis) {
   if (!s) return set_error(SV_EINVAL, "null state");
   if (!c) return set_error(SV_EINVAL, "null circuit");
   Opts o = resolve(s, opt, 1);
   tuned_options(s, c, opt, o);
+  o.product = basis && o.moves;
   KeyBytes k;
   k.val((int)0x51);
   circuit_key(k, c);
@@ -1003,6 +1045,7 @@ sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, co
   k.val(o.tc_in_tile);
   k.val(o.oz);
   k.val(o.moves);
+  k.val(o.product);
   k.val((int)s->dt);
   if (params && c->n_params > 0) k.bytes(params, sizeof(double) * c->n_params);
   const uint64_t h = k.hash();
@@ -1245,13 +1288,22 @@ sv_status sv_apply_circuit(sv_state *s, const sv_circuit *c, const double *param
   }
   ProgramRef cp;
   Opts o;
-  SV_TRY(get_program(s, c, params, opt, &cp, &o));
+  // a program for the basis state the handle knows of; not where the caller
+  // records the launches, which may replay them on another state
+  cudaStreamCaptureStatus recording = cudaStreamCaptureStatusNone;
+  if (s && s->basis_known) SV_CUDA(cudaStreamIsCapturing(s->stream, &recording));
+  SV_TRY(get_program(s, c, params, opt, &cp, &o,
+                     s && s->basis_known && recording == cudaStreamCaptureStatusNone));
+  sv_status st = SV_OK;
+  if (o.mode == SV_MODE_PER_GATE) {
+    st = run_blocks_per_gate(s, cp->blocks);
+  } else if ((st = upload_program(s, *cp)) == SV_OK) {
+    LaunchEnv E;
+    E.v0 = s->amps;
+    st = launch_program(s, cp->prog, cp->lay, cp->op0s, E);
+  }
   s->basis_known = false;
-  if (o.mode == SV_MODE_PER_GATE) return run_blocks_per_gate(s, cp->blocks);
-  SV_TRY(upload_program(s, *cp));
-  LaunchEnv E;
-  E.v0 = s->amps;
-  return launch_program(s, cp->prog, cp->lay, cp->op0s, E);
+  return st;
 }
 
 sv_status sv_plan_info(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,

@@ -145,6 +145,10 @@ constexpr uint32_t kPassOz = 0x1000;
 // amplitudes (qubits hi_pos[0..m)); mat0: 16-byte index of its MoveDesc
 // (k_moves.cu)
 constexpr uint32_t kPassMoves = 0x2000;
+// TilePass.flags: the state, a known basis state, through one single-qubit gate
+// per qubit, written as the product it is; mat0: 16-byte index of 2 x 2
+// complex128 matrices of the n qubits (host copy; k_moves.cu)
+constexpr uint32_t kPassProduct = 0x4000;
 constexpr int kTcTileM = 12;          // tile size that gives M = 128 groups for a 5-qubit block
 size_t tc_tile_smem(sv_prec mode);    // shared memory of a 12-qubit tile pass with TOP_TC ops
 struct TilePass {
@@ -374,6 +378,7 @@ struct Opts {   // all int: hashed as key bytes, so no padding
   int tc_in_tile = 0;
   int oz = 0;   // complex128: blocks of 5 qubits on the tensor cores where they all qualify
   int moves = 0;   // runs of permutation gates as moves (k_moves.cu)
+  int product = 0;   // the state is a known basis state when the program runs
 };
 constexpr int kSmall128 = 17;   // widest complex128 state with the small-state plan
 Opts resolve(const sv_state *s, const sv_options *o, int nvec);
@@ -408,6 +413,10 @@ bool gate_moves(const Gate &g, std::vector<Move> &out);
 std::vector<std::vector<Move>> plan_moves(const std::vector<Move> &moves, int m);
 void emit_moves(DeviceProgram &prog, const std::vector<Move> &moves, int n, int m, std::vector<uint32_t> &op0s);
 sv_status launch_moves(sv_state *s, const TilePass &p, cudaStream_t stream);
+// Single-qubit gates before a run, on a known basis state: one matrix per qubit.
+struct HostPass;
+bool product_of(const std::vector<Gate> &gates, int n, std::vector<cd> &U);
+sv_status launch_product(sv_state *s, const TilePass &p, const HostPass &host, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------
 // program caches
@@ -504,8 +513,9 @@ struct CachedProgram {
 };
 using ProgramRef = std::shared_ptr<const CachedProgram>;
 constexpr size_t kProgramCacheDefault = 2048;
+// basis: the program will run on the basis state s knows it holds.
 sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,
-                      ProgramRef *out, Opts *o_out);
+                      ProgramRef *out, Opts *o_out, bool basis = false);
 sv_status upload_program(sv_state *s, const CachedProgram &cp);
 // Set a kernel attribute once per (kernel, device, attribute, value); thread-safe.
 sv_status func_attr_once(const void *fn, int device, cudaFuncAttribute attr, int value);

@@ -129,3 +129,36 @@ def test_in_batches_graphs_and_small_workspaces(svlib):
     torch.cuda.synchronize()
     assert torch.equal(amps, a[3].amps)
     N.lib().sv_destroy(h)
+
+
+@pytest.mark.parametrize("n,dt", [(15, "c64"), (16, "c128"), (19, "c64")])
+def test_product_states_before_a_run(svlib, oracle, n, dt):
+    """Single-qubit gates on a known basis state (with a phase of its own), then
+    a run: against the same circuit on a state the handle does not know, and the
+    oracle's product; the state is not taken for known afterwards."""
+    from paper_2106_13995_gb300 import _native as N
+    from paper_2106_13995_gb300 import circuit as B
+    rng = np.random.default_rng(n)
+    c = B.Circuit(n)
+    for q in range(n):
+        for name in ("H", "U3", "T", "X")[:int(rng.integers(0, 5))]:
+            c.append(name, (q,), tuple(rng.uniform(0, 6, 3)) if name == "U3" else (), ())
+    for op in reversible(B, n, 150, rng).ops:
+        c.ops.append(op)
+    ph = B.Circuit(n).append("S", (1,), (), ())
+    m, p = svlib.marshal(c), svlib.marshal(ph)
+    index = int(rng.integers(1 << n)) | 2
+    a, b = (svlib.StateVector(n, dt).set_basis(index) for _ in range(2))
+    for s in (a, b):
+        s.apply_circuit(p)
+    N.check(N.lib().sv_mark_modified(b.h))
+    for s in (a, b):
+        s.apply_circuit(m)
+    want = b.numpy().astype(np.complex128)
+    # a product of n factors rounded twice against tile passes of 3-qubit blocks
+    tol = 64 * np.finfo(np.float32 if dt == "c64" else np.float64).eps
+    assert np.max(np.abs(a.numpy() - want)) <= tol * np.max(np.abs(want))
+    for s in (a, b):
+        s.apply_circuit(m)
+    want = b.numpy().astype(np.complex128)
+    assert np.max(np.abs(a.numpy() - want)) <= 4 * tol * np.max(np.abs(want))
