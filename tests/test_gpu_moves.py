@@ -162,3 +162,44 @@ def test_product_states_before_a_run(svlib, oracle, n, dt):
         s.apply_circuit(m)
     want = b.numpy().astype(np.complex128)
     assert np.max(np.abs(a.numpy() - want)) <= 4 * tol * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("n,dt", [(16, "c64"), (16, "c128")])
+def test_recorded_launches_replay_on_other_states(svlib, n, dt):
+    """Dense gates, a run and dense gates again, recorded by the caller from a
+    known basis state: replays act on whatever the state holds (no product state
+    is recorded), as the same calls do."""
+    from paper_2106_13995_gb300 import circuit as B
+    rng = np.random.default_rng(n)
+    c = B.Circuit(n)
+    for q in range(n):
+        c.append("H", (q,), (), ())
+    for op in reversible(B, n, 150, rng).ops:
+        c.ops.append(op)
+    for q in range(n):
+        c.append("RY", (q,), (0.1 + 0.2 * q,), ())
+    m = svlib.marshal(c)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        s = svlib.StateVector(n, dt, stream=side)
+        s.set_basis(3)
+        s.amps.zero_()
+        s.amps[6] = 1.0
+        s.apply_circuit(m, opts=svlib.options())
+        from paper_2106_13995_gb300 import _native as N
+        N.check(N.lib().sv_mark_modified(s.h))
+        s.apply_circuit(m)          # the program that is recorded, resident
+        s.set_basis(3)
+        side.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            s.apply_circuit(m)
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(1)
+        s.amps.normal_(generator=gen)
+        t = svlib.StateVector(n, dt, stream=side)
+        t.amps.copy_(s.amps)
+        g.replay()
+        t.apply_circuit(m)
+        side.synchronize()
+        assert torch.equal(s.amps, t.amps)
