@@ -181,12 +181,14 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
         for (uint32_t l = threadIdx.x; l < TS; l += blockDim.x) v1[l] = czero<C>();
         break;
       case TOP_DOT: {
-        R part = 0;
+        R part = 0, norm = 0;
         for (uint32_t l = threadIdx.x; l < TS; l += blockDim.x) {
           const C a = v0[l], c = v1[l];   // same slot in both vectors: the swizzle cancels
           part += a.x * c.x + a.y * c.y;
+          norm += a.x * a.x + a.y * a.y;
         }
-        block_acc<R>(part, acc + op.slot);
+        block_acc<R>(part, acc + op.mat);
+        block_acc<R>(norm, acc + op.mat + 1);
         break;
       }
       default:

@@ -51,7 +51,7 @@ enum TileOpKind : uint8_t {
   TOP_GRAD = 2,      // acc[slot] += Im <v1 | G v0>, G = X/Y/Z/P1(-2) on one local target
   TOP_PAULI = 3,     // v1[l ^ xm] += c * phase * (-1)^{popcount(l & zm)} v0[l]
   TOP_ZERO = 4,      // v1 <- 0
-  TOP_DOT = 5,       // acc[slot] += Re <v0 | v1>
+  TOP_DOT = 5,       // acc[mat] += Re <v0 | v1>, acc[mat + 1] += <v0 | v0>
   TOP_TC = 6,        // 5-qubit dense block on the tensor cores (12-qubit tiles)
   TOP_PERM = 7,      // permutation block (k = 1..3): member y moves to member perm[y]; controls as TOP_DENSE
   TOP_GRADU = 8,     // TOP_GRAD then the 1-qubit matrix (per-batch pool) on both vectors, in one sweep
@@ -83,7 +83,7 @@ struct TileOp {
   uint32_t mat;       // offset (complex entries) into the matrix pool; TOP_PAULI: coeff index
   uint32_t gcmask_lo; // controls outside the tile, as a mask of global bits (low 32)
   uint16_t gcmask_hi; // ... bits 32..47
-  int16_t slot;       // accumulator slot (TOP_GRAD / TOP_DOT); TOP_PAULI: x mask (local)
+  int16_t slot;       // accumulator slot (TOP_GRAD); TOP_PAULI: x mask (local)
 };
 static_assert(sizeof(TileOp) == 32, "TileOp must stay 32 bytes");
 

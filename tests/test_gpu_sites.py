@@ -59,3 +59,43 @@ def test_passes_beyond_the_op_count(svlib, oracle):
     psi, lam = svlib.StateVector(n, "c64").set_basis(0), svlib.StateVector(n, "c64")
     ev, g = svlib.adjoint_grad(psi, lam, c, p, W.tfim(n))
     check(oracle, c, p, W.tfim(n), ev, g)
+
+
+def test_energy_of_long_circuits(svlib, oracle):
+    """The norm that FP32 rounding adds or takes is divided out: energies of 120
+    layers within 2^-22 of the terms' weights (a sum of FP32 products in FP64;
+    undivided, 1440 gates drift by several times that), over several seeds."""
+    n, layers = 6, 120
+    c = W.hea(n, layers)
+    terms = W.tfim(n)
+    psi, lam = svlib.StateVector(n, "c64"), svlib.StateVector(n, "c64")
+    for seed in range(6):
+        p = W.hea_params(1, c.n_params, seed)[0] * 0.1
+        ev, g = svlib.adjoint_grad(psi.set_basis(0), lam, c, p, terms)
+        ev_o, g_o, _ = oracle.adjoint_grad(c, p, terms)
+        # the angles' matrices and 1440 gates' rounding turn the state as well:
+        # a random walk of 2^-24 a gate
+        tol = (2.0 ** -22 + 2.0 ** -24 * np.sqrt(2 * c.n_params)) * sum(abs(t[2]) for t in terms)
+        assert abs(ev - ev_o) <= tol
+    # a state the handle does not know is not taken for a unit vector
+    half = np.zeros(1 << n, dtype=np.complex64)
+    half[0] = 0.5
+    ev4, g4 = svlib.adjoint_grad(psi.load(half), lam, c, p, terms)
+    assert abs(4 * ev4 - ev) <= 1e-4 * abs(ev) and np.max(np.abs(4 * g4 - g)) <= 1e-4 * max(1, np.max(np.abs(g)))
+
+
+def test_more_accumulators_than_15_bits(svlib):
+    """22800 parameters, 34200 probe components: the energy's accumulator lies
+    behind them (complex128, whose probes are one per parameter, as reference;
+    FP32 rounding of 22800 gates grows as a random walk to 1e-5)."""
+    n = 6
+    c = W.hea(n, 1900)
+    p = W.hea_params(1, c.n_params, 3)[0] * 0.05
+    out = []
+    for dt in ("c64", "c128"):
+        psi, lam = svlib.StateVector(n, dt).set_basis(0), svlib.StateVector(n, dt)
+        out.append(svlib.adjoint_grad(psi, lam, c, p, W.tfim(n)))
+        psi.close()
+        lam.close()
+    (e0, g0), (e1, g1) = out
+    assert abs(e0 - e1) <= 1e-3 and np.max(np.abs(g0 - g1)) <= 1e-3
