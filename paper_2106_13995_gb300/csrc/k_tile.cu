@@ -196,6 +196,7 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
     }
   }
   __syncthreads();
+  if constexpr (!COH) pass_start();
   const bool store0 = !(P.flags & 2u), store1 = P.nvec > 1 && !(P.flags & 4u);
   for (uint32_t i = 0; i * blockDim.x + threadIdx.x < nunits; i++) {
     const uint32_t l = (i * blockDim.x + threadIdx.x) * UN::APU;
@@ -214,7 +215,6 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
 template <typename R>
 __global__ void __launch_bounds__(kTilePassThreads, kTilePassMinBlocks) k_tile(const __grid_constant__ TilePass P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pass_start();
   pass_wait();
   tile_body<R, false>(P, blockIdx.x, blockIdx.y, smem_raw);
 }
@@ -225,6 +225,7 @@ template <class Inl>
 __global__ void __launch_bounds__(kTilePassThreads, kTilePassMinBlocks)
     k_tile_inl(const __grid_constant__ TilePass P, const __grid_constant__ Inl I) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_wait();
   tile_body<float, false, true, Inl>(P, blockIdx.x, 0, smem_raw, &I);
 }
 static_assert(sizeof(TilePass) + sizeof(TileInline) <= 32000, "kernel parameters exceed 32 KB");
@@ -381,9 +382,9 @@ static bool launch_inl(sv_state *s, const TilePass &p, const HostPass &h, dim3 g
   Inl inl;   // copied into the launch
   if (!build_inline(p, h, inl, threads)) return false;
   st = func_attr_once((const void *)k_tile_inl<Inl>, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10);
-  // (not launch_early: with a parameter block of several KB that costs more than
-  // it hides, 18 qubits of U3 + CZ 368 us and 436)
-  if (st == SV_OK) k_tile_inl<Inl><<<grid, threads, smem, stream>>>(p, inl);
+  if (st != SV_OK) return true;
+  const cudaError_t e = launch_early(k_tile_inl<Inl>, grid, threads, smem, stream, p, inl);
+  if (e != cudaSuccess) st = cuda_error(e, "k_tile_inl");
   return true;
 }
 
@@ -426,7 +427,6 @@ __global__ void __launch_bounds__(kTilePassThreads) k_tile_tperm(const __grid_co
   using UN = Unit<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *v = reinterpret_cast<C *>(smem_raw);
-  pass_start();
   pass_wait();
   const uint32_t TS = 1u << P.m;
   const uint64_t base = tile_base(P, blockIdx.x);
@@ -460,6 +460,7 @@ __global__ void __launch_bounds__(kTilePassThreads) k_tile_tperm(const __grid_co
     }
   }
   __syncthreads();
+  pass_start();
   for (uint32_t i0 = 0; i0 * blockDim.x + threadIdx.x < nunits; i0 += kBatch) {
     uint16_t src[kBatch][UN::APU];
 #pragma unroll

@@ -166,7 +166,6 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   uint64_t copied = 0, c = 0;
   if (tid == 0)
     for (; copied < 2 && copied < total; copied++) copy_b(copied);
-  pass_start();
   pass_wait();
   uint64_t thr = tid & segmask;
   for (uint32_t x = tid >> P.L; x; x &= x - 1) thr |= 1ull << P.hi_pos[__ffs(x) - 1];
@@ -289,6 +288,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       __syncthreads();
     }
     if (failed) break;
+    if (t + gridDim.x >= ntiles) pass_start();
 #pragma unroll
     for (uint32_t i = 0; i < 8; i++)
       __stcs(reinterpret_cast<int4 *>(amps + (base | thr | s_trip[i])),

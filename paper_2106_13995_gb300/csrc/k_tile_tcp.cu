@@ -246,6 +246,8 @@ __device__ __forceinline__ bool tcp_block(const TcpTable &T, int i, uint32_t ts,
   return true;
 }
 
+// EARLY: a programmatic launch (sv_device.cuh)
+template <bool EARLY>
 __global__ void __launch_bounds__(kPThreads, 1)
     k_tile_tcp(const __grid_constant__ TilePass P, const __grid_constant__ TcpTable T) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -303,6 +305,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   const uint32_t ts = sbase + (uint32_t)g * kPTileBytes;
   const uint32_t lthr = G.tid * 2;
   const TcpAddr A{(lthr & segmask) | spread_hi(P, lthr & ~segmask), s_trip};
+  if constexpr (EARLY) pass_wait();
   bool failed = false;
   uint64_t cur = t < ntiles ? tile_base(P, t) : 0;
   for (; t < ntiles && !failed; t += stride) {
@@ -333,6 +336,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
       failed = true;
       break;
     }
+    if constexpr (EARLY)
+      if (t + stride >= ntiles) pass_start();   // the group's last tile
     int4 *o0 = reinterpret_cast<int4 *>(P.v0);
 #pragma unroll
     for (uint32_t i = 0; i < kPUnits; i++)
@@ -501,14 +506,23 @@ bool tcp_pass_ok(const TilePass &p, const HostPass &host) {
 
 sv_status launch_tile_tcp(sv_state *s, const TilePass &p, const HostPass &host, cudaStream_t stream) {
   if (!tcp_pass_ok(p, host)) return set_error(SV_EINVAL, "internal: not a pure tensor-core tile pass");
-  SV_TRY(func_attr_once((const void *)k_tile_tcp, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                        (int)tcp_smem_bytes(kTcpMaxBlocks)));
+  for (const void *fn : {(const void *)k_tile_tcp<false>, (const void *)k_tile_tcp<true>})
+    SV_TRY(func_attr_once(fn, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcp_smem_bytes(kTcpMaxBlocks)));
   const uint64_t ntiles = 1ull << (p.n - p.m);
   const uint64_t per_cta = (uint64_t)kPGroups;
   const int grid = (int)std::min<uint64_t>((ntiles + per_cta - 1) / per_cta, (uint64_t)s->sm_count);
   TcpTable tab;
   tcp_build_table(p, host, tab);
-  k_tile_tcp<<<grid, kPThreads, tcp_smem_bytes(p.nops), stream>>>(p, tab);
+  // programmatic launches up to four tiles a group: grid circuits of 15 qubits
+  // 76 us to 54, 21 qubits 202 to 166, 23 qubits 710 to 650; where the passes
+  // are long they disturb the groups' rhythm (26 qubits 5.4 ms to 5.6, 30 qubits
+  // 108 to 122)
+  if (ntiles <= 4 * per_cta * (uint64_t)s->sm_count) {
+    SV_CUDA(launch_early(k_tile_tcp<true>, dim3((unsigned)grid), kPThreads, tcp_smem_bytes(p.nops), stream, p, tab));
+    g_launches++;
+    return SV_OK;
+  }
+  k_tile_tcp<false><<<grid, kPThreads, tcp_smem_bytes(p.nops), stream>>>(p, tab);
   g_launches++;
   SV_CUDA(cudaGetLastError());
   return SV_OK;

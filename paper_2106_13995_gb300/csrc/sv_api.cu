@@ -1096,7 +1096,7 @@ int64_t sv_program_cache_limit(int64_t max_programs) {
 }
 
 size_t sv_workspace_bytes(int n, sv_dtype dt) {
-  if (n < 1 || n > 34 || (dt != SV_C64 && dt != SV_C128)) return 0;
+  if (n < 1 || n > 34) return 0;
   return moves_off(n) + moves_bytes(n, dt);
 }
 

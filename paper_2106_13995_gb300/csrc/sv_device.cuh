@@ -89,12 +89,16 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(smem)), "l"(gmem)
                : "memory");
 }
-// Programmatic launches (launch_early): a pass lets the next one's CTAs start as
-// soon as all of its own run, and waits for the pass before it to be complete
-// before it touches amplitudes.  What a launch costs on the way (the time from
-// one pass's end to the next one's start, and the next one's set-up) then passes
-// while the last one works: 20 layers of U3 + CZ in complex128, 12 qubits 481 us
-// to 421, 16 qubits 424 to 383; a gradient step of 16 qubits 522 to 466.
+// Programmatic launches (launch_early): a pass lets the next one's CTAs start once
+// all of its own have called pass_start, and waits for the pass before it to be
+// complete before it touches amplitudes.  What a launch costs on the way (the time
+// from one pass's end to the next one's start, and the next one's set-up) then
+// passes while the last one works: 20 layers of U3 + CZ in complex128, 12 qubits
+// 481 us to 420, 16 qubits 424 to 377; 40 layers in complex64, 18 qubits 366 to
+// 314; a gradient step of 16 qubits 522 to 462.  Tile passes call pass_start
+// before their stores: the next pass's CTAs then take the SMs as these leave them
+// (called first thing, 18 qubits took 436 us).  Passes of sites call it first and
+// read their matrices meanwhile (462 us against 471).
 __device__ __forceinline__ void pass_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
