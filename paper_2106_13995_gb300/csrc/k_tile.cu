@@ -111,6 +111,11 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
   const C *pmats = P.pmats ? reinterpret_cast<const C *>(P.pmats) + (size_t)b * P.pmats_stride : nullptr;
   double *acc = P.acc ? P.acc + (size_t)b * P.acc_stride : nullptr;
 
+  if constexpr (!COH && !INL && sizeof(R) == 4)
+    if (P.flags & kPassShift) {
+      __syncthreads();
+      shift_energy(v0, v1, TS, acc + P.mat0);
+    }
   for (int oi = 0; oi < P.nops; oi++) {
     __syncthreads();
     TileOp op;
@@ -181,14 +186,16 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
         for (uint32_t l = threadIdx.x; l < TS; l += blockDim.x) v1[l] = czero<C>();
         break;
       case TOP_DOT: {
-        R part = 0, norm = 0;
+        R part = 0, norm = 0, im = 0;
         for (uint32_t l = threadIdx.x; l < TS; l += blockDim.x) {
           const C a = v0[l], c = v1[l];   // same slot in both vectors: the swizzle cancels
           part += a.x * c.x + a.y * c.y;
           norm += a.x * a.x + a.y * a.y;
+          im += a.x * c.y - a.y * c.x;
         }
         block_acc<R>(part, acc + op.mat);
         block_acc<R>(norm, acc + op.mat + 1);
+        block_acc<R>(im, acc + op.mat + 2);
         break;
       }
       default:

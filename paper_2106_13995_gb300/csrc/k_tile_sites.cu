@@ -201,6 +201,10 @@ __global__ void __launch_bounds__(kSitesThreads, 3) k_tile_sites(const __grid_co
     }
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
+  if (TWO && (P.flags & kPassShift)) {
+    __syncthreads();
+    shift_energy(reinterpret_cast<const float2 *>(smem_raw), reinterpret_cast<float2 *>(smem_raw) + TS, TS, acc + P.mat0);
+  }
   for (int oi = 0; oi < P.nops; oi++) {
     __syncthreads();
     if (TWO && oi > 0) flush_probes(ent + (uint32_t)(oi - 1) * kSitesEntry, red[(oi - 1) & 1], acc);

@@ -35,7 +35,7 @@ struct AdjointProgram {
   bool sites = false;
   std::vector<AdjSite> fwd_sites, rev_sites;
   std::vector<int> rev_slot, rev_comps;
-  int n_acc = 0;                 // accumulators, the energy's and the norm's excluded
+  int n_acc = 0;                 // accumulators, TOP_DOT's three excluded
   int n_mats = 0;                // per-batch 2 x 2 matrices
 };
 
@@ -219,7 +219,12 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     b.site_mat = rev_mat.data();
     b.site_slot = A.rev_slot.data();
     b.site_comps = A.rev_comps.data();
+    const size_t first = A.prog.passes.size();
     append_passes(A.prog, A.op0s, split_sites(passes), b, rev_off, st);
+    if (sites && st == SV_OK && A.prog.passes.size() > first) {
+      A.prog.passes[first].flags |= kPassShift;
+      A.prog.passes[first].mat0 = (uint32_t)A.n_acc;
+    }
   }
   return st;
 }
@@ -384,7 +389,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
                        {tbl.data(), tbl.size() * sizeof(void *)},
                        {pm.data(), pm.size()}},
                       {L.ops_off, L.mats_off, L.coeffs_off, L.tbl_off, L.pmats_off}, L.end));
-  const size_t acc_stride = (size_t)A.n_acc + 2;
+  const size_t acc_stride = (size_t)A.n_acc + 3;
   const size_t acc_bytes = acc_stride * B * sizeof(double);
   if (acc_bytes > red_bytes(s->n)) return set_error(SV_ENOMEM, "workspace too small for the gradient batch");
   double *acc = reinterpret_cast<double *>(s->ws + kWsRed);

@@ -51,7 +51,7 @@ enum TileOpKind : uint8_t {
   TOP_GRAD = 2,      // acc[slot] += Im <v1 | G v0>, G = X/Y/Z/P1(-2) on one local target
   TOP_PAULI = 3,     // v1[l ^ xm] += c * phase * (-1)^{popcount(l & zm)} v0[l]
   TOP_ZERO = 4,      // v1 <- 0
-  TOP_DOT = 5,       // acc[mat] += Re <v0 | v1>, acc[mat + 1] += <v0 | v0>
+  TOP_DOT = 5,       // acc[mat] += Re <v0 | v1>, acc[mat + 1] += <v0 | v0>, acc[mat + 2] += Im <v0 | v1>
   TOP_TC = 6,        // 5-qubit dense block on the tensor cores (12-qubit tiles)
   TOP_PERM = 7,      // permutation block (k = 1..3): member y moves to member perm[y]; controls as TOP_DENSE
   TOP_GRADU = 8,     // TOP_GRAD then the 1-qubit matrix (per-batch pool) on both vectors, in one sweep
@@ -145,6 +145,9 @@ constexpr uint32_t kPassOz = 0x1000;
 // amplitudes (qubits hi_pos[0..m)); mat0: 16-byte index of its MoveDesc
 // (k_moves.cu)
 constexpr uint32_t kPassMoves = 0x2000;
+// TilePass.flags: v1 -= e v0 first, e = <v0 | v1> / <v0 | v0> from the accumulators
+// mat0 to mat0 + 2 (a gradient's first reverse pass, complex64)
+constexpr uint32_t kPassShift = 0x8000;
 // TilePass.flags: the state, a known basis state, through one single-qubit gate
 // per qubit, written as the product it is; mat0: 16-byte index of 2 x 2
 // complex128 matrices of the n qubits (host copy; k_moves.cu)

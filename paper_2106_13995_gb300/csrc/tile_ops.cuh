@@ -532,6 +532,24 @@ __device__ __forceinline__ void block_acc(R part, double *dst) {
   if ((threadIdx.x & 31) == 0) atomicAdd(dst, (double)part);
 }
 
+// lambda <- lambda - e psi with e = <psi | lambda> / <psi | psi> (acc[0] + i acc[2]
+// over acc[1]): it changes no gradient, Im <psi | G | psi> being 0 and Im e, 0
+// but for rounding, an error of every probe.  What is left, (H - E) psi, rounds
+// in FP32 by the energy's spread instead of the energy: near a basis state, whose
+// one large amplitude carries most of lambda, the phase that hundreds of
+// roundings turned it by was most of the gradient's error.
+__device__ __forceinline__ void shift_energy(const float2 *v0, float2 *v1, uint32_t n, const double *acc) {
+  const double norm = acc[1];
+  const float e = norm > 0 ? (float)(acc[0] / norm) : 0.f, o = norm > 0 ? (float)(acc[2] / norm) : 0.f;
+  for (uint32_t l = threadIdx.x; l < n; l += blockDim.x) {
+    const float2 a = v0[l];   // same slot in both vectors
+    float2 c = v1[l];
+    c.x = fmaf(-e, a.x, fmaf(o, a.y, c.x));
+    c.y = fmaf(-e, a.y, fmaf(-o, a.x, c.y));
+    v1[l] = c;
+  }
+}
+
 template <typename R>
 __device__ void grad_op(const typename Cx<R>::T *__restrict__ psi,
                         const typename Cx<R>::T *__restrict__ lam, int m, const TileOp &op,
