@@ -96,6 +96,8 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   r.moves = s->n >= kMovesMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
             r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE &&
             s->ws_bytes >= moves_off(s->n) + moves_bytes(s->n, s->dt);
+  r.small = r.prec == SV_PREC_PLAIN && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
+            r.tile_m < std::min(plain64 ? 13 : 12, s->n);
   r.L = std::min(r.L, r.tile_m);
   if (s->dt == SV_C64 && r.L < 1) r.L = 1;
   return r;
@@ -1027,6 +1029,26 @@ sv_status upload_program(sv_state *s, const CachedProgram &cp) {
   return SV_OK;
 }
 
+// The next plan to try for a program that outgrows the program area: without
+// exact tensor-core passes (56 KB a block), without permutation runs, with the
+// tiles and fusion width of large states (more gates meet in a larger tile's
+// tables and blocks).  False: there is none.
+static bool leaner(const sv_state *s, Opts &o) {
+  if (o.oz) {
+    o.oz = 0;
+  } else if (o.moves) {
+    o.moves = o.product = 0;
+  } else if (o.small) {
+    o.small = 0;
+    o.fusion_k = 3;
+    o.tile_m = std::min(s->dt == SV_C64 ? 13 : 12, s->n);
+    o.L = std::min(3, o.tile_m);
+  } else {
+    return false;
+  }
+  return true;
+}
+
 sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,
                       ProgramRef *out, Opts *o_out, bool basis) {
   if (!s) return set_error(SV_EINVAL, "null state");
@@ -1055,6 +1077,10 @@ sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, co
     SV_TRY(circuit_to_gates(c, params, s->n, gates, false));
     auto built = std::make_shared<CachedProgram>();
     SV_TRY(build_circuit_program(s, gates, o, *built));
+    for (Opts p = o; built->lay.end > kWsProgBytes && leaner(s, p);) {
+      built = std::make_shared<CachedProgram>();
+      SV_TRY(build_circuit_program(s, gates, p, *built));
+    }
     built->serial = next_program_serial();
     cp = g_cache.insert(s, k, h, std::move(built));
   }

@@ -77,7 +77,7 @@ void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt
   tune_load_locked();
   auto it = g_tune.find(tune_key(s->n, s->dt, c));
   if (it == g_tune.end() || it->second.first == 0) return;   // not tuned, or the defaults were fastest
-  o.oz = o.moves = 0;   // the pair was timed on the CUDA cores' tile passes
+  o.oz = o.moves = o.small = 0;   // the pair was timed on the CUDA cores' tile passes
   if (want_k) o.fusion_k = it->second.first;
   if (want_m) o.tile_m = std::min(it->second.second, s->n);
 }

@@ -382,6 +382,7 @@ struct Opts {   // all int: hashed as key bytes, so no padding
   int oz = 0;   // complex128: blocks of 5 qubits on the tensor cores where they all qualify
   int moves = 0;   // runs of permutation gates as moves (k_moves.cu)
   int product = 0;   // the state is a known basis state when the program runs
+  int small = 0;   // default tiles and fusion width of a small state
 };
 constexpr int kSmall128 = 17;   // widest complex128 state with the small-state plan
 Opts resolve(const sv_state *s, const sv_options *o, int nvec);

@@ -1,0 +1,31 @@
+// Programs as the library builds them, on a host-only state (test only).
+#include <cstring>
+
+#include "../../paper_2106_13995_gb300/csrc/sv_internal.h"
+
+using namespace sv;
+
+static sv_state host_state(int n, int dt) {
+  sv_state s;
+  s.n = n;
+  s.dt = (sv_dtype)dt;
+  s.ws_bytes = sv_workspace_bytes(n, (sv_dtype)dt);
+  return s;
+}
+
+// Build a circuit's program: returns the status, *end the bytes of the program
+// area it takes, flags[0 .. *n_passes) each pass's flags (at most cap).
+extern "C" int program_build(const sv_circuit *c, int dt, const sv_options *opt, uint64_t *end, uint32_t *flags, int cap,
+                             int *n_passes) {
+  sv_state s = host_state(c->n_qubits, dt);
+  ProgramRef cp;
+  Opts o;
+  const sv_status st = get_program(&s, c, nullptr, opt, &cp, &o);
+  if (st != SV_OK) return (int)st;
+  *end = cp->lay.end;
+  *n_passes = (int)cp->prog.passes.size();
+  for (int i = 0; i < *n_passes && i < cap; i++) flags[i] = cp->prog.passes[i].flags;
+  return SV_OK;
+}
+
+extern "C" uint64_t program_area() { return kWsProgBytes; }
