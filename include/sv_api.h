@@ -68,12 +68,17 @@ typedef enum { SV_C64 = 0, SV_C128 = 1 } sv_dtype;
  * kernel; blocks with controls stay on the CUDA cores.  Split-TF32 applies
  * dense 4- and 5-qubit blocks on the tensor cores (a 4-qubit block padded
  * with an idle qubit), as passes of their own unless tile_m is 12.
- * complex128 states always use FP64 arithmetic whatever the mode.  Their
- * circuits of uncontrolled blocks run on the tensor cores from 14 qubits on
- * where options are left at 0 (SV_PREC_PLAIN): products of exact integer
- * digits of the FP64 numbers, joined and rounded to FP64 once per block.  The
- * digits are relative to the largest number a block mixes: an amplitude
- * keeps an absolute error below 2^-57 of it. */
+ * complex128 states keep FP64 accuracy whatever the mode, by FP64 arithmetic
+ * or, from 14 qubits on with options left at 0 (SV_PREC_PLAIN), on the tensor
+ * cores: products of exact integer digits of the FP64 numbers, joined and
+ * rounded to FP64 once per fused block.  The digits are relative to the largest
+ * of the amplitudes that a block's gates mix with one another, and a circuit
+ * takes this path only where each of its blocks (no controls beyond 5 qubits)
+ * mixes all of those by factors within 2^6 of its largest.  Every amplitude
+ * then keeps what FP64 arithmetic gives it: one rounding of the result, and an
+ * error of about 2^-53 of the magnitudes added up in it, also beside amplitudes
+ * many orders larger.  Other circuits (rotations by small angles, say) take
+ * FP64 arithmetic throughout. */
 typedef enum {
   SV_PREC_PLAIN = 0,       /* FP32 FMA on CUDA cores */
   SV_PREC_TC_BF16X3 = 1,   /* tensor cores, split-BF16 (3 products), FP32 accumulate */

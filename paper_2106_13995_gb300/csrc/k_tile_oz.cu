@@ -5,14 +5,14 @@
 // block needs 32 of them per amplitude.  Here a block is the GEMM of K9 (M =
 // 128 groups, N = K = 64, the real embedding of U) on digits: every FP64
 // number becomes seven signed 9-bit integers (oz_digits.cuh) relative to the
-// largest number of its group, the 28 products of digits i, j with i + j <= 6
+// largest number of its group's part (oz_parts), the 28 products of digits i, j with i + j <= 6
 // run as FP16 MMAs whose FP32 sums are exact integers, and the seven sums per
 // result are joined in 64-bit integers and rounded to FP64 once.  No FP64
 // arithmetic is left but one integer conversion per number.
 //
 // One persistent CTA per SM: 512 threads, four to a row (TMEM lane).  Per
 // block: every thread gathers 8 amplitudes of its row from the tile in shared
-// memory, finds the row's exponent with the row's other threads, and stores
+// memory, finds the parts' exponents with the row's other threads, and stores
 // the digits as FP16 A operands in TMEM (224 columns); one thread issues the
 // MMAs of the first 32 result columns (7 x 32 TMEM columns of sums); the
 // threads read those sums, the MMAs of the other 32 columns start, and the
@@ -26,8 +26,9 @@
 //
 // Bound (21 qubits, 9.3 us per tile and block): the chain gather - digits - MMA
 // - join of one tile; without the join 0.28 less, with a seventh of the MMAs
-// 0.13 less.  A 23-qubit grid circuit of 20 cycles: 27.2 ms in FP64 arithmetic,
-// 4.4 ms here.
+// 0.13 less.  A 23-qubit grid circuit of 20 cycles: 24.1 ms in FP64 arithmetic,
+// 4.5 ms here (4.3 with one exponent for all of a row, which lost the low bits of
+// small amplitudes next to large ones that their block does not mix).
 //
 // Every wait is bounded, as in K9.
 #include <algorithm>
@@ -46,7 +47,10 @@ constexpr int kOzThreads = 512;
 constexpr uint32_t kOzTileBytes = (1u << kTcTileM) * 16;     // 64 KB
 constexpr uint32_t kOzBRows = kOzDigits * 64;                 // of B: half of the columns, digit, 32 columns
 constexpr uint32_t kOzBBytes = kOzBRows * 64 * 2;             // 56 KB
-constexpr uint32_t kOzSmB = kOzTileBytes, kOzSmExp = kOzSmB + 2 * kOzBBytes, kOzSmBar = kOzSmExp + 4 * 128 * 4;
+// largest high words of the members (or of the threads' shares) and exponents
+// of the parts, 32 x 128 each
+constexpr uint32_t kOzSmB = kOzTileBytes, kOzSmHi = kOzSmB + 2 * kOzBBytes, kOzSmExp = kOzSmHi + 32 * 128 * 4;
+constexpr uint32_t kOzSmBar = kOzSmExp + 32 * 128 * 4;
 constexpr uint32_t kOzSmem = kOzSmBar + 8 * 3 + 8;
 static_assert(kOzSmem <= 227u * 1024u, "shared memory of a CTA");
 constexpr uint32_t kOzTmemCols = 512, kOzTmemD = kOzDigits * 32;   // A digits, then the sums
@@ -60,7 +64,13 @@ struct OzTable {
   uint32_t rbit[kOzMaxBlocks][7];
   int32_t eu[kOzMaxBlocks];
   uint32_t mat[kOzMaxBlocks];   // 16-byte index of the packed operand in the pool
+  // parts of the block: their number, each one's input members as a mask, and
+  // the part of every input and output member
+  uint32_t nparts[kOzMaxBlocks];
+  uint32_t mask[kOzMaxBlocks][32];
+  uint8_t in[kOzMaxBlocks][32], out[kOzMaxBlocks][32];
 };
+static_assert(kOzBBytes == kOzOperandBytes, "operand size");
 
 // byte offset of tile amplitude l (linear over GF(2)); see tcp_row_positions
 // for how lanes are kept apart
@@ -126,7 +136,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   const uint32_t sbase = smem_u32(smem);
   const uint32_t bar_mma = sbase + kOzSmBar, bar_b = bar_mma + 8;
   uint32_t *slot = reinterpret_cast<uint32_t *>(smem + kOzSmBar + 24);
-  uint32_t *sexp = reinterpret_cast<uint32_t *>(smem + kOzSmExp);
+  uint32_t *shi = reinterpret_cast<uint32_t *>(smem + kOzSmHi), *sexp = reinterpret_cast<uint32_t *>(smem + kOzSmExp);
   const uint32_t tid = threadIdx.x, row = tid & 127u, g = tid >> 7;
   const int nb = P.nops;
   const uint32_t segmask = (1u << P.L) - 1;
@@ -194,23 +204,40 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       uint32_t s0 = 0;
 #pragma unroll
       for (int b = 0; b < 7; b++) s0 ^= ((row >> b) & 1u) ? T.rbit[bi][b] : 0u;
-      // gather, and the row's exponent
+      // gather, and the exponents of the row's parts
       double2 x[8];
-      uint32_t E = 0;   // largest high word without its sign
+      uint32_t hi[8];   // largest high word without its sign
 #pragma unroll
       for (int j = 0; j < 8; j++) {
         x[j] = *reinterpret_cast<const double2 *>(smem + (s0 ^ T.soff[bi][8 * g + j]));
-        E = max(E, max((uint32_t)__double2hiint(x[j].x) & 0x7fffffffu, (uint32_t)__double2hiint(x[j].y) & 0x7fffffffu));
+        hi[j] = max((uint32_t)__double2hiint(x[j].x) & 0x7fffffffu, (uint32_t)__double2hiint(x[j].y) & 0x7fffffffu);
       }
-      sexp[g * 128 + row] = E;
-      __syncthreads();
-      E = oz_exponent(max(max(sexp[row], sexp[128 + row]), max(sexp[256 + row], sexp[384 + row])));
+      const uint32_t np = T.nparts[bi];
+      uint32_t E = 0;   // of the row, where the block is one part
+      if (np == 1) {
+#pragma unroll
+        for (int j = 0; j < 8; j++) E = max(E, hi[j]);
+        shi[g * 128 + row] = E;
+        __syncthreads();
+        E = oz_exponent(max(max(shi[row], shi[128 + row]), max(shi[256 + row], shi[384 + row])));
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; j++) shi[(8 * g + j) * 128 + row] = hi[j];
+        __syncthreads();
+        for (uint32_t p = g; p < np; p += 4) {
+          uint32_t e = 0;
+          for (uint32_t m = T.mask[bi][p]; m; m &= m - 1) e = max(e, shi[(__ffs(m) - 1) * 128 + row]);
+          sexp[p * 128 + row] = oz_exponent(e);
+        }
+        __syncthreads();
+      }
       // digits: fields of (re, im) side by side as FP16 1024 + field, less 1280
       uint64_t wr[8], wi[8];
 #pragma unroll
       for (int j = 0; j < 8; j++) {
-        wr[j] = oz_fields((uint32_t)__double2hiint(x[j].x), (uint32_t)__double2loint(x[j].x), E);
-        wi[j] = oz_fields((uint32_t)__double2hiint(x[j].y), (uint32_t)__double2loint(x[j].y), E);
+        const uint32_t e = np == 1 ? E : sexp[T.in[bi][8 * g + j] * 128 + row];
+        wr[j] = oz_fields((uint32_t)__double2hiint(x[j].x), (uint32_t)__double2loint(x[j].x), e);
+        wi[j] = oz_fields((uint32_t)__double2hiint(x[j].y), (uint32_t)__double2loint(x[j].y), e);
       }
 #pragma unroll
       for (int i = 0; i < kOzDigits; i++) {
@@ -244,8 +271,6 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       }
       // (if the operand never landed nothing was committed, and the wait below
       // runs out)
-      const int k = (int)E + T.eu[bi] - 1081;
-      const bool bad = E == 0x7ffu;
 #pragma unroll
       for (int h = 0; h < 2; h++) {
         ok = ok && mbar_wait(bar_mma, phase, kOzSpin);
@@ -275,6 +300,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         for (int j = 0; j < 4; j++) {
           double2 o;
           uint32_t v[kOzDigits];
+          const uint32_t e = np == 1 ? E : sexp[T.out[bi][16 * h + 4 * g + j] * 128 + row];
+          const int k = (int)e + T.eu[bi] - 1081;
+          const bool bad = e == 0x7ffu;
 #pragma unroll
           for (int s = 0; s < kOzDigits; s++) v[s] = r[s][2 * j];
           o.x = oz_join(v, k, bad);
@@ -393,6 +421,54 @@ static bool oz_pack_digits(const std::vector<cd> &U, std::vector<uint16_t> &out,
   return true;
 }
 
+// The parts of a block: inputs and outputs that its gates connect (mag: the
+// product of the gates' entry magnitudes), labelled 0, 1, ...; in[y] and out[y]
+// are the labels of member y.  A control, an idle or padding qubit, a diagonal
+// or a permuted one splits the members, and digits are relative to the largest
+// number of a part.  FP64 arithmetic leaves a result within rounding of
+// sum_y mag[r][y] |x_y|; the digits add about 2^-60 of the powers of two above
+// the part's largest number and above the matrix's entries (2^eu).  So a block
+// qualifies where every entry of mag within a part is at least 2^-6 2^eu: the
+// digits' share is then at most about one FP64 rounding of that sum, whatever
+// the amplitudes are.  Others (a rotation by a small angle next to a large
+// amplitude) keep FP64 arithmetic.
+bool oz_parts(const std::vector<double> &mag, int eu, uint8_t *in, uint8_t *out) {
+  double least = HUGE_VAL;
+  int root[64];   // inputs 0..31, outputs 32..63
+  for (int x = 0; x < 64; x++) root[x] = x;
+  auto find = [&](int x) {
+    while (root[x] != x) x = root[x] = root[root[x]];
+    return x;
+  };
+  int entries = 0;
+  for (int r = 0; r < 32; r++)
+    for (int y = 0; y < 32; y++) {
+      const double m = mag[(size_t)r * 32 + y];
+      if (m == 0) continue;
+      if (!(m > 0)) return false;
+      least = std::min(least, m);
+      entries++;
+      root[find(32 + r)] = find(y);
+    }
+  if (!(least >= std::ldexp(1.0, eu - 6))) return false;
+  int label[64], n = 0, ins[32] = {}, outs[32] = {};
+  std::fill(label, label + 64, -1);
+  for (int y = 0; y < 32; y++) {
+    const int f = find(y);
+    if (label[f] < 0) label[f] = n++;
+    in[y] = (uint8_t)label[f];
+    ins[in[y]]++;
+  }
+  for (int r = 0; r < 32; r++) {
+    const int f = find(32 + r);
+    if (label[f] < 0) return false;   // a row of zeros
+    out[r] = (uint8_t)label[f];
+    outs[out[r]]++;
+  }
+  for (int p = 0; p < n; p++) entries -= ins[p] * outs[p];
+  return entries == 0;   // every input of a part reaches every output of it
+}
+
 // Row bits of a block: the first three lane bits take tile positions of
 // different bank classes ({0,3,6,9}, {1,4,7,10}, {2,5,8,11}: 8 lanes of a
 // 16-byte access then reach 8 banks), the others follow in order.
@@ -429,6 +505,13 @@ sv_status launch_tile_oz(sv_state *s, const TilePass &p, const HostPass &host, c
     for (int b = 0; b < 7; b++) T.rbit[i][b] = oz_slot(1u << rows[b]);
     T.eu[i] = op.slot;
     T.mat[i] = op.mat;
+    const uint8_t *parts = host.mats + 16 * (size_t)op.mat + kOzOperandBytes;
+    for (int y = 0; y < 32; y++) {
+      T.in[i][y] = parts[y];
+      T.out[i][y] = parts[32 + y];
+      T.mask[i][parts[y]] |= 1u << y;
+      T.nparts[i] = std::max(T.nparts[i], parts[y] + 1u);
+    }
   }
   const uint64_t ntiles = 1ull << (p.n - p.m);
   const int grid = (int)std::min<uint64_t>(ntiles, (uint64_t)s->sm_count);

@@ -9,7 +9,9 @@
 // product splits into 7 x 7 digit products whose sums by weight i + j are
 // exact in the tensor cores' FP32 accumulators (the splitting of Ozaki, Ogita,
 // Oishi and Rump, Numerical Algorithms 59, 2012).  Weights i + j <= 6 are
-// kept: what is dropped lies 2^-58 below a result of the row's size.
+// kept.  What is dropped is at most 2^-60 of 2^e times the matrix's 2^e a term:
+// digits of random signs add up to about as much in a dot product, 64 terms of
+// one sign to 2^-54.
 #pragma once
 
 #include <stdint.h>

@@ -24,8 +24,9 @@ static int index_of(const std::vector<int> &v, int q) {
 
 // Embed a (controlled) gate on `targets`/`controls` into a dense matrix over
 // the qubit list `Q` (which contains all of them).
-static std::vector<cd> embed(const std::vector<cd> &U, const std::vector<int> &targets,
-                             const std::vector<int> &controls, const std::vector<int> &Q) {
+template <typename T>
+static std::vector<T> embed(const std::vector<T> &U, const std::vector<int> &targets,
+                            const std::vector<int> &controls, const std::vector<int> &Q) {
   const int kq = (int)Q.size();
   const int D = 1 << kq;
   const int d = 1 << (int)targets.size();
@@ -35,10 +36,10 @@ static std::vector<cd> embed(const std::vector<cd> &U, const std::vector<int> &t
   int tmask = 0, cmask = 0;
   for (int p : tpos) tmask |= 1 << p;
   for (int p : cpos) cmask |= 1 << p;
-  std::vector<cd> E((size_t)D * D, 0.0);
+  std::vector<T> E((size_t)D * D, T(0.0));
   for (int col = 0; col < D; col++) {
     if ((col & cmask) != cmask) {
-      E[(size_t)col * D + col] = 1.0;
+      E[(size_t)col * D + col] = T(1.0);
       continue;
     }
     int ct = 0;
@@ -52,12 +53,13 @@ static std::vector<cd> embed(const std::vector<cd> &U, const std::vector<int> &t
   return E;
 }
 
-static std::vector<cd> matmul(const std::vector<cd> &A, const std::vector<cd> &B, int D) {
-  std::vector<cd> C((size_t)D * D, 0.0);
+template <typename T>
+static std::vector<T> matmul(const std::vector<T> &A, const std::vector<T> &B, int D) {
+  std::vector<T> C((size_t)D * D, T(0.0));
   for (int i = 0; i < D; i++)
     for (int k = 0; k < D; k++) {
-      cd a = A[(size_t)i * D + k];
-      if (a == cd(0.0)) continue;
+      const T a = A[(size_t)i * D + k];
+      if (a == T(0.0)) continue;
       for (int j = 0; j < D; j++) C[(size_t)i * D + j] += a * B[(size_t)k * D + j];
     }
   return C;
@@ -71,7 +73,40 @@ static bool is_diagonal(const std::vector<cd> &U, int k) {
   return true;
 }
 
-std::vector<Block> fuse(const std::vector<Gate> &gates, int K) {
+static std::vector<double> magnitudes(const std::vector<cd> &U) {
+  std::vector<double> m(U.size());
+  for (size_t e = 0; e < U.size(); e++) m[e] = std::abs(U[e]);
+  return m;
+}
+
+// M over the qubits Q, multiplied from the left by a gate's entry magnitudes.
+static void gate_magnitudes(const Gate &g, const std::vector<int> &Q, std::vector<double> &M) {
+  const int D = 1 << (int)Q.size(), d = 1 << (int)g.targets.size();
+  int cmask = 0, off[64], tmask = 0;
+  for (int q : g.controls) cmask |= 1 << index_of(Q, q);
+  for (int y = 0; y < d; y++) {
+    off[y] = 0;
+    for (size_t j = 0; j < g.targets.size(); j++) off[y] |= ((y >> j) & 1) << index_of(Q, g.targets[j]);
+    tmask |= off[y];
+  }
+  double m[64 * 64], rows[64 * 64];
+  for (int e = 0; e < d * d; e++) m[e] = std::abs(g.U[e]);
+  for (int base = 0; base < D; base++) {
+    if ((base & tmask) || (base & cmask) != cmask) continue;
+    for (int y = 0; y < d; y++) std::copy_n(&M[(size_t)(base | off[y]) * D], D, rows + (size_t)y * D);
+    for (int r = 0; r < d; r++) {
+      double *to = &M[(size_t)(base | off[r]) * D];
+      std::fill(to, to + D, 0.0);
+      for (int y = 0; y < d; y++) {
+        const double a = m[r * d + y];
+        if (a == 0) continue;
+        for (int c = 0; c < D; c++) to[c] += a * rows[(size_t)y * D + c];
+      }
+    }
+  }
+}
+
+std::vector<Block> fuse(const std::vector<Gate> &gates, int K, bool mags) {
   std::vector<Block> blocks;
   blocks.reserve(gates.size());
   std::vector<int> last(64, -1);
@@ -89,9 +124,13 @@ std::vector<Block> fuse(const std::vector<Gate> &gates, int K) {
         if (index_of(uni, q) < 0) uni.push_back(q);
       if ((int)uni.size() <= K) {
         const int D = 1 << (int)uni.size();
-        std::vector<cd> Ub = embed(b.U, b.qubits, {}, uni);
-        std::vector<cd> Ug = embed(g.U, g.targets, g.controls, uni);
-        b.U = matmul(Ug, Ub, D);
+        const std::vector<cd> Ug = embed(g.U, g.targets, g.controls, uni);
+        if (uni.size() > b.qubits.size()) b.U = embed(b.U, b.qubits, {}, uni);
+        b.U = matmul(Ug, b.U, D);
+        if (mags) {
+          if (uni.size() > b.qubits.size()) b.mag = embed(b.mag, b.qubits, {}, uni);
+          gate_magnitudes(g, uni, b.mag);
+        }
         b.qubits = uni;
         // the block's older qubits may already have later blocks: keep those
         for (int q : uni) last[q] = std::max(last[q], bstar);
@@ -120,6 +159,7 @@ std::vector<Block> fuse(const std::vector<Gate> &gates, int K) {
       nb.qubits = Q;
       nb.U = embed(g.U, g.targets, g.controls, Q);
     }
+    if (mags) nb.mag = magnitudes(nb.U);
     blocks.push_back(std::move(nb));
     const int idx = (int)blocks.size() - 1;
     for (int q : Q) last[q] = idx;
@@ -239,6 +279,11 @@ std::vector<Block> merge_in_passes(std::vector<PassPlan> passes, int K) {
           const std::vector<cd> Ua = embed(A.U, A.qubits, {}, uni);
           const std::vector<cd> Ub = embed(ops[j].U, ops[j].qubits, {}, uni);
           A.U = matmul(Ub, Ua, D);   // ops[j] acts after ops[i]
+          if (!A.mag.empty()) {
+            const std::vector<double> Ma = embed(A.mag, A.qubits, {}, uni);
+            const std::vector<double> Mb = embed(ops[j].mag, ops[j].qubits, {}, uni);
+            A.mag = matmul(Mb, Ma, D);
+          }
           A.qubits = uni;
           A.diag = is_diagonal(A.U, (int)uni.size());
           alive[j] = 0;

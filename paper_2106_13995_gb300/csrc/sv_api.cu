@@ -85,12 +85,13 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   const bool default_m = !(o && o->tile_m > 0);
   r.tc_in_tile = r.prec != SV_PREC_PLAIN && (explicit12 || (r.prec == SV_PREC_TC_BF16X3 && default_m));
   // complex128 states of at least 14 qubits: 5-qubit blocks on the tensor
-  // cores, exactly (k_tile_oz), unless a fusion width or tile size is asked
-  // for (20 layers of U3 + CZ, against 7-qubit tiles of the CUDA cores: 14
-  // qubits 357 us against 569, 16 qubits 457 against 669; grid circuits of 17
-  // qubits 181 against 480, of 23 qubits 5.0 ms against 30).  Below, one or two
-  // SMs run all blocks in turn, and what preparing the operands adds to a
-  // circuit's first run (30 us a block) is more than its blocks save
+  // cores (k_tile_oz) where all of a circuit's qualify, unless a fusion width
+  // or tile size is asked for (grid circuits of 20 cycles, against the CUDA
+  // cores' best tiles: 14 qubits 57 us against 124, 16 qubits 122 against 231,
+  // 20 qubits of 12 cycles 323 against 1528, 23 qubits 4.5 ms against 24.1).
+  // Below, one or two SMs run all blocks in turn, and what preparing the
+  // operands adds to a circuit's first run (30 us a block) is more than its
+  // blocks save
   r.oz = s->dt == SV_C128 && s->n >= kOzMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
          r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE;
   r.moves = s->n >= kMovesMinQubits && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
@@ -691,11 +692,15 @@ static void pad_in_tile(Block &blk, const std::vector<int> &S) {
     if (p >= (int)S.size()) continue;
     if (std::find(blk.qubits.begin(), blk.qubits.end(), S[p]) == blk.qubits.end()) blk.qubits.push_back(S[p]);
   }
-  std::vector<cd> U5(32 * 32, 0.0);
-  for (int r = 0; r < 32; r++)
-    for (int c = 0; c < 32; c++)
-      if ((r >> k) == (c >> k)) U5[(size_t)r * 32 + c] = blk.U[(size_t)(r & (d - 1)) * d + (c & (d - 1))];
-  blk.U = std::move(U5);
+  auto pad = [&](auto &U) {
+    std::decay_t<decltype(U)> U5(32 * 32, 0.0);
+    for (int r = 0; r < 32; r++)
+      for (int c = 0; c < 32; c++)
+        if ((r >> k) == (c >> k)) U5[(size_t)r * 32 + c] = U[(size_t)(r & (d - 1)) * d + (c & (d - 1))];
+    U = std::move(U5);
+  };
+  pad(blk.U);
+  if (!blk.mag.empty()) pad(blk.mag);
   blk.diag = false;
 }
 
@@ -726,12 +731,12 @@ static void move_to_end(std::vector<Block> &from, std::vector<Block> &to) {
 
 // Append a complex128 program of exact tensor-core passes, if every fused block of at
 // most 5 qubits qualifies: uncontrolled (wider or controlled ones stay on the
-// CUDA cores, and a program is all of one kind), digits within the exact range,
-// not all of them permutations (those move amplitudes in table passes), and the
+// CUDA cores, and a program is all of one kind), digits within the exact range
+// and as good as FP64 for every amplitude (oz_parts), not all of them permutations (those move amplitudes in table passes), and the
 // operands fit the program area.  False leaves `out` as it was.
 static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
   const int n = s->n, m = kTcTileM, L = o.L;
-  std::vector<Block> blocks = fuse(gates, 5);
+  std::vector<Block> blocks = fuse(gates, 5, true);
   if (m < n) {
     std::vector<PassPlan> first = plan_passes(blocks, n, m, L, kOzMaxBlocks, kMaxMatPerPass);
     if (first.empty()) return false;
@@ -745,7 +750,7 @@ static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates,
     moves = moves && permutation_of(b.U, (int)b.qubits.size(), perm);
     b.kind = TOP_TC;
   }
-  if (moves || out.prog.mats.size() + blocks.size() * kOzDigits * 64 * 64 * 2 + (64 << 10) > kWsProgBytes) return false;
+  if (moves || out.prog.mats.size() + blocks.size() * kOzBlockBytes + (64 << 10) > kWsProgBytes) return false;
   std::vector<PassPlan> passes = plan_passes(blocks, n, m, L, kOzMaxBlocks, kOzMaxBlocks * 1024 + 1023);
   if (passes.empty()) return false;
   CachedProgram prog;
@@ -776,11 +781,14 @@ static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates,
       for (int j = 0; j < 5; j++) op.t[j] = (uint8_t)loc[b.qubits[j]];
       std::vector<uint16_t> packed;
       int eu = 0;
-      if (!oz_pack_matrix(b.U, packed, eu) || eu < -1000 || eu > 1000) return false;
+      uint8_t parts[64];
+      if (!oz_pack_matrix(b.U, packed, eu) || eu < -1000 || eu > 1000 || !oz_parts(b.mag, eu, parts, parts + 32))
+        return false;
       op.slot = (int16_t)eu;
       op.mat = (uint32_t)(prog.prog.mats.size() / 16);
       const uint8_t *q = reinterpret_cast<const uint8_t *>(packed.data());
       prog.prog.mats.insert(prog.prog.mats.end(), q, q + packed.size() * 2);
+      prog.prog.mats.insert(prog.prog.mats.end(), parts, parts + 64);
       prog.prog.ops.push_back(op);
     }
     prog.prog.passes.push_back(tp);

@@ -214,6 +214,7 @@ struct Block {
   std::vector<int> qubits;     // targets (matrix bit order)
   std::vector<int> controls;   // remaining controls (unfused controlled gates)
   std::vector<cd> U;
+  std::vector<double> mag;     // product of the gates' entry magnitudes (where fuse() was asked for it)
   bool diag = false;
   bool fusable = true;
   int param = -1;              // parametric single gate (batched / gradient)
@@ -248,7 +249,8 @@ bool unitarity_checks();
 double unitarity_error(const std::vector<cd> &U, int k);
 
 // planner.cpp
-std::vector<Block> fuse(const std::vector<Gate> &gates, int fusion_k);
+// mags: blocks also carry the product of their gates' entry magnitudes
+std::vector<Block> fuse(const std::vector<Gate> &gates, int fusion_k, bool mags = false);
 struct PassPlan {
   std::vector<int> S;          // tile qubits: S[0..L) = 0..L-1, then sorted high qubits
   std::vector<Block> ops;
@@ -607,7 +609,10 @@ std::string tcp_layout_selftest(const TilePass &p, const HostPass &host, int *pa
 // exact tensor-core passes of complex128 states (k_tile_oz.cu)
 constexpr int kOzMaxBlocks = 12;
 constexpr int kOzMinQubits = 14;
+constexpr size_t kOzOperandBytes = 7 * 64 * 64 * 2;   // FP16 digits of a block's matrix; 32 + 32 part labels follow
+constexpr size_t kOzBlockBytes = kOzOperandBytes + 64;
 bool oz_pack_matrix(const std::vector<cd> &U, std::vector<uint16_t> &out, int &eu);
+bool oz_parts(const std::vector<double> &mag, int eu, uint8_t *in, uint8_t *out);
 sv_status launch_tile_oz(sv_state *s, const TilePass &p, const HostPass &host, cudaStream_t stream);
 // tensor-core 5-qubit block (k_tc.cu)
 size_t tc_matrix_words(sv_prec mode, int k);
