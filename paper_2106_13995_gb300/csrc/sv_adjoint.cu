@@ -33,6 +33,8 @@ struct AdjointProgram {
   // reverse site's first accumulator and components (bits: X, Y, Z);
   // without them one matrix per instance and one accumulator per parameter
   bool sites = false;
+  bool split = false;            // some pass of sites was cut at other ops
+  int folded = 0;                // gates that sites take: 4 per parametric gate, 3 per permutation
   std::vector<AdjSite> fwd_sites, rev_sites;
   std::vector<int> rev_slot, rev_comps;
   int n_acc = 0;                 // accumulators, TOP_DOT's three excluded
@@ -72,7 +74,7 @@ void drop_adjoint_programs(const sv_state *s) {
 
 // Passes of TOP_SITES ops have a kernel of their own: split a pass where it
 // changes between them and other ops, and beyond the kernel's op count.
-static std::vector<PassPlan> split_sites(const std::vector<PassPlan> &passes) {
+static std::vector<PassPlan> split_sites(const std::vector<PassPlan> &passes, bool &split) {
   std::vector<PassPlan> out;
   for (const PassPlan &P : passes) {
     size_t i = 0;
@@ -83,6 +85,7 @@ static std::vector<PassPlan> split_sites(const std::vector<PassPlan> &passes) {
       while (i < P.ops.size() && (P.ops[i].kind == TOP_SITES) == sites &&
              (!sites || Q.ops.size() < (size_t)kMaxSitesOps))
         Q.ops.push_back(P.ops[i++]);
+      split = split || (i < P.ops.size() && (P.ops[i].kind == TOP_SITES) != sites);
       out.push_back(std::move(Q));
     } while (i < P.ops.size());
   }
@@ -113,6 +116,10 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     A.inst_gate.push_back(g.param_gate);
   }
   const int G = (int)gates.size();
+  int perm[64];
+  for (const Gate &g : gates)
+    if (g.inst >= 0) A.folded += 4;
+    else if (g.targets.size() + g.controls.size() <= 3 && permutation_of(g.U, (int)g.targets.size(), perm)) A.folded += 3;
   A.sites = sites;
   A.n_acc = A.n_params;
   A.n_mats = 2 * A.n_inst;
@@ -152,7 +159,7 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     if (passes.empty() && !blocks.empty()) return set_error(SV_EINVAL, "internal: pass planning failed");
     BuildCtx b{s->dt, s->n, m, L, 1, 0};
     b.site_mat = fwd_mat.data();
-    append_passes(A.prog, A.op0s, split_sites(passes), b, fwd_off, st);
+    append_passes(A.prog, A.op0s, split_sites(passes, A.split), b, fwd_off, st);
   }
   // lambda = H psi
   {
@@ -220,7 +227,7 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     b.site_slot = A.rev_slot.data();
     b.site_comps = A.rev_comps.data();
     const size_t first = A.prog.passes.size();
-    append_passes(A.prog, A.op0s, split_sites(passes), b, rev_off, st);
+    append_passes(A.prog, A.op0s, split_sites(passes, A.split), b, rev_off, st);
     if (sites && st == SV_OK && A.prog.passes.size() > first) {
       A.prog.passes[first].flags |= kPassShift;
       A.prog.passes[first].mat0 = (uint32_t)A.n_acc;
@@ -308,28 +315,10 @@ static sv_status check_batch(sv_state *const *psi, int B, int n, sv_dtype dt, cu
   return SV_OK;
 }
 
-static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B, const sv_circuit *c,
-                               const double *params, const sv_pauli_term *terms, int nt, const sv_options *opt,
-                               double *ev_out, double *grad_out) {
-  if (!psi || !lam || B < 1 || !c || !ev_out || (c->n_params > 0 && (!params || !grad_out)))
-    return set_error(SV_EINVAL, "null argument");
-  sv_state *s = psi[0];
-  if (!s) return set_error(SV_EINVAL, "null state");
-  SV_TRY(check_batch(psi, B, s->n, s->dt, s->stream));
-  SV_TRY(check_batch(lam, B, s->n, s->dt, s->stream));
-  // complex64 states that start as a basis state have norm 1 after the circuit;
-  // what FP32 rounding makes of it (1e-6 after some hundred gates, the largest
-  // part of the energy's error) is divided out
-  std::vector<char> unit(B, 0);
-  for (int b = 0; b < B; b++) {
-    unit[b] = s->dt == SV_C64 && psi[b]->basis_known;
-    psi[b]->basis_known = lam[b]->basis_known = false;
-  }
-  if (nt < 0 || (nt > 0 && !terms)) return set_error(SV_EINVAL, "bad term list");
-  const uint64_t lim = (1ull << s->n) - 1;
-  for (int t = 0; t < nt; t++)
-    if ((terms[t].x_mask & ~lim) || (terms[t].z_mask & ~lim))
-      return set_error(SV_EINVAL, "Pauli mask references a qubit >= n");
+// The program of a circuit's gradient for B parameter sets, from the cache or
+// built.
+static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms,
+                                 int nt, const sv_options *opt, int B, std::shared_ptr<const AdjointProgram> &Ap) {
   Opts o1 = resolve(s, opt, 1), o2 = resolve(s, opt, 2);
   // defaults for the gradient program (measured on the 20-qubit, 64-set
   // ansatz): fusion width 2 and 12-qubit tiles for both sweeps
@@ -357,16 +346,67 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
   // matrices fit the program area); complex128 ones are bound by FP64
   // arithmetic, which the probes of three components a site would add to
   const bool sites = s->dt == SV_C64 && s->n >= 3 && o1.tile_m >= 3 && o2.tile_m >= 3;
-  const int np = c->n_params;
   k.val((int)sites);
   const uint64_t kh = k.hash();
-  std::shared_ptr<const AdjointProgram> Ap = g_adj_cache.find(s, k, kh);
+  Ap = g_adj_cache.find(s, k, kh);
   if (!Ap) {
     auto built = std::make_shared<AdjointProgram>();
     SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, sites, *built));
+    if (built->split) {
+      // Fixed gates that are not permutations cut passes of sites; a launch
+      // more, with its read and write of the vectors, costs what four
+      // parametric or five permutation gates in sites save (ms
+      // in sites and with a probe and a matrix per gate, six layers of RY and
+      // RZ, 26 qubits: CNOT ladder, no cut 32.5 and 87, H before each RY 73 and
+      // 91, one CZ a layer 41 and 92, CZ ladder 128 and 119, CZ bricks 112 and
+      // 82, only the last layer parametric 58 and 49; 16 qubits 0.28 and 0.76,
+      // 0.63 and 0.81, 0.37 and 0.80, 0.80 and 0.85, 0.73 and 0.65, 0.49 and
+      // 0.45)
+      auto plain = std::make_shared<AdjointProgram>();
+      SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, false, *plain));
+      const int more = (int)built->prog.passes.size() - (int)plain->prog.passes.size();
+      if (16 * more > built->folded) built = std::move(plain);
+    }
     built->serial = next_program_serial();
     Ap = g_adj_cache.insert(s, k, kh, std::move(built));
   }
+  return SV_OK;
+}
+
+sv_status adjoint_passes(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt,
+                         const sv_options *opt, int B, int *n_passes, int *sites) {
+  std::shared_ptr<const AdjointProgram> Ap;
+  SV_TRY(adjoint_program(s, c, params, terms, nt, opt, B, Ap));
+  *n_passes = (int)Ap->prog.passes.size();
+  *sites = Ap->sites;
+  return SV_OK;
+}
+
+static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B, const sv_circuit *c,
+                               const double *params, const sv_pauli_term *terms, int nt, const sv_options *opt,
+                               double *ev_out, double *grad_out) {
+  if (!psi || !lam || B < 1 || !c || !ev_out || (c->n_params > 0 && (!params || !grad_out)))
+    return set_error(SV_EINVAL, "null argument");
+  sv_state *s = psi[0];
+  if (!s) return set_error(SV_EINVAL, "null state");
+  SV_TRY(check_batch(psi, B, s->n, s->dt, s->stream));
+  SV_TRY(check_batch(lam, B, s->n, s->dt, s->stream));
+  // complex64 states that start as a basis state have norm 1 after the circuit;
+  // what FP32 rounding makes of it (1e-6 after some hundred gates, the largest
+  // part of the energy's error) is divided out
+  std::vector<char> unit(B, 0);
+  for (int b = 0; b < B; b++) {
+    unit[b] = s->dt == SV_C64 && psi[b]->basis_known;
+    psi[b]->basis_known = lam[b]->basis_known = false;
+  }
+  if (nt < 0 || (nt > 0 && !terms)) return set_error(SV_EINVAL, "bad term list");
+  const uint64_t lim = (1ull << s->n) - 1;
+  for (int t = 0; t < nt; t++)
+    if ((terms[t].x_mask & ~lim) || (terms[t].z_mask & ~lim))
+      return set_error(SV_EINVAL, "Pauli mask references a qubit >= n");
+  const int np = c->n_params;
+  std::shared_ptr<const AdjointProgram> Ap;
+  SV_TRY(adjoint_program(s, c, params, terms, nt, opt, B, Ap));
   const AdjointProgram &A = *Ap;
   // per-batch matrices, state pointer tables
   std::vector<uint8_t> pm;

@@ -527,6 +527,10 @@ sv_status upload_program(sv_state *s, const CachedProgram &cp);
 sv_status func_attr_once(const void *fn, int device, cudaFuncAttribute attr, int value);
 void drop_graphs(const sv_state *s);
 void drop_adjoint_programs(const sv_state *s);
+// passes that a gradient of B parameter sets launches, and whether they are made
+// of sites (sv_adjoint.cu)
+sv_status adjoint_passes(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt,
+                         const sv_options *opt, int B, int *n_passes, int *sites);
 
 // kernels (launchers), all enqueue on s->stream
 sv_status launch_set_basis(sv_state *s, uint64_t index);

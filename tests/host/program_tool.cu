@@ -29,3 +29,13 @@ extern "C" int program_build(const sv_circuit *c, int dt, const sv_options *opt,
 }
 
 extern "C" uint64_t program_area() { return kWsProgBytes; }
+
+// Passes a gradient of B parameter sets launches (complex64), *sites whether
+// they are made of sites; -status on an error.
+extern "C" int gradient_passes(const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt, int B,
+                               int dt, int *sites) {
+  sv_state s = host_state(c->n_qubits, dt);
+  int n = 0;
+  const sv_status st = adjoint_passes(&s, c, params, terms, nt, nullptr, B, &n, sites);
+  return st == SV_OK ? n : -(int)st;
+}

@@ -70,3 +70,46 @@ def test_small_state_plans_take_no_more_than_large_tiles(tool, dt):
     large, _ = build(tool, c, dt, sim.options(fusion_k=3, tile_m=13 if dt == SV_C64 else 12))
     small, _ = build(tool, c, dt)
     assert large <= tool.program_area() and small <= tool.program_area()
+
+
+# ---- gradients ----------------------------------------------------------------
+def ansatz(n, layers, entangle, fixed=()):
+    """RY and RZ on every qubit behind `fixed` gates, then two-qubit gates."""
+    ops, np_ = [], 0
+    for k in range(layers):
+        for q in range(n):
+            ops += [W.Op(f, (q,)) for f in fixed]
+            for r in ("RY", "RZ"):
+                ops.append(W.Op(r, (q,), param=np_))
+                np_ += 1
+        ops += entangle(k)
+    return W.Circuit(n, ops, n_params=np_)
+
+
+def gradient(tool, c, sets, dt=SV_C64):
+    """(passes a gradient launches, whether they are made of sites)"""
+    from paper_2106_13995_gb300 import _native as N, sim
+    m, p, t = sim.marshal(c), np.ones(max(1, c.n_params)), W.tfim(c.n_qubits)
+    terms, sites = (N.SvPauliTerm * len(t))(*[N.SvPauliTerm(*x) for x in t]), C.c_int()
+    n = tool.gradient_passes(C.byref(m.c), p.ctypes.data_as(C.c_void_p), terms, len(t), sets, dt, C.byref(sites))
+    assert n > 0, n
+    return n, bool(sites.value)
+
+
+@pytest.mark.parametrize("n,sets,layers", [(16, 1, 6), (20, 64, 10), (26, 1, 6)])
+def test_fixed_gates_do_not_cut_gradients_into_many_passes(tool, n, sets, layers):
+    """Sites are kept where what they fold is worth the launches they add to a
+    plan of single gates."""
+    def ladder(gate):
+        return lambda k: [W.Op(gate, (q, q + 1)) if gate != "X" else W.Op("X", (q + 1,), (q,)) for q in range(n - 1)]
+
+    def bricks(k):
+        return [W.Op("CZ", (q, q + 1)) for q in range(k % 2, n - 1, 2)]
+
+    plain = gradient(tool, ansatz(n, layers, ladder("CZ")), sets)
+    brick = gradient(tool, ansatz(n, layers, bricks), sets)
+    assert not plain[1] and not brick[1] and brick[0] <= plain[0] <= 40
+    cnots, sites = gradient(tool, ansatz(n, layers, ladder("X")), sets)
+    assert sites and cnots <= 1.25 * plain[0]
+    mixed, sites = gradient(tool, ansatz(n, layers, ladder("X"), ("H",)), sets)
+    assert 16 * (mixed - plain[0]) <= 4 * 2 * n * layers + 3 * (n - 1) * layers or not sites
