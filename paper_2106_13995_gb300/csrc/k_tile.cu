@@ -194,8 +194,10 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
           im += a.x * c.y - a.y * c.x;
         }
         block_acc<R>(part, acc + op.mat);
-        block_acc<R>(norm, acc + op.mat + 1);
-        block_acc<R>(im, acc + op.mat + 2);
+        if (op.gen) {
+          block_acc<R>(norm, acc + op.mat + 1);
+          block_acc<R>(im, acc + op.mat + 2);
+        }
         break;
       }
       default:

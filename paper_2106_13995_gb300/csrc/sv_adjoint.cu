@@ -37,7 +37,8 @@ struct AdjointProgram {
   int folded = 0;                // gates that sites take: 4 per parametric gate, 3 per permutation
   std::vector<AdjSite> fwd_sites, rev_sites;
   std::vector<int> rev_slot, rev_comps;
-  int n_acc = 0;                 // accumulators, TOP_DOT's three excluded
+  int n_acc = 0;                 // accumulators of the probes; TOP_DOT's follow
+  bool norms = false;            // TOP_DOT takes <psi|psi> and Im <psi|lambda> too
   int n_mats = 0;                // per-batch 2 x 2 matrices
 };
 
@@ -102,7 +103,7 @@ static void append_passes(DeviceProgram &prog, std::vector<uint32_t> &op0s, cons
 
 static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *params0,
                                const sv_pauli_term *terms, int nt, const Opts &o1, const Opts &o2, bool sites,
-                               AdjointProgram &A) {
+                               bool norms, AdjointProgram &A) {
   std::vector<Gate> gates;
   SV_TRY(circuit_to_gates(c, params0, s->n, gates, true));
   A.n_params = c->n_params;
@@ -121,6 +122,7 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     if (g.inst >= 0) A.folded += 4;
     else if (g.targets.size() + g.controls.size() <= 3 && permutation_of(g.U, (int)g.targets.size(), perm)) A.folded += 3;
   A.sites = sites;
+  A.norms = norms;
   A.n_acc = A.n_params;
   A.n_mats = 2 * A.n_inst;
   std::vector<Block> fwd_blocks, rev_blocks;
@@ -191,6 +193,7 @@ static sv_status build_adjoint(sv_state *s, const sv_circuit *c, const double *p
     Block dot;
     dot.kind = TOP_DOT;
     dot.slot = A.n_acc;
+    dot.gen = norms;
     passes.back().ops.push_back(dot);
     for (size_t i = 0; i < passes.size() && st == SV_OK; i++) {
       BuildCtx b{s->dt, s->n, m, L, 2, (i == 0 ? 1u : 0u) | 2u};
@@ -316,9 +319,11 @@ static sv_status check_batch(sv_state *const *psi, int B, int n, sv_dtype dt, cu
 }
 
 // The program of a circuit's gradient for B parameter sets, from the cache or
-// built.
+// built.  lean: the one that takes least of the workspace, a probe and a matrix
+// per gate, one accumulator per parameter and one for the energy.
 static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms,
-                                 int nt, const sv_options *opt, int B, std::shared_ptr<const AdjointProgram> &Ap) {
+                                 int nt, const sv_options *opt, int B, bool lean,
+                                 std::shared_ptr<const AdjointProgram> &Ap) {
   Opts o1 = resolve(s, opt, 1), o2 = resolve(s, opt, 2);
   // defaults for the gradient program (measured on the 20-qubit, 64-set
   // ansatz): fusion width 2 and 12-qubit tiles for both sweeps
@@ -329,7 +334,7 @@ static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double 
     // 497 -> 398; at 20 qubits 700 -> 776)
     int lb = 0;
     while ((2 << lb) <= B) lb++;
-    o1.tile_m = o2.tile_m = std::min(s->dt == SV_C64 && s->n + lb <= 18 ? 10 : 12, s->n);
+    o1.tile_m = o2.tile_m = std::min(s->dt == SV_C64 && !lean && s->n + lb <= 18 ? 10 : 12, s->n);
     o1.L = o2.L = std::min(o1.L, o1.tile_m);
   }
   // cache key: circuit structure, terms, options (parameters enter only the
@@ -341,17 +346,17 @@ static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double 
   k.val(o1);
   k.val(o2);
   k.val(s->dt);
-  // complex64 programs are made of sites (their accumulators, at most one and
-  // a half per parametric gate, fit the reduction area whenever the gates'
-  // matrices fit the program area); complex128 ones are bound by FP64
+  // complex64 programs are made of sites; complex128 ones are bound by FP64
   // arithmetic, which the probes of three components a site would add to
-  const bool sites = s->dt == SV_C64 && s->n >= 3 && o1.tile_m >= 3 && o2.tile_m >= 3;
+  const bool sites = s->dt == SV_C64 && !lean && s->n >= 3 && o1.tile_m >= 3 && o2.tile_m >= 3;
+  const bool norms = s->dt == SV_C64 && !lean;
   k.val((int)sites);
+  k.val((int)norms);
   const uint64_t kh = k.hash();
   Ap = g_adj_cache.find(s, k, kh);
   if (!Ap) {
     auto built = std::make_shared<AdjointProgram>();
-    SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, sites, *built));
+    SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, sites, norms, *built));
     if (built->split) {
       // Fixed gates that are not permutations cut passes of sites; a launch
       // more, with its read and write of the vectors, costs what four
@@ -363,7 +368,7 @@ static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double 
       // 0.63 and 0.81, 0.37 and 0.80, 0.80 and 0.85, 0.73 and 0.65, 0.49 and
       // 0.45)
       auto plain = std::make_shared<AdjointProgram>();
-      SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, false, *plain));
+      SV_TRY(build_adjoint(s, c, params, terms, nt, o1, o2, false, norms, *plain));
       const int more = (int)built->prog.passes.size() - (int)plain->prog.passes.size();
       if (16 * more > built->folded) built = std::move(plain);
     }
@@ -373,12 +378,33 @@ static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double 
   return SV_OK;
 }
 
-sv_status adjoint_passes(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt,
-                         const sv_options *opt, int B, int *n_passes, int *sites) {
+// Bytes of the workspace for B parameter sets.
+static ProgLayout adjoint_layout(const sv_state *s, const AdjointProgram &A, int B) {
+  return layout_of(A.prog, 2 * (size_t)B * sizeof(void *), (size_t)B * A.n_mats * 4 * amp_bytes(s->dt));
+}
+static size_t adjoint_acc_stride(const AdjointProgram &A) { return (size_t)A.n_acc + (A.norms ? 3 : 1); }
+
+// The same, lean where the program would outgrow the workspace (a site takes
+// 128 bytes a sweep on its own, a single gate 128 in all).
+static sv_status fitting_program(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms,
+                                 int nt, const sv_options *opt, int B, std::shared_ptr<const AdjointProgram> &Ap) {
+  for (bool lean : {false, true}) {
+    SV_TRY(adjoint_program(s, c, params, terms, nt, opt, B, lean, Ap));
+    if (adjoint_layout(s, *Ap, B).end <= kWsProgBytes &&
+        adjoint_acc_stride(*Ap) * B * sizeof(double) <= red_bytes(s->n))
+      break;
+  }
+  return SV_OK;
+}
+
+sv_status adjoint_plan(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt,
+                       const sv_options *opt, int B, AdjointPlan &out) {
   std::shared_ptr<const AdjointProgram> Ap;
-  SV_TRY(adjoint_program(s, c, params, terms, nt, opt, B, Ap));
-  *n_passes = (int)Ap->prog.passes.size();
-  *sites = Ap->sites;
+  SV_TRY(fitting_program(s, c, params, terms, nt, opt, B, Ap));
+  out.passes = (int)Ap->prog.passes.size();
+  out.sites = Ap->sites;
+  out.prog_bytes = adjoint_layout(s, *Ap, B).end;
+  out.acc_bytes = adjoint_acc_stride(*Ap) * B * sizeof(double);
   return SV_OK;
 }
 
@@ -406,7 +432,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
       return set_error(SV_EINVAL, "Pauli mask references a qubit >= n");
   const int np = c->n_params;
   std::shared_ptr<const AdjointProgram> Ap;
-  SV_TRY(adjoint_program(s, c, params, terms, nt, opt, B, Ap));
+  SV_TRY(fitting_program(s, c, params, terms, nt, opt, B, Ap));
   const AdjointProgram &A = *Ap;
   // per-batch matrices, state pointer tables
   std::vector<uint8_t> pm;
@@ -421,7 +447,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
     tbl[b] = psi[b]->amps;
     tbl[B + b] = lam[b]->amps;
   }
-  const ProgLayout L = layout_of(A.prog, tbl.size() * sizeof(void *), pm.size());
+  const ProgLayout L = adjoint_layout(s, A, B);
   SV_TRY(stage_upload(s,
                       {{A.prog.ops.data(), A.prog.ops.size() * sizeof(TileOp)},
                        {A.prog.mats.data(), A.prog.mats.size()},
@@ -429,7 +455,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
                        {tbl.data(), tbl.size() * sizeof(void *)},
                        {pm.data(), pm.size()}},
                       {L.ops_off, L.mats_off, L.coeffs_off, L.tbl_off, L.pmats_off}, L.end));
-  const size_t acc_stride = (size_t)A.n_acc + 3;
+  const size_t acc_stride = adjoint_acc_stride(A);
   const size_t acc_bytes = acc_stride * B * sizeof(double);
   if (acc_bytes > red_bytes(s->n)) return set_error(SV_ENOMEM, "workspace too small for the gradient batch");
   double *acc = reinterpret_cast<double *>(s->ws + kWsRed);
@@ -492,7 +518,7 @@ static sv_status adjoint_batch(sv_state *const *psi, sv_state *const *lam, int B
     } else {
       for (int p = 0; p < np; p++) grad_out[(size_t)b * np + p] = hb[p];
     }
-    const double norm = hb[A.n_acc + 1];
+    const double norm = A.norms ? hb[A.n_acc + 1] : 1.0;
     if (unit[b] && norm > 0.5 && norm < 2.0) {
       ev_out[b] /= norm;
       for (int p = 0; p < np; p++) grad_out[(size_t)b * np + p] /= norm;

@@ -594,6 +594,7 @@ sv_status emit_pass(DeviceProgram &prog, const PassPlan &P, const BuildCtx &b,
       op.mat = (uint32_t)prog.coeffs.size();
       prog.coeffs.push_back(blk.coeff);
     } else if (op.kind == TOP_DOT) {
+      op.gen = (uint8_t)blk.gen;
       op.mat = (uint32_t)blk.slot;   // (sites have more accumulators than 15 bits count)
     }
     op.gcmask_lo = (uint32_t)gcm;

@@ -51,7 +51,7 @@ enum TileOpKind : uint8_t {
   TOP_GRAD = 2,      // acc[slot] += Im <v1 | G v0>, G = X/Y/Z/P1(-2) on one local target
   TOP_PAULI = 3,     // v1[l ^ xm] += c * phase * (-1)^{popcount(l & zm)} v0[l]
   TOP_ZERO = 4,      // v1 <- 0
-  TOP_DOT = 5,       // acc[mat] += Re <v0 | v1>, acc[mat + 1] += <v0 | v0>, acc[mat + 2] += Im <v0 | v1>
+  TOP_DOT = 5,       // acc[mat] += Re <v0 | v1>; with gen acc[mat + 1] += <v0 | v0>, acc[mat + 2] += Im <v0 | v1>
   TOP_TC = 6,        // 5-qubit dense block on the tensor cores (12-qubit tiles)
   TOP_PERM = 7,      // permutation block (k = 1..3): member y moves to member perm[y]; controls as TOP_DENSE
   TOP_GRADU = 8,     // TOP_GRAD then the 1-qubit matrix (per-batch pool) on both vectors, in one sweep
@@ -527,10 +527,14 @@ sv_status upload_program(sv_state *s, const CachedProgram &cp);
 sv_status func_attr_once(const void *fn, int device, cudaFuncAttribute attr, int value);
 void drop_graphs(const sv_state *s);
 void drop_adjoint_programs(const sv_state *s);
-// passes that a gradient of B parameter sets launches, and whether they are made
-// of sites (sv_adjoint.cu)
-sv_status adjoint_passes(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt,
-                         const sv_options *opt, int B, int *n_passes, int *sites);
+// What a gradient of B parameter sets launches and takes of the workspace
+// (sv_adjoint.cu).
+struct AdjointPlan {
+  int passes = 0, sites = 0;   // sites: made of them
+  size_t prog_bytes = 0, acc_bytes = 0;
+};
+sv_status adjoint_plan(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt,
+                       const sv_options *opt, int B, AdjointPlan &out);
 
 // kernels (launchers), all enqueue on s->stream
 sv_status launch_set_basis(sv_state *s, uint64_t index);

@@ -30,12 +30,18 @@ extern "C" int program_build(const sv_circuit *c, int dt, const sv_options *opt,
 
 extern "C" uint64_t program_area() { return kWsProgBytes; }
 
-// Passes a gradient of B parameter sets launches (complex64), *sites whether
-// they are made of sites; -status on an error.
+// Passes a gradient of B parameter sets launches, *sites whether they are made of
+// sites, *prog and *acc the bytes of the program and of the reduction area it
+// takes; -status on an error.
 extern "C" int gradient_passes(const sv_circuit *c, const double *params, const sv_pauli_term *terms, int nt, int B,
-                               int dt, int *sites) {
+                               int dt, int *sites, uint64_t *prog, uint64_t *acc) {
   sv_state s = host_state(c->n_qubits, dt);
-  int n = 0;
-  const sv_status st = adjoint_passes(&s, c, params, terms, nt, nullptr, B, &n, sites);
-  return st == SV_OK ? n : -(int)st;
+  AdjointPlan p;
+  const sv_status st = adjoint_plan(&s, c, params, terms, nt, nullptr, B, p);
+  *sites = p.sites;
+  *prog = p.prog_bytes;
+  *acc = p.acc_bytes;
+  return st == SV_OK ? p.passes : -(int)st;
 }
+
+extern "C" uint64_t reduction_area(int n) { return red_bytes(n); }

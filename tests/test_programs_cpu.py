@@ -15,7 +15,7 @@ OZ, MOVES = 0x1000, 0x2000   # kPassOz, kPassMoves
 @pytest.fixture(scope="module")
 def tool():
     L = load("program_tool")
-    L.program_area.restype = C.c_uint64
+    L.program_area.restype = L.reduction_area.restype = C.c_uint64
     return L
 
 
@@ -87,12 +87,16 @@ def ansatz(n, layers, entangle, fixed=()):
 
 
 def gradient(tool, c, sets, dt=SV_C64):
-    """(passes a gradient launches, whether they are made of sites)"""
+    """(passes a gradient launches, whether they are made of sites); it must
+    fit the workspace."""
     from paper_2106_13995_gb300 import _native as N, sim
     m, p, t = sim.marshal(c), np.ones(max(1, c.n_params)), W.tfim(c.n_qubits)
     terms, sites = (N.SvPauliTerm * len(t))(*[N.SvPauliTerm(*x) for x in t]), C.c_int()
-    n = tool.gradient_passes(C.byref(m.c), p.ctypes.data_as(C.c_void_p), terms, len(t), sets, dt, C.byref(sites))
+    prog, acc = C.c_uint64(), C.c_uint64()
+    n = tool.gradient_passes(C.byref(m.c), p.ctypes.data_as(C.c_void_p), terms, len(t), sets, dt, C.byref(sites),
+                             C.byref(prog), C.byref(acc))
     assert n > 0, n
+    assert prog.value <= tool.program_area() and acc.value <= tool.reduction_area(c.n_qubits)
     return n, bool(sites.value)
 
 
@@ -113,3 +117,27 @@ def test_fixed_gates_do_not_cut_gradients_into_many_passes(tool, n, sets, layers
     assert sites and cnots <= 1.25 * plain[0]
     mixed, sites = gradient(tool, ansatz(n, layers, ladder("X"), ("H",)), sets)
     assert 16 * (mixed - plain[0]) <= 4 * 2 * n * layers + 3 * (n - 1) * layers or not sites
+
+
+@pytest.mark.parametrize("dt", [SV_C64, SV_C128])
+def test_deep_gradients_fit_as_single_gates(tool, dt):
+    """RX and a Toffoli in turn on three qubits: an op of 128 bytes a sweep and
+    two matrices of 32 for each pair in sites, 256 bytes in all as single gates
+    (384 in complex128)."""
+    depth = 30000 if dt == SV_C64 else 20000
+    ops = []
+    for k in range(depth):
+        a, b, d = k % 3, (k + 1) % 3, (k + 2) % 3
+        ops += [W.Op("RX", (a,), param=k), W.Op("X", (b,), (a, d))]
+    c = W.Circuit(6, ops, n_params=depth)
+    gradient(tool, c, 1, dt)
+
+
+@pytest.mark.parametrize("dt", [SV_C64, SV_C128])
+def test_accumulators_leave_room_for_every_parameter(tool, dt):
+    """As many parameters as the reduction area holds beside the energy, most of
+    them without a gate."""
+    n, sets = 8, 64
+    c = W.Circuit(n, [W.Op("RX", (q,), param=q) for q in range(n)],
+                  n_params=tool.reduction_area(n) // 8 // sets - 1)
+    gradient(tool, c, sets, dt)
