@@ -330,7 +330,10 @@ sv_status sv_sample(sv_state *s, int64_t n_shots, uint64_t seed, uint64_t *out_h
  * psi_out = circuit(theta) psi_in:  forward sweep on psi, lambda = H psi,
  * then a reverse sweep that un-applies each gate from both vectors and adds
  * Im<lambda|G_j|psi> for each parametric gate U_j = exp(-i theta G_j / 2)
- * (RX, RY, RZ; PHASE with G = diag(0, -2)); no tape of states is kept.
+ * (RX, RY, RZ; PHASE with G = diag(0, -2)); no tape of states is kept.  For
+ * complex64 states and unitary circuits, E and the gradient are divided by
+ * <psi_out|psi_out> / <psi_in|psi_in> as measured where it differs from 1 by
+ * less than 1e-3: the norm that FP32 rounding added or took.
  *   psi:            in = psi_in; out = psi_out.
  *   lambda_scratch: a state of the same width and dtype (clobbered).
  *   params:         host FP64, c->n_params.

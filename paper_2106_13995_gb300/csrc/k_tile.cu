@@ -111,11 +111,13 @@ __device__ __forceinline__ void tile_body(const TilePass &P, uint64_t tile, int 
   const C *pmats = P.pmats ? reinterpret_cast<const C *>(P.pmats) + (size_t)b * P.pmats_stride : nullptr;
   double *acc = P.acc ? P.acc + (size_t)b * P.acc_stride : nullptr;
 
-  if constexpr (!COH && !INL && sizeof(R) == 4)
+  if constexpr (!COH && !INL && sizeof(R) == 4) {
     if (P.flags & kPassShift) {
       __syncthreads();
       shift_energy(v0, v1, TS, acc + P.mat0);
     }
+    if (P.flags & kPassNorm) block_acc<R>(loaded_norm(v0, nunits), acc + P.mat0);
+  }
   for (int oi = 0; oi < P.nops; oi++) {
     __syncthreads();
     TileOp op;
@@ -544,7 +546,7 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
   const int threads = pass_threads(s, p.m, (int)p.nvec, (uint64_t)grid.x * grid.y);
   if (host && sites_pass_ok(p, *host)) return launch_tile_sites(s, p, batch, threads, stream);
   sv_status st = SV_OK;
-  const bool try_inl = host && s->dt == SV_C64 && batch == 1 && p.nvec == 1;
+  const bool try_inl = host && s->dt == SV_C64 && batch == 1 && p.nvec == 1 && !(p.flags & kPassNorm);
   if (try_inl && (launch_inl<TileInlineSmall>(s, p, *host, grid, threads, smem, stream, st) ||
                   launch_inl<TileInlineMid>(s, p, *host, grid, threads, smem, stream, st) ||
                   launch_inl<TileInline>(s, p, *host, grid, threads, smem, stream, st)))

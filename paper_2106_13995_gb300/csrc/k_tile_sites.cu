@@ -205,6 +205,16 @@ __global__ void __launch_bounds__(kSitesThreads, 3) k_tile_sites(const __grid_co
     __syncthreads();
     shift_energy(reinterpret_cast<const float2 *>(smem_raw), reinterpret_cast<float2 *>(smem_raw) + TS, TS, acc + P.mat0);
   }
+  if (!TWO && (P.flags & kPassNorm)) {
+    const float p = warp_sum(loaded_norm(reinterpret_cast<const float2 *>(smem_raw), nunits));
+    if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = p;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0;
+      for (uint32_t w = 0; w < (T + 31) / 32; w++) t += (double)red[0][w];
+      atomicAdd(acc + P.mat0, t);
+    }
+  }
   for (int oi = 0; oi < P.nops; oi++) {
     __syncthreads();
     if (TWO && oi > 0) flush_probes(ent + (uint32_t)(oi - 1) * kSitesEntry, red[(oi - 1) & 1], acc);

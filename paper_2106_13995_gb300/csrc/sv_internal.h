@@ -148,6 +148,9 @@ constexpr uint32_t kPassMoves = 0x2000;
 // TilePass.flags: v1 -= e v0 first, e = <v0 | v1> / <v0 | v0> from the accumulators
 // mat0 to mat0 + 2 (a gradient's first reverse pass, complex64)
 constexpr uint32_t kPassShift = 0x8000;
+// TilePass.flags: acc[mat0] += <v0 | v0> before the ops (a gradient's first
+// forward pass, complex64)
+constexpr uint32_t kPassNorm = 0x10000;
 // TilePass.flags: the state, a known basis state, through one single-qubit gate
 // per qubit, written as the product it is; mat0: 16-byte index of 2 x 2
 // complex128 matrices of the n qubits (host copy; k_moves.cu)

@@ -550,6 +550,17 @@ __device__ __forceinline__ void shift_energy(const float2 *v0, float2 *v1, uint3
   }
 }
 
+// sum |psi|^2 over the 16-byte units (complex64) that this thread loaded
+__device__ __forceinline__ float loaded_norm(const float2 *v0, uint32_t nunits) {
+  float p = 0;
+  for (uint32_t u = threadIdx.x; u < nunits; u += blockDim.x) {
+    const uint32_t vs = smem_u32(v0);
+    const float2 a = lds_c(vs + swb<float>(2 * u), v0), b = lds_c(vs + swb<float>(2 * u + 1), v0);
+    p = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(b.x, b.x, fmaf(b.y, b.y, p))));
+  }
+  return p;
+}
+
 template <typename R>
 __device__ void grad_op(const typename Cx<R>::T *__restrict__ psi,
                         const typename Cx<R>::T *__restrict__ lam, int m, const TileOp &op,
