@@ -358,10 +358,16 @@ sv_status sv_adjoint_grad_batch(sv_state *const *psi, sv_state *const *lam, int 
 
 /* Time candidate (fusion_k in 2..6, tile_m in 10..13, limited by n) pairs
  * for this circuit on `scratch` (its contents are clobbered; the circuit must
- * not be parametric) and write the fastest into *inout.  The choice is
+ * not be parametric) and write the fastest into *inout.  With inout->prec ==
+ * SV_PREC_PLAIN the defaults are timed too; where they are fastest, their
+ * fusion width and tile size are written, or 0 for both if the circuit runs on
+ * paths that only options left at 0 take (complex128 tensor-core passes,
+ * permutation runs).  The choice is
  * cached per (n, dtype, op-count bucket, widest op) in memory and, if the
  * SV_TUNE_CACHE environment variable names a file, in that JSON file;
- * sv_apply_circuit and sv_apply_circuit_batch use it for options left at 0.
+ * sv_apply_circuit and sv_apply_circuit_batch use it for options left at 0
+ * (a pair from a file written before the defaults were timed replaces their
+ * tile passes only).
  * Only CUDA-core timings (inout->prec == SV_PREC_PLAIN) enter the cache, and
  * only calls in that precision mode read it: the tensor-core modes keep
  * 5-qubit blocks and 12-qubit tiles.  Synchronises. */

@@ -18,10 +18,15 @@
 namespace sv {
 
 // ---------------------------------------------------------------------------
-// autotune cache: (n, dtype, op-count bucket, widest op) -> (fusion_k, tile_m)
+// autotune cache: (n, dtype, op-count bucket, widest op) -> (fusion_k, tile_m),
+// 0 where the defaults were faster than every pair
 // ---------------------------------------------------------------------------
 using TuneKey = std::tuple<int, int, int, int>;
-static std::map<TuneKey, std::pair<int, int>> g_tune;
+struct Tuned {
+  int k, m;
+  int vs_defaults;   // timed against the defaults with all their paths
+};
+static std::map<TuneKey, Tuned> g_tune;
 static std::mutex g_tune_mu;
 static bool g_tune_loaded = false;
 
@@ -43,10 +48,12 @@ static void tune_load_locked() {
   if (!f) return;
   char line[512];
   while (std::fgets(line, sizeof line, f)) {
-    int n, dt, b, a, k, m;
-    if (std::sscanf(line, " {\"n\": %d, \"dtype\": %d, \"ops_bucket\": %d, \"arity\": %d, \"fusion_k\": %d, \"tile_m\": %d",
-                    &n, &dt, &b, &a, &k, &m) == 6)
-      g_tune[TuneKey(n, dt, b, a)] = {k, m};
+    int n, dt, b, a, k, m, v = 0;   // (files of earlier builds end with tile_m)
+    if (std::sscanf(line,
+                    " {\"n\": %d, \"dtype\": %d, \"ops_bucket\": %d, \"arity\": %d, \"fusion_k\": %d, \"tile_m\": %d, "
+                    "\"vs_defaults\": %d",
+                    &n, &dt, &b, &a, &k, &m, &v) >= 6)
+      g_tune[TuneKey(n, dt, b, a)] = {k, m, v};
   }
   std::fclose(f);
 }
@@ -59,9 +66,11 @@ static void tune_save_locked() {
   std::fprintf(f, "[\n");
   size_t i = 0;
   for (auto &kv : g_tune) {
-    std::fprintf(f, "  {\"n\": %d, \"dtype\": %d, \"ops_bucket\": %d, \"arity\": %d, \"fusion_k\": %d, \"tile_m\": %d}%s\n",
+    std::fprintf(f,
+                 "  {\"n\": %d, \"dtype\": %d, \"ops_bucket\": %d, \"arity\": %d, \"fusion_k\": %d, \"tile_m\": %d, "
+                 "\"vs_defaults\": %d}%s\n",
                  std::get<0>(kv.first), std::get<1>(kv.first), std::get<2>(kv.first), std::get<3>(kv.first),
-                 kv.second.first, kv.second.second, ++i < g_tune.size() ? "," : "");
+                 kv.second.k, kv.second.m, kv.second.vs_defaults, ++i < g_tune.size() ? "," : "");
   }
   std::fprintf(f, "]\n");
   std::fclose(f);
@@ -76,10 +85,13 @@ void tuned_options(const sv_state *s, const sv_circuit *c, const sv_options *opt
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_load_locked();
   auto it = g_tune.find(tune_key(s->n, s->dt, c));
-  if (it == g_tune.end() || it->second.first == 0) return;   // not tuned, or the defaults were fastest
-  o.oz = o.moves = o.small = 0;   // the pair was timed on the CUDA cores' tile passes
-  if (want_k) o.fusion_k = it->second.first;
-  if (want_m) o.tile_m = std::min(it->second.second, s->n);
+  if (it == g_tune.end() || it->second.k == 0) return;   // not tuned, or the defaults were fastest
+  // a pair that beat the defaults takes the place of all their paths; one that
+  // was never timed against them, of their tile passes
+  if (it->second.vs_defaults) o.oz = o.moves = 0;
+  o.small = 0;
+  if (want_k) o.fusion_k = it->second.k;
+  if (want_m) o.tile_m = std::min(it->second.m, s->n);
 }
 
 // ---------------------------------------------------------------------------
@@ -431,9 +443,22 @@ sv_status sv_autotune(sv_state *s, const sv_circuit *c, sv_options *inout) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (ms0 <= best) bk = bm = 0;
+  if (ms0 <= best) {
+    // as a pair, if it gives the same program; 0 keeps the defaults
+    ProgramRef cp, ep;
+    Opts o, eo;
+    SV_TRY(get_program(s, c, nullptr, &def, &cp, &o));
+    sv_options e = def;
+    e.fusion_k = o.fusion_k;
+    e.tile_m = o.tile_m;
+    SV_TRY(get_program(s, c, nullptr, &e, &ep, &eo));
+    const bool same = ep->prog.passes.size() == cp->prog.passes.size() && ep->prog.mats == cp->prog.mats;
+    inout->fusion_k = same ? e.fusion_k : 0;
+    inout->tile_m = same ? e.tile_m : 0;
+    bk = bm = 0;
+  }
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tune[tune_key(s->n, s->dt, c)] = {bk, bm};
+  g_tune[tune_key(s->n, s->dt, c)] = {bk, bm, 1};
   tune_save_locked();
   return SV_OK;
 }

@@ -45,3 +45,15 @@ extern "C" int gradient_passes(const sv_circuit *c, const double *params, const 
 }
 
 extern "C" uint64_t reduction_area(int n) { return red_bytes(n); }
+
+// Options a circuit runs with after the autotuner's cache: fusion width, tile
+// size, and whether the tensor-core and permutation paths are open.
+extern "C" void tuned(const sv_circuit *c, int dt, int *out) {
+  sv_state s = host_state(c->n_qubits, dt);
+  Opts o = resolve(&s, nullptr, 1);
+  tuned_options(&s, c, nullptr, o);
+  out[0] = o.fusion_k;
+  out[1] = o.tile_m;
+  out[2] = o.oz;
+  out[3] = o.moves;
+}
