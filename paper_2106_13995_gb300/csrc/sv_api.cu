@@ -1061,7 +1061,7 @@ static bool leaner(const sv_state *s, Opts &o) {
 sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,
                       ProgramRef *out, Opts *o_out, bool basis) {
   if (!s) return set_error(SV_EINVAL, "null state");
-  if (!c) return set_error(SV_EINVAL, "null circuit");
+  SV_TRY(check_circuit(c, s->n));
   Opts o = resolve(s, opt, 1);
   tuned_options(s, c, opt, o);
   o.product = basis && o.moves;

@@ -243,6 +243,9 @@ using AdjSite = std::vector<int>;   // parametric instances, in order
 int gate_arity(int gate);                                    // -1 unknown
 bool gate_matrix(int gate, const double *angles, std::vector<cd> &U);
 int gate_generator(int gate);                                // 1=X 2=Y 3=Z 4=diag(0,-2), 0 none
+// What has to hold before a circuit's arrays are read for a cache key: its
+// width, and the sizes of its matrices.
+sv_status check_circuit(const sv_circuit *c, int n);
 sv_status circuit_to_gates(const sv_circuit *c, const double *params, int n,
                            std::vector<Gate> &out, bool keep_params_unfused);
 std::vector<cd> adjoint_of(const std::vector<cd> &U, int k);
