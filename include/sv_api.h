@@ -233,10 +233,14 @@ sv_status sv_apply_gate(sv_state *s, const int32_t *targets, int k, const int32_
 sv_status sv_apply_circuit(sv_state *s, const sv_circuit *c, const double *params,
                            const sv_options *opt);
 
-/* Report how sv_apply_circuit would execute this circuit with these options:
- * the number of fused blocks and of tile passes (one kernel launch, one read
- * and one write of the state each).  Builds and caches the plan; launches
- * nothing.  Same errors as sv_apply_circuit. */
+/* Report how sv_apply_circuit would execute this circuit with these options
+ * on a state it knows nothing about (on a known basis state, sv_set_basis,
+ * there may be no pass, or a product write in place of the first ones): the
+ * number of fused blocks and of passes, one read and one write of the state
+ * each.  A pass is one kernel launch; that of a permutation run is one per chunk
+ * of 2^22 amplitudes (complex128 2^21, an eighth of a smaller state) and one
+ * more.  Builds and caches the plan; launches nothing.  Same errors as
+ * sv_apply_circuit. */
 sv_status sv_plan_info(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,
                        int64_t *n_blocks, int64_t *n_passes);
 
@@ -244,8 +248,9 @@ sv_status sv_plan_info(sv_state *s, const sv_circuit *c, const double *params, c
  * summed over its fused blocks.  A dense k-qubit block with c controls
  * costs 4 * 2^k / 2^c (each affected amplitude takes 2^k complex
  * multiply-adds of 4 real ones), a diagonal block 4 / 2^c; blocks run on
- * the tensor cores count as dense blocks of the size they run at (split-BF16
- * tile passes pad every block to 5 qubits: 128 each).  This is the work the tile passes'
+ * the tensor cores count as dense blocks of the size they run at (their tile
+ * passes pad every block to 5 qubits: 128 each), gates moved by a permutation
+ * run not at all.  This is the work the tile passes'
  * arithmetic roofline counts (times 2^n amplitudes, 2 flops each).
  *   fma_per_amp: host pointer, receives the sum.
  * Builds and caches the plan; launches nothing.  Same errors as

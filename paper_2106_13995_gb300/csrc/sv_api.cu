@@ -996,6 +996,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
         rest.clear();
         for (const std::vector<Move> &p : passes) emit_moves(out.prog, p, s->n, m, out.op0s);
         std::vector<Block> blocks = fuse(run, o.fusion_k);
+        for (Block &b : blocks) b.kind = TOP_PERM;   // (counted, not multiplied)
         move_to_end(blocks, out.blocks);
         i = e;
         continue;
@@ -1359,7 +1360,8 @@ sv_status sv_plan_fmas(sv_state *s, const sv_circuit *c, const double *params, c
   SV_TRY(get_program(s, c, params, opt, &cp, &o));
   double f = 0;
   for (const Block &b : cp->blocks) {
-    // split-BF16 tile passes run every tensor-core block as a 5-qubit block
+    // tensor-core tile passes (split-BF16, complex128 digits) run every block as
+    // a 5-qubit block
     if (b.kind == TOP_TC) {
       f += 4.0 * 32.0;
       continue;

@@ -57,3 +57,10 @@ extern "C" void tuned(const sv_circuit *c, int dt, int *out) {
   out[2] = o.oz;
   out[3] = o.moves;
 }
+
+// sv_plan_fmas on a host-only state
+extern "C" double plan_fmas(const sv_circuit *c, int dt) {
+  sv_state s = host_state(c->n_qubits, dt);
+  double f = -1;
+  return sv_plan_fmas(&s, c, nullptr, nullptr, &f) == SV_OK ? f : -1;
+}

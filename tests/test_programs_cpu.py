@@ -16,6 +16,7 @@ OZ, MOVES = 0x1000, 0x2000   # kPassOz, kPassMoves
 def tool():
     L = load("program_tool")
     L.program_area.restype = L.reduction_area.restype = C.c_uint64
+    L.plan_fmas.restype = C.c_double
     return L
 
 
@@ -70,6 +71,19 @@ def test_small_state_plans_take_no_more_than_large_tiles(tool, dt):
     large, _ = build(tool, c, dt, sim.options(fusion_k=3, tile_m=13 if dt == SV_C64 else 12))
     small, _ = build(tool, c, dt)
     assert large <= tool.program_area() and small <= tool.program_area()
+
+
+@pytest.mark.parametrize("dt", [SV_C64, SV_C128])
+def test_moved_gates_are_no_arithmetic(tool, dt):
+    """A permutation run adds no multiply-adds to the dense gates around it."""
+    from paper_2106_13995_gb300 import sim
+    n = 24
+    rng = np.random.default_rng(3)
+    head, run = dense(n, 6, 3, rng), toffolis(n, 300, rng)
+    _, flags = build(tool, W.Circuit(n, head + run), dt)
+    assert any(f & MOVES for f in flags)
+    count = [tool.plan_fmas(C.byref(sim.marshal(W.Circuit(n, ops)).c), dt) for ops in (head, head + run, run)]
+    assert count[0] == count[1] > 0 and count[2] == 0
 
 
 # ---- gradients ----------------------------------------------------------------
