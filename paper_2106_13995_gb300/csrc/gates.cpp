@@ -129,7 +129,8 @@ sv_status check_circuit(const sv_circuit *c, int n) {
   return SV_OK;
 }
 
-// Op i of a circuit of the right width, validated.  g's vectors are reused.
+// Op i of a circuit of the right width, validated, into a new gate or over an
+// earlier op's (whose vectors are reused).
 static sv_status op_to_gate(const sv_circuit *c, int i, const double *params, int n, bool keep_params_unfused, Gate &g) {
   const sv_op &op = c->ops[i];
   auto fail = [&](const std::string &what) { return set_error(SV_EINVAL, "op " + std::to_string(i) + ": " + what); };
@@ -141,6 +142,8 @@ static sv_status op_to_gate(const sv_circuit *c, int i, const double *params, in
   uint64_t seen = 0;
   g.targets.clear();
   g.controls.clear();
+  g.param = g.param_gate = -1;
+  g.fixed_structure = false;
   for (int j = 0; j < k + op.n_controls; j++) {
     int q = j < k ? op.targets[j] : op.controls[j - k];
     if (q < 0 || q >= n) return fail("qubit out of range");

@@ -410,7 +410,6 @@ static sv_status emit_sites(DeviceProgram &prog, const Block &blk, const BuildCt
     const int site = j < (int)blk.qubits.size() ? blk.site[j] : -1;
     d.mat[j] = site >= 0 ? b.site_mat[site] : -1;
     if (site < 0) continue;
-    d.any |= 1u << j;
     if (b.site_slot) {
       d.slot[j] = b.site_slot[site];
       d.comps |= (uint32_t)b.site_comps[site] << (4 * j);

@@ -65,7 +65,7 @@ enum TileOpKind : uint8_t {
 struct SitesDesc {
   uint32_t ld[8], st[8];
   int32_t mat[3];
-  uint32_t any;        // targets with a matrix, as a bit mask
+  uint32_t pad;
   int32_t slot[3];
   uint32_t comps;      // 4 bits per target
 };

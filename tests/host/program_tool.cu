@@ -64,3 +64,17 @@ extern "C" double plan_fmas(const sv_circuit *c, int dt) {
   double f = -1;
   return sv_plan_fmas(&s, c, nullptr, nullptr, &f) == SV_OK ? f : -1;
 }
+
+// |index> through the circuit op by op, as sv_apply_circuit follows a known
+// basis state: 1 and the final index and amplitude, 0 when some gate does not
+// keep a basis state, -status on an error.
+extern "C" int follow_basis(const sv_circuit *c, const double *params, uint64_t index, uint64_t *out_index, double *amp) {
+  cd a = 1.0;
+  bool stays = false;
+  const sv_status st = propagate_circuit(c, params, c->n_qubits, index, a, stays);
+  if (st != SV_OK) return -(int)st;
+  *out_index = index;
+  amp[0] = a.real();
+  amp[1] = a.imag();
+  return stays;
+}
