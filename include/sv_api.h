@@ -277,9 +277,10 @@ sv_status sv_plan_fmas(sv_state *s, const sv_circuit *c, const double *params, c
  * and replayed as a CUDA graph from then on.  fusion_k / tile_m left at 0 take the autotuner's cached
  * choice for the circuit's shape, if any.  All states must be distinct and
  * share one stream and device; the first state's workspace holds the batch
- * tables.  Enqueues only (no synchronisation).  Errors: SV_EINVAL (arguments,
- * per-gate mode), SV_ENOMEM (batch tables exceed the first state's reduction
- * area), SV_ECUDA. */
+ * tables, and a batch whose tables do not fit there goes in halves, one after
+ * the other.  Enqueues only (no synchronisation).  Errors: SV_EINVAL (arguments,
+ * per-gate mode), SV_ENOMEM (one state's tables exceed its reduction area),
+ * SV_ECUDA. */
 sv_status sv_apply_circuit_batch(sv_state *const *states, int B, const sv_circuit *const *circs,
                                  const double *const *params, const sv_options *opt);
 

@@ -113,19 +113,15 @@ constexpr size_t kMaxGraphs = 64;
 
 constexpr uint64_t kDefaultSpin = 1ull << 23;   // ~1 s of 128 ns polls
 
-static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *const *circs,
-                           const double *const *params, const sv_options *opt) {
+// The states of a batch, their programs uploaded, in one call.  A batch whose
+// tables outgrow the first state's workspace goes in halves, one after the
+// other, each with the tables in its own first state's.  head: the whole
+// batch's first state, whose error flag a wait that runs out sets.
+static sv_status launch_batch(sv_state *head, sv_state *const *states, int B, const ProgramRef *cps,
+                              const sv_options *opt) {
   sv_state *s0 = states[0];
-  // the programs stay alive for the whole call even if the cache evicts them
-  std::vector<ProgramRef> cps(B);
-  std::vector<Opts> os(B);
   int maxP = 0, m_max = 1;
-  for (int b = 0; b < B; b++) {
-    SV_TRY(get_program(states[b], circs[b], params ? params[b] : nullptr, opt, &cps[b], &os[b]));
-    if (os[b].mode == SV_MODE_PER_GATE) return set_error(SV_EINVAL, "per-gate mode has no batched form");
-    maxP = std::max(maxP, (int)cps[b]->prog.passes.size());
-  }
-  for (int b = 0; b < B; b++) SV_TRY(upload_program(states[b], *cps[b]));
+  for (int b = 0; b < B; b++) maxP = std::max(maxP, (int)cps[b]->prog.passes.size());
   // Wide states run as one ordinary launch per pass, spread over the fan-out
   // streams; the persistent queue is for the rest, whose passes cost less
   // than a launch.  The launches take their matrices from parameter blocks
@@ -257,7 +253,11 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
   const size_t o_ch = take(sizeof(uint32_t) * nd);
   const size_t o_done = take(sizeof(uint32_t) * nd + 2 * sizeof(unsigned long long));
   const size_t total = off;
-  if (total > red_bytes(s0->n)) return set_error(SV_ENOMEM, "batch too large for the first state's workspace");
+  if (total > red_bytes(s0->n)) {
+    if (B == 1) return set_error(SV_ENOMEM, "batch too large for the first state's workspace");
+    SV_TRY(launch_batch(head, states, B / 2, cps, opt));
+    return launch_batch(head, states + B / 2, B - B / 2, cps + B / 2, opt);
+  }
   char *tb = s0->ws + kWsRed;
   SV_TRY(stage_upload_to(s0, tb,
                          {{desc.data(), sizeof(TilePass) * nd}, {first.data(), sizeof(unsigned long long) * nd},
@@ -273,7 +273,7 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
   A.chunk = reinterpret_cast<const uint32_t *>(tb + o_ch);
   A.done = reinterpret_cast<uint32_t *>(tb + o_done);
   A.next_item = reinterpret_cast<unsigned long long *>(tb + o_done + ((sizeof(uint32_t) * nd + 7) & ~(size_t)7));
-  A.err = reinterpret_cast<uint32_t *>(s0->ws + kWsCtrl + kWsErrFlag);
+  A.err = reinterpret_cast<uint32_t *>(head->ws + kWsCtrl + kWsErrFlag);
   A.total_items = items;
   A.ndesc = nd;
   A.spin_limit = (opt && opt->timeout_cycles) ? opt->timeout_cycles : kDefaultSpin;
@@ -290,7 +290,7 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
   // batch layout, then replay
   GraphKey gk;
   gk.first = s0;
-  gk.second.reserve(4 * (size_t)B + 1);
+  gk.second.reserve(4 * (size_t)B + 2);
   for (int b = 0; b < B; b++) {
     gk.second.push_back(cps[b]->serial);
     gk.second.push_back((uint64_t)(uintptr_t)states[b]->amps);
@@ -298,6 +298,7 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
     gk.second.push_back((uint64_t)wide[b]);
   }
   gk.second.push_back(A.spin_limit);
+  gk.second.push_back((uint64_t)(uintptr_t)A.err);
   std::lock_guard<std::mutex> lk(g_graphs_mu);
   auto it = g_graphs.find(gk);
   if (it == g_graphs.end()) {
@@ -338,6 +339,19 @@ static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *con
   SV_CUDA(cudaGraphLaunch(it->second.exec, s0->stream));
   g_launches++;
   return SV_OK;
+}
+
+static sv_status run_batch(sv_state *const *states, int B, const sv_circuit *const *circs,
+                           const double *const *params, const sv_options *opt) {
+  // the programs stay alive for the whole call even if the cache evicts them
+  std::vector<ProgramRef> cps(B);
+  for (int b = 0; b < B; b++) {
+    Opts o;
+    SV_TRY(get_program(states[b], circs[b], params ? params[b] : nullptr, opt, &cps[b], &o));
+    if (o.mode == SV_MODE_PER_GATE) return set_error(SV_EINVAL, "per-gate mode has no batched form");
+  }
+  for (int b = 0; b < B; b++) SV_TRY(upload_program(states[b], *cps[b]));
+  return launch_batch(states[0], states, B, cps.data(), opt);
 }
 
 void drop_graphs(const sv_state *s) {
