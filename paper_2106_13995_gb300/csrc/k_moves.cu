@@ -186,7 +186,7 @@ sv_status launch_moves(sv_state *s, const TilePass &p, cudaStream_t stream) {
 // A permutation of 2^k values as multi-controlled X, appended in order (the
 // transformation-based synthesis of Miller, Maslov and Dueck, DAC 2003: values
 // are put right in increasing order by gates that leave smaller ones alone).
-static void perm_to_moves(const int *perm, int k, const std::vector<int> &q, uint64_t controls, std::vector<Move> &out) {
+void perm_to_moves(const int *perm, int k, const std::vector<int> &q, uint64_t controls, std::vector<Move> &out) {
   std::vector<int> p(perm, perm + (1 << k));
   std::vector<std::pair<int, int>> gates;   // (control mask, target bit), applied to the outputs
   auto apply = [&](int cm, int t) {

@@ -6,6 +6,7 @@
 #include <map>
 #include <tuple>
 
+#include "moves.cuh"
 #include "oz_digits.cuh"
 #include "sv_internal.h"
 
@@ -98,7 +99,7 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
             r.prec == SV_PREC_PLAIN && r.mode != SV_MODE_PER_GATE &&
             s->ws_bytes >= moves_off(s->n) + moves_bytes(s->n, s->dt);
   r.small = r.prec == SV_PREC_PLAIN && nvec == 1 && default_m && !(o && o->fusion_k > 0) &&
-            r.tile_m < std::min(plain64 ? 13 : 12, s->n);
+            r.mode != SV_MODE_PER_GATE && r.tile_m < std::min(plain64 ? 13 : 12, s->n);
   r.L = std::min(r.L, r.tile_m);
   if (s->dt == SV_C64 && r.L < 1) r.L = 1;
   return r;
@@ -260,15 +261,17 @@ void put_pairs_c64(std::vector<uint8_t> &pool, const cd *U, int k) {
 // global qubit positions[8], 4 bytes padding, then 2^g tables of 2^m uint16
 // (table v serves the tiles whose global control qubits read v's bits).
 // Returns false (nothing appended) if the pass does not qualify.
+//
+// A table is composed on bit planes, as the kernel of permutation runs does it:
+// plane i holds bit i of where 64 amplitudes at a time have got to, a block is a
+// few multi-controlled X, and each is an AND and an XOR of words.  (Amplitude by
+// amplitude the tables were nearly all of a circuit's first pass.)
 static bool table_pass(const PassPlan &P, const BuildCtx &b, const int *loc, int m, std::vector<uint8_t> &pool,
                        uint32_t &mat0) {
   if (b.nvec != 1 || m > 16 || P.ops.empty()) return false;
   struct PB {
-    uint32_t lc = 0, tmask = 0;
-    uint64_t gc = 0;
-    int k = 0;
-    int t[6];
-    int perm[64];
+    uint64_t gc = 0;           // control qubits outside the tile
+    std::vector<Move> moves;   // on tile positions
   };
   std::vector<PB> pbs;
   uint64_t gall = 0;
@@ -277,22 +280,24 @@ static bool table_pass(const PassPlan &P, const BuildCtx &b, const int *loc, int
         blk.xmask || blk.qubits.size() > 6)
       return false;
     PB pb;
-    pb.k = (int)blk.qubits.size();
-    if (!permutation_of(blk.U, pb.k, pb.perm)) return false;
-    for (int j = 0; j < pb.k; j++) {
-      if (loc[blk.qubits[j]] < 0) return false;
-      pb.t[j] = loc[blk.qubits[j]];
-      pb.tmask |= 1u << pb.t[j];
+    int perm[64];
+    if (!permutation_of(blk.U, (int)blk.qubits.size(), perm)) return false;
+    std::vector<int> t;
+    for (int q : blk.qubits) {
+      if (loc[q] < 0) return false;
+      t.push_back(loc[q]);
     }
+    uint64_t lc = 0;
     for (int q : blk.controls) {
-      if (loc[q] >= 0) pb.lc |= 1u << loc[q];
+      if (loc[q] >= 0) lc |= 1ull << loc[q];
       else pb.gc |= 1ull << q;
     }
+    perm_to_moves(perm, (int)t.size(), t, lc, pb.moves);
     gall |= pb.gc;
-    pbs.push_back(pb);
+    pbs.push_back(std::move(pb));
   }
   const int g = __builtin_popcountll(gall);
-  const uint32_t N = 1u << m;
+  const uint32_t N = 1u << m, words = std::max(1u, N / 64);
   const size_t bytes = 16 + ((size_t)N << g) * sizeof(uint16_t);
   // at most 5 global control qubits, and tables take at most half the
   // workspace's program area
@@ -302,30 +307,37 @@ static bool table_pass(const PassPlan &P, const BuildCtx &b, const int *loc, int
     int i = 0;
     for (uint64_t x = gall; x; x &= x - 1) gq[i++] = __builtin_ctzll(x);
   }
-  std::vector<uint32_t> x(N);
+  std::vector<uint64_t> planes((size_t)m * words), on(words);
   std::vector<uint16_t> tab((size_t)N << g);
   for (uint32_t v = 0; v < (1u << g); v++) {
     uint64_t gset = 0;
     for (int i = 0; i < g; i++)
       if ((v >> i) & 1u) gset |= 1ull << gq[i];
-    for (uint32_t l = 0; l < N; l++) x[l] = l;
+    for (int i = 0; i < m; i++)
+      for (uint32_t w = 0; w < words; w++)
+        planes[(size_t)i * words + w] = i >= 6              ? ((w >> (i - 6)) & 1u ? ~0ull : 0ull)
+                                        : i == 5            ? 0xffffffff00000000ull
+                                                            : word_pattern(i) * 0x100000001ull;
     for (const PB &pb : pbs) {
       if (pb.gc & ~gset) continue;   // a global control reads 0 in these tiles
-      for (uint32_t l = 0; l < N; l++) {
-        const uint32_t xv = x[l];
-        if ((xv & pb.lc) != pb.lc) continue;
-        int c = 0;
-        for (int j = 0; j < pb.k; j++) c |= (int)((xv >> pb.t[j]) & 1u) << j;
-        const int r = pb.perm[c];
-        if (r == c) continue;
-        uint32_t nv = xv & ~pb.tmask;
-        for (int j = 0; j < pb.k; j++) nv |= (uint32_t)((r >> j) & 1) << pb.t[j];
-        x[l] = nv;
+      for (const Move &mv : pb.moves) {
+        std::fill(on.begin(), on.end(), ~0ull);
+        for (uint64_t c = mv.controls; c; c &= c - 1) {
+          const uint64_t *p = &planes[(size_t)__builtin_ctzll(c) * words];
+          for (uint32_t w = 0; w < words; w++) on[w] &= p[w];
+        }
+        uint64_t *p = &planes[(size_t)mv.target * words];
+        for (uint32_t w = 0; w < words; w++) p[w] ^= on[w];
       }
     }
-    // the amplitude at tile slot l ends at x[l]: gather out[x[l]] = in[l]
+    // the amplitude at tile slot l ends at x: gather out[x] = in[l]
     uint16_t *t = tab.data() + (size_t)v * N;
-    for (uint32_t l = 0; l < N; l++) t[x[l]] = (uint16_t)l;
+    for (uint32_t l0 = 0; l0 < N; l0 += 32) {
+      uint32_t x[32] = {0};
+      for (int i = 0; i < m; i++) x[i] = (uint32_t)(planes[(size_t)i * words + l0 / 64] >> (l0 & 63u));
+      transpose32(x);
+      for (uint32_t l = l0; l < std::min(N, l0 + 32); l++) t[x[l - l0]] = (uint16_t)l;
+    }
   }
   while (pool.size() % 16) pool.push_back(0);
   mat0 = (uint32_t)(pool.size() / 16);
@@ -806,11 +818,42 @@ static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates,
   return true;
 }
 
+// The options with the tiles and fusion width of large states.
+static Opts large_tiles(const sv_state *s, const Opts &o) {
+  Opts r = o;
+  r.small = 0;
+  r.fusion_k = 3;
+  r.tile_m = std::min(s->dt == SV_C64 ? 13 : 12, s->n);
+  r.L = std::min(3, r.tile_m);
+  return r;
+}
+
+// complex128 blocks of 4 and more qubits leave most threads of a 7- or 8-qubit
+// tile without a group; from 17 qubits on, where that is no longer hidden, a
+// circuit that does most of its arithmetic in them takes large tiles (20 dense
+// 5-qubit blocks: 16 qubits 3149 us against 3139, 17 qubits 4615 against 3129, 20
+// qubits 18.2 ms against 6.2).
+static bool wide_blocks(const sv_state *s, const std::vector<Block> &blocks) {
+  if (s->dt != SV_C128 || s->n < 17) return false;
+  double wide = 0, all = 0;
+  for (const Block &b : blocks) {
+    const double f = b.diag ? 1.0 : std::ldexp(1.0, (int)b.qubits.size());
+    all += f;
+    if (b.qubits.size() >= 4 && !b.diag) wide += f;
+  }
+  return 2 * wide > all;
+}
+
 // Append a program of tile passes for `gates` to `out` (its layout is left to
 // the caller).
 static sv_status append_gates(sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
   if (o.oz && append_oz_program(s, gates, o, out)) return SV_OK;
   std::vector<Block> blocks = fuse(gates, o.fusion_k);
+  if (o.small && wide_blocks(s, blocks)) {
+    Opts l = large_tiles(s, o);
+    l.oz = 0;
+    return append_gates(s, gates, l, out);
+  }
   if (o.mode == SV_MODE_PER_GATE) {
     out.blocks = std::move(blocks);
     return SV_OK;
@@ -935,6 +978,56 @@ static size_t count_passes(const sv_state *s, const std::vector<Gate> &gates, co
   return plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass).size();
 }
 
+// Small states: about how long a permutation run takes as tile passes, in us.  A
+// gather table takes one launch's time whatever it holds, and a larger tile holds
+// more gates (of random Toffolis, complex64, 11 qubits: 19 at 7.4 us, 13 qubits: 28
+// at 8.3; complex128, 7 qubits: 8 at 3.8 to 5, 12 qubits: 24 at 7.6); passes that
+// table_pass turns down go gate by gate.  used: bytes of the matrix pool before it.
+static double run_us(const sv_state *s, const std::vector<Gate> &run, const Opts &o, size_t used) {
+  const bool c64 = s->dt == SV_C64, large = o.tile_m >= (c64 ? 13 : 12);
+  const std::vector<Block> blocks = fuse(run, o.fusion_k);
+  int m = o.tile_m, L = o.L;
+  if (!fit_tile(blocks, s->n, lmin(s->dt), mmax(s->dt, 1), m, L)) return HUGE_VAL;
+  double us = 0;
+  for (const PassPlan &P : plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass)) {
+    uint64_t tile = 0, controls = 0;
+    for (int q : P.S) tile |= 1ull << q;
+    for (const Block &b : P.ops)
+      for (int q : b.controls) controls |= 1ull << q;
+    const int g = __builtin_popcountll(controls & ~tile);
+    const size_t bytes = ((size_t)2 << (m + std::min(g, 6)));
+    us += std::ldexp(2.0 * (double)amp_bytes(s->dt), s->n) / 2.5e6;
+    if (g <= 5 && used + bytes <= kWsProgBytes / 2) {
+      used += bytes;
+      us += c64 ? (large ? 8.2 : 7.2) : (large ? 7.6 : 4.2);
+    } else {
+      us += 4.0 + (double)P.ops.size() * (c64 ? (large ? 0.92 : 0.55) : (large ? 1.28 : 0.45));
+    }
+  }
+  return us;
+}
+static double moves_us(const sv_state *s, size_t passes) {
+  return (double)passes * (33.0 + std::ldexp((double)amp_bytes(s->dt), s->n) * 1.6e-6);
+}
+
+// How a run of permutation gates on a small state goes: with the gates around it
+// in small tiles, in large tiles of its own, or as `passes` passes of moves (0: no
+// moves), whichever is fastest.  whole: the run is the whole circuit; else its ends
+// cost passes that it would share with the gates around it, and short runs stay
+// with those.  used: bytes of the pool before it.  Random Toffolis on a dense state,
+// against small tiles or moves: complex64, 12 qubits, 300 of them 16 us and 74, 16
+// qubits 100 and 140; complex128, 12 qubits 16 and 149, 16 qubits 116 and 370.
+enum class Run { kWithRest, kLarge, kMoves };
+static Run small_run(const sv_state *s, const std::vector<Gate> &run, size_t passes, bool whole, const Opts &o,
+                     size_t used) {
+  if (!whole && count_passes(s, run, o) < 6) return Run::kWithRest;
+  // (large tables take longer to compose: not for a few percent)
+  const double small = run_us(s, run, o, used), large = 1.15 * run_us(s, run, large_tiles(s, o), used);
+  const double ends = whole ? 0 : 8.0, moved = passes ? moves_us(s, passes) : HUGE_VAL;
+  if (std::min(large, moved) + ends >= small) return Run::kWithRest;
+  return large <= moved ? Run::kLarge : Run::kMoves;
+}
+
 // Single-qubit gates in front of everything else, on a known basis state, as a
 // product pass; false: nothing appended.
 static bool append_product(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, CachedProgram &out) {
@@ -962,7 +1055,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
   std::vector<Gate> rest;   // gates not yet in the program
   size_t i = 0;
   const int m = moves_m(s->n, s->dt);
-  while (o.moves && i < gates.size()) {
+  while ((o.moves || o.small) && i < gates.size()) {
     std::vector<Move> moves;
     size_t e = i;
     // (a plain X that comes first on its qubit goes with the gates before the
@@ -986,17 +1079,31 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
       }
     }
     if (run.size() >= kMovesMinGates) {
-      const std::vector<std::vector<Move>> passes = plan_moves(moves, m);
+      const std::vector<std::vector<Move>> passes = o.moves ? plan_moves(moves, m) : std::vector<std::vector<Move>>();
       // (at most 9 ops of 16 bytes a move, 8 of them for many controls)
-      const bool fits = out.prog.mats.size() + 9 * 16 * moves.size() + 256 * passes.size() <= kWsProgBytes / 2;
-      if (fits && count_passes(s, run, o) >= moves_worth(s->n) * passes.size()) {
+      const bool fits =
+          o.moves && out.prog.mats.size() + 9 * 16 * moves.size() + 256 * passes.size() <= kWsProgBytes / 2;
+      Run route = Run::kWithRest;
+      if (o.small) {
+        const bool whole = rest.empty() && before.empty() && out.prog.passes.empty() && e == gates.size();
+        route = small_run(s, run, fits ? passes.size() : 0, whole, o, out.prog.mats.size());
+      } else if (fits && count_passes(s, run, o) >= moves_worth(s->n) * passes.size()) {
+        route = Run::kMoves;
+      }
+      if (route != Run::kWithRest) {
         rest.insert(rest.end(), before.begin(), before.end());
         if (!rest.empty() && !append_product(s, rest, o, out)) SV_TRY(append_gates(s, rest, o, out));
         rest.clear();
-        for (const std::vector<Move> &p : passes) emit_moves(out.prog, p, s->n, m, out.op0s);
-        std::vector<Block> blocks = fuse(run, o.fusion_k);
-        for (Block &b : blocks) b.kind = TOP_PERM;   // (counted, not multiplied)
-        move_to_end(blocks, out.blocks);
+        if (route == Run::kLarge) {
+          Opts l = large_tiles(s, o);
+          l.oz = 0;
+          SV_TRY(append_gates(s, run, l, out));
+        } else {
+          for (const std::vector<Move> &p : passes) emit_moves(out.prog, p, s->n, m, out.op0s);
+          std::vector<Block> blocks = fuse(run, o.fusion_k);
+          for (Block &b : blocks) b.kind = TOP_PERM;   // (counted, not multiplied)
+          move_to_end(blocks, out.blocks);
+        }
         i = e;
         continue;
       }
@@ -1005,7 +1112,7 @@ static sv_status build_circuit_program(sv_state *s, const std::vector<Gate> &gat
     rest.insert(rest.end(), gates.begin() + i, gates.begin() + e);
     i = e;
   }
-  if (!o.moves) SV_TRY(append_gates(s, gates, o, out));
+  if (!o.moves && !o.small) SV_TRY(append_gates(s, gates, o, out));
   else if (!rest.empty()) SV_TRY(append_gates(s, rest, o, out));
   out.lay = layout_of(out.prog, 0, 0);
   return SV_OK;
@@ -1048,10 +1155,7 @@ static bool leaner(const sv_state *s, Opts &o) {
   } else if (o.moves) {
     o.moves = o.product = 0;
   } else if (o.small) {
-    o.small = 0;
-    o.fusion_k = 3;
-    o.tile_m = std::min(s->dt == SV_C64 ? 13 : 12, s->n);
-    o.L = std::min(3, o.tile_m);
+    o = large_tiles(s, o);
   } else {
     return false;
   }
@@ -1077,6 +1181,7 @@ sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, co
   k.val(o.oz);
   k.val(o.moves);
   k.val(o.product);
+  k.val(o.small);
   k.val((int)s->dt);
   if (params && c->n_params > 0) k.bytes(params, sizeof(double) * c->n_params);
   const uint64_t h = k.hash();

@@ -420,6 +420,8 @@ struct Move {             // X on `target` where all of `controls` are 1
   uint64_t controls;
   int target;
 };
+// Append a permutation of 2^k values on bits q, under controls, as moves.
+void perm_to_moves(const int *perm, int k, const std::vector<int> &q, uint64_t controls, std::vector<Move> &out);
 // Append a gate as moves if it is a fixed permutation of at most 3 targets.
 bool gate_moves(const Gate &g, std::vector<Move> &out);
 std::vector<std::vector<Move>> plan_moves(const std::vector<Move> &moves, int m);
