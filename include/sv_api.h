@@ -261,7 +261,8 @@ sv_status sv_plan_fmas(sv_state *s, const sv_circuit *c, const double *params, c
 /* Apply circs[b] (with parameters params[b], host FP64, either may repeat)
  * to states[b] for b < B, states of any widths, in one call: every circuit
  * is fused and planned into tile passes as by sv_apply_circuit.  The narrow
- * states (below 19 qubits, below 14 when replayed from a graph) go through ONE
+ * states (below 18 qubits, complex128 below 15; replayed from a graph below 14,
+ * below 16 where the batch has more than 40 of 14 and 15) go through ONE
  * persistent launch: a cooperative kernel works through the queue of all
  * their (state, pass, tile) items in pass order, a tile of pass p waiting
  * until pass p-1 of its own state is complete (Sec. I motivates many

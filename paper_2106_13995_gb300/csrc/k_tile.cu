@@ -559,14 +559,19 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
   return SV_OK;
 }
 
-sv_status launch_tile_persist(sv_state *s, const PersistArgs &A, int m_max, int *grid_out, cudaStream_t st) {
+sv_status launch_tile_persist(sv_state *s, const PersistArgs &A, int m_max, uint64_t wave, int *grid_out, cudaStream_t st) {
   const size_t smem = tile_smem(s->dt, m_max, 1);
   if (smem > (200u << 10)) return set_error(SV_EINVAL, "tile too large for shared memory");
   const void *fn = s->dt == SV_C64 ? (const void *)k_tile_persist<float> : (const void *)k_tile_persist<double>;
   SV_TRY(func_attr_once(fn, s->device, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10));
   // 16 amplitudes a thread: smaller tiles take smaller CTAs and more of them,
-  // so the items of many states are in flight at once
-  const int threads = std::max(128, std::min(kTileMaxThreads, 1 << std::max(0, m_max - 4)));
+  // so the items of many states are in flight at once.  The 7- and 8-qubit tiles of
+  // complex128 states keep 32 or 64 of 128 threads busy; once the states' tiles
+  // outnumber twice the CTAs of 128, CTAs of 64 and twice as many of them are faster
+  // (40 layers of U3 + CZ: 256 states of 12 qubits 10.1 ms to 7.7, of 14 qubits 42.9
+  // to 31.9; 16 of 12 qubits 1.36 to 1.46)
+  int threads = std::max(128, std::min(kTileMaxThreads, 1 << std::max(0, m_max - 4)));
+  if (s->dt == SV_C128 && m_max <= 8 && wave > 16ull * (unsigned)s->sm_count) threads = 64;
   int per_sm = 0;
   SV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
   if (per_sm < 1) return set_error(SV_EUNSUPPORTED, "persistent tile kernel does not fit on an SM");

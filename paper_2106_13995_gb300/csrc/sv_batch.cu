@@ -126,19 +126,26 @@ static sv_status launch_batch(sv_state *head, sv_state *const *states, int B, co
   // streams; the persistent queue is for the rest, whose passes cost less
   // than a launch.  The launches take their matrices from parameter blocks
   // and overlap freely; the queue's tile body reads them from memory and
-  // waits between passes.  48 circuits of depth 40 replayed from a graph:
-  // 20 qubits 40.7 ms in the queue, 18.1 as launches, 17-18 qubits 7.1 and
-  // 4.2, 14-16 qubits 1.84 and 1.97 (but 8.5 and 6.3 for 10-22 qubits
-  // together), 10-13 qubits 1.13 and 1.25.  Without a graph each launch costs
-  // the host 4-5 us, as much as a pass of 19 qubits.
-  const int wide_n = opt && opt->mode == SV_MODE_TILED_GRAPH ? 14 : 19;
+  // waits between passes.  Without a graph each launch costs the host 4-5 us
+  // (40 layers of U3 + CZ, in the queue and as launches, ms: complex64, 16 states
+  // of 18 qubits 3.9 and 1.9, 64 of 17 5.7 and 5.8, 64 of 16 2.9 and 5.4;
+  // complex128, 64 states of 16 qubits 36 and 34, 16 of 15 6.8 and 4.3, 64 of 14 8.2
+  // and 10.7).  Replayed from a graph a launch costs about 1.2 us, which the
+  // narrowest states save only while few of them wait for each other (16, 48 and
+  // 128 states of 14 qubits 0.97 and 0.47, 1.18 and 1.37, 2.1 and 3.7; of 15 qubits
+  // 1.1 and 0.49, 1.42 and 1.45, 2.7 and 3.9; of 16 qubits 1.5 and 0.66, 2.2 and
+  // 1.9, 5.9 and 5.2; 10-13 qubits 1.13 and 1.25 for 48 circuits).
+  int mid = 0;   // states of 14 and 15 qubits
+  for (int b = 0; b < B; b++) mid += states[b]->n == 14 || states[b]->n == 15;
+  const bool graphed = opt && opt->mode == SV_MODE_TILED_GRAPH;
+  auto wide_n = [&](const sv_state *s) { return graphed ? (mid <= 40 ? 14 : 16) : s->dt == SV_C64 ? 18 : 15; };
   std::vector<char> wide(B, 0);
   for (int b = 0; b < B; b++) {
     bool has_tc = false;
     // (tensor-core and permutation passes have kernels of their own, which
     // the persistent queue does not run)
     for (const TilePass &tp : cps[b]->prog.passes) has_tc |= (tp.flags & (kPassTC | kPassHasTC | kPassTable | kPassOz | kPassMoves)) != 0;
-    wide[b] = !cps[b]->prog.passes.empty() && (has_tc || states[b]->n >= wide_n);
+    wide[b] = !cps[b]->prog.passes.empty() && (has_tc || states[b]->n >= wide_n(states[b]));
     if (!wide[b])
       for (const TilePass &tp : cps[b]->prog.passes) m_max = std::max(m_max, tp.m);
   }
@@ -148,7 +155,7 @@ static sv_status launch_batch(sv_state *head, sv_state *const *states, int B, co
   std::vector<int32_t> dep;
   std::vector<uint32_t> ntiles, chunk;
   std::vector<int> last_desc(B, -1);
-  unsigned long long items = 0;
+  unsigned long long items = 0, wave = 0;   // wave: tiles of the states' first passes
   for (int p = 0; p < maxP; p++)
     for (int b = 0; b < B; b++) {
       const CachedProgram &cp = *cps[b];
@@ -170,6 +177,7 @@ static sv_status launch_batch(sv_state *head, sv_state *const *states, int B, co
       chunk.push_back(ch);
       last_desc[b] = (int)desc.size() - 1;
       items += (nt + ch - 1) / ch;
+      if (p == 0) wave += nt;
     }
   const uint32_t nd = (uint32_t)desc.size();
   // The wide states' passes, as ordinary launches.  The states are
@@ -281,7 +289,7 @@ static sv_status launch_batch(sv_state *head, sv_state *const *states, int B, co
   auto record = [&](cudaStream_t st) -> sv_status {
     if (nd > 0) {
       SV_CUDA(cudaMemsetAsync(tb + o_done, 0, zero_bytes, st));
-      SV_TRY(launch_tile_persist(s0, A, m_max, nullptr, st));
+      SV_TRY(launch_tile_persist(s0, A, m_max, wave, nullptr, st));
     }
     return launch_wide(st);
   };

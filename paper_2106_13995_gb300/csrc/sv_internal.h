@@ -641,7 +641,7 @@ sv_status launch_dense_tc6(sv_state *s, void *amps, const int *targets, const ui
 // one pass of a program (tile pass or tensor-core block) on stream st
 sv_status launch_any_pass(sv_state *s, const TilePass &tp, int batch, cudaStream_t st,
                           const HostPass *host = nullptr);
-sv_status launch_tile_persist(sv_state *s, const PersistArgs &A, int m_max, int *grid_out, cudaStream_t st);
+sv_status launch_tile_persist(sv_state *s, const PersistArgs &A, int m_max, uint64_t wave, int *grid_out, cudaStream_t st);
 sv_status launch_wait_selftest(cudaStream_t st, const uint32_t *never, uint32_t *err, uint64_t limit);
 int tile_threads(int m, sv_dtype dt);
 size_t tile_smem(sv_dtype dt, int m, int nvec);
