@@ -419,6 +419,20 @@ static int pass_threads(const sv_state *s, int m, int nvec, uint64_t tiles) {
   return t;
 }
 
+// Shared memory to ask for so that no SM takes more than its share of a pass's
+// tiles.  The CTAs of a programmatic launch start while the pass before it drains,
+// on the SMs that happen to be free, up to as many as fit: passes of one to a few
+// tiles per SM then took as long as the fullest SM (three tiles of 256, where two a
+// SM is the share: 21 qubits, complex64, QFT 1004 us, 828 with ordinary launches
+// and 813 so; U3 + CZ on 18 qubits, 40 layers, complex64 316 us to 289, complex128
+// 3.78 ms to 2.96; 20 dense 5-qubit blocks, 20 qubits, complex128 6.2 ms to 5.3).
+// Only on the state's own stream: a batch's streams share the SMs.
+static size_t share_smem(const sv_state *s, size_t smem, uint64_t tiles, cudaStream_t stream) {
+  const uint64_t sms = (uint64_t)s->sm_count, share = (tiles + sms - 1) / sms;
+  if (stream != s->stream || 2 * tiles <= sms || share > 16) return smem;
+  return std::max(smem, (((size_t)227 << 10) / (size_t)(share + 1)) & ~(size_t)127);
+}
+
 size_t tile_smem(sv_dtype dt, int m, int nvec) { return (size_t)nvec * ((size_t)1 << m) * amp_bytes(dt); }
 
 
@@ -543,18 +557,19 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
   }
   if (smem > (200u << 10)) return set_error(SV_EINVAL, "tile too large for shared memory");
   dim3 grid((unsigned)(1ull << (p.n - p.m)), (unsigned)batch);
+  const size_t smem_cta = share_smem(s, smem, (uint64_t)grid.x * grid.y, stream);
   const int threads = pass_threads(s, p.m, (int)p.nvec, (uint64_t)grid.x * grid.y);
   if (host && sites_pass_ok(p, *host)) return launch_tile_sites(s, p, batch, threads, stream);
   sv_status st = SV_OK;
   const bool try_inl = host && s->dt == SV_C64 && batch == 1 && p.nvec == 1 && !(p.flags & kPassNorm);
-  if (try_inl && (launch_inl<TileInlineSmall>(s, p, *host, grid, threads, smem, stream, st) ||
-                  launch_inl<TileInlineMid>(s, p, *host, grid, threads, smem, stream, st) ||
-                  launch_inl<TileInline>(s, p, *host, grid, threads, smem, stream, st)))
+  if (try_inl && (launch_inl<TileInlineSmall>(s, p, *host, grid, threads, smem_cta, stream, st) ||
+                  launch_inl<TileInlineMid>(s, p, *host, grid, threads, smem_cta, stream, st) ||
+                  launch_inl<TileInline>(s, p, *host, grid, threads, smem_cta, stream, st)))
     SV_TRY(st);
   else if (s->dt == SV_C64)
-    SV_CUDA(launch_early(k_tile<float>, grid, threads, smem, stream, p));
+    SV_CUDA(launch_early(k_tile<float>, grid, threads, smem_cta, stream, p));
   else
-    SV_CUDA(launch_early(k_tile<double>, grid, threads, smem, stream, p));
+    SV_CUDA(launch_early(k_tile<double>, grid, threads, smem_cta, stream, p));
   g_launches++;
   return SV_OK;
 }

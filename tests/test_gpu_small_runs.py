@@ -36,3 +36,14 @@ def test_wide_blocks(svlib, oracle, n):
     want = oracle.run(c, psi)
     assert np.max(np.abs(s.load(psi).apply_circuit(c).numpy() - want)) <= 1e-13 * np.max(np.abs(want))
     s.close()
+
+
+@pytest.mark.parametrize("n", [18, 19, 20, 21])
+@pytest.mark.parametrize("dt", ["c64", "c128"])
+def test_tiles_from_one_to_many_per_sm(svlib, oracle, dt, n):
+    """Passes whose CTAs are held to their share of each SM, twice in a row."""
+    c = W.random_u3_cz(n, 3, n)
+    s = svlib.StateVector(n, dt).set_basis(0).apply_circuit(c).apply_circuit(c)
+    want = oracle.run(c, oracle.run(c))
+    assert np.max(np.abs(s.numpy() - want)) <= (1e-5 if dt == "c64" else 1e-13) * np.max(np.abs(want))
+    s.close()
