@@ -118,14 +118,28 @@ std::vector<cd> adjoint_of(const std::vector<cd> &U, int k) {
   return A;
 }
 
-sv_status check_circuit(const sv_circuit *c, int n) {
+static sv_status check_width(const sv_circuit *c, int n) {
   if (!c || (c->n_ops > 0 && !c->ops)) return set_error(SV_EINVAL, "null circuit");
   if (c->n_qubits != n)
     return set_error(SV_EINVAL, "circuit width " + std::to_string(c->n_qubits) +
                                     " does not match the state's " + std::to_string(n));
+  return SV_OK;
+}
+
+sv_status circuit_key(KeyBytes &k, const sv_circuit *c, int n) {
+  SV_TRY(check_width(c, n));
+  k.b.reserve(k.b.size() + sizeof(sv_op) * (size_t)std::max(0, c->n_ops) + sizeof(double) * (size_t)std::max(0, c->n_params) + 256);
+  k.val(c->n_qubits);
+  k.val(c->n_ops);
+  k.val(c->n_params);
+  if (c->n_ops > 0) k.bytes(c->ops, sizeof(sv_op) * (size_t)c->n_ops);
   for (int i = 0; i < c->n_ops; i++)
-    if (c->ops[i].gate == SV_GATE_MATRIX && (c->ops[i].n_targets < 1 || c->ops[i].n_targets > 6))
-      return set_error(SV_EINVAL, "op " + std::to_string(i) + ": wrong number of targets");
+    if (c->ops[i].gate == SV_GATE_MATRIX) {
+      const int t = c->ops[i].n_targets;
+      if (t < 1 || t > 6) return set_error(SV_EINVAL, "op " + std::to_string(i) + ": wrong number of targets");
+      if (c->matrices && c->ops[i].matrix_offset >= 0)
+        k.bytes(c->matrices + 2 * c->ops[i].matrix_offset, sizeof(double) * 2 << (2 * t));
+    }
   return SV_OK;
 }
 
@@ -176,7 +190,7 @@ static sv_status op_to_gate(const sv_circuit *c, int i, const double *params, in
 
 sv_status circuit_to_gates(const sv_circuit *c, const double *params, int n,
                            std::vector<Gate> &out, bool keep_params_unfused) {
-  SV_TRY(check_circuit(c, n));
+  SV_TRY(check_width(c, n));
   out.clear();
   out.reserve(c->n_ops);
   for (int i = 0; i < c->n_ops; i++) {
@@ -244,7 +258,7 @@ bool propagate_basis(const std::vector<Gate> &gates, uint64_t &index, cd &amp) {
 // converted one at a time: converting all of them cost a call on a small state
 // more than its launches (1080 gates: about 100 us).
 sv_status propagate_circuit(const sv_circuit *c, const double *params, int n, uint64_t &index, cd &amp, bool &stays) {
-  SV_TRY(check_circuit(c, n));
+  SV_TRY(check_width(c, n));
   stays = false;
   Gate g;
   for (int i = 0; i < c->n_ops; i++) {

@@ -343,7 +343,6 @@ static sv_status check_batch(sv_state *const *psi, int B, int n, sv_dtype dt, cu
 static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double *params, const sv_pauli_term *terms,
                                  int nt, const sv_options *opt, int B, bool lean,
                                  std::shared_ptr<const AdjointProgram> &Ap) {
-  SV_TRY(check_circuit(c, s->n));
   Opts o1 = resolve(s, opt, 1), o2 = resolve(s, opt, 2);
   // defaults for the gradient program (measured on the 20-qubit, 64-set
   // ansatz): fusion width 2 and 12-qubit tiles for both sweeps
@@ -361,7 +360,7 @@ static sv_status adjoint_program(sv_state *s, const sv_circuit *c, const double 
   // per-batch matrices, uploaded every call)
   KeyBytes k;
   k.val((int)0xad);
-  circuit_key(k, c);
+  SV_TRY(circuit_key(k, c, s->n));
   if (nt) k.bytes(terms, sizeof(sv_pauli_term) * nt);
   k.val(o1);
   k.val(o2);

@@ -139,19 +139,6 @@ uint64_t KeyBytes::hash() const {
   return h ^ (h >> 31);
 }
 
-void circuit_key(KeyBytes &k, const sv_circuit *c) {
-  k.b.reserve(k.b.size() + sizeof(sv_op) * (size_t)std::max(0, c->n_ops) + sizeof(double) * (size_t)std::max(0, c->n_params) + 256);
-  k.val(c->n_qubits);
-  k.val(c->n_ops);
-  k.val(c->n_params);
-  if (c->n_ops > 0) k.bytes(c->ops, sizeof(sv_op) * (size_t)c->n_ops);
-  for (int i = 0; i < c->n_ops; i++)
-    if (c->ops[i].gate == SV_GATE_MATRIX && c->matrices && c->ops[i].matrix_offset >= 0) {
-      const int d = 1 << c->ops[i].n_targets;
-      k.bytes(c->matrices + 2 * c->ops[i].matrix_offset, sizeof(double) * 2 * d * d);
-    }
-}
-
 static std::atomic<uint64_t> g_serial{0};
 uint64_t next_program_serial() { return ++g_serial; }
 
@@ -1165,13 +1152,12 @@ static bool leaner(const sv_state *s, Opts &o) {
 sv_status get_program(sv_state *s, const sv_circuit *c, const double *params, const sv_options *opt,
                       ProgramRef *out, Opts *o_out, bool basis) {
   if (!s) return set_error(SV_EINVAL, "null state");
-  SV_TRY(check_circuit(c, s->n));
+  KeyBytes k;
+  k.val((int)0x51);
+  SV_TRY(circuit_key(k, c, s->n));
   Opts o = resolve(s, opt, 1);
   tuned_options(s, c, opt, o);
   o.product = basis && o.moves;
-  KeyBytes k;
-  k.val((int)0x51);
-  circuit_key(k, c);
   k.val(o.fusion_k);
   k.val(o.tile_m);
   k.val(o.L);

@@ -243,9 +243,6 @@ using AdjSite = std::vector<int>;   // parametric instances, in order
 int gate_arity(int gate);                                    // -1 unknown
 bool gate_matrix(int gate, const double *angles, std::vector<cd> &U);
 int gate_generator(int gate);                                // 1=X 2=Y 3=Z 4=diag(0,-2), 0 none
-// What has to hold before a circuit's arrays are read for a cache key: its
-// width, and the sizes of its matrices.
-sv_status check_circuit(const sv_circuit *c, int n);
 sv_status circuit_to_gates(const sv_circuit *c, const double *params, int n,
                            std::vector<Gate> &out, bool keep_params_unfused);
 std::vector<cd> adjoint_of(const std::vector<cd> &U, int k);
@@ -448,8 +445,9 @@ struct KeyBytes {
   template <typename T> void val(const T &v) { bytes(&v, sizeof(T)); }
   uint64_t hash() const;
 };
-// key material of a circuit (ops, the matrices its MATRIX ops use)
-void circuit_key(KeyBytes &k, const sv_circuit *c);
+// key material of a circuit (ops, the matrices its MATRIX ops use); its width and
+// the sizes of its matrices are checked before they are read
+sv_status circuit_key(KeyBytes &k, const sv_circuit *c, int n);
 uint64_t next_program_serial();
 
 // A bounded, thread-safe cache of immutable programs per state handle.
