@@ -728,6 +728,30 @@ static void move_to_end(std::vector<Block> &from, std::vector<Block> &to) {
   to.insert(to.end(), std::make_move_iterator(from.begin()), std::make_move_iterator(from.end()));
 }
 
+// Circuits that mostly move amplitudes (a GHZ state, X layers before a few dense
+// gates): a tensor-core block takes its time whatever it does, 10 us a tile and SM,
+// FP64 arithmetic only that of the blocks that are no permutations (GHZ of 14
+// qubits 43 us against 16, of 22 qubits 431 against 298).  Weighed where three fifths
+// of the gates are permutations.
+static bool mostly_moves(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, size_t oz_blocks) {
+  int perm[64];
+  size_t n_perm = 0;
+  for (const Gate &g : gates) n_perm += permutation_of(g.U, (int)g.targets.size(), perm) ? 1 : 0;
+  if (5 * n_perm < 3 * gates.size()) return false;
+  const std::vector<Block> blocks = fuse(gates, o.fusion_k);
+  int m = o.tile_m, L = o.L;
+  if (!fit_tile(blocks, s->n, lmin(s->dt), mmax(s->dt, 1), m, L)) return false;
+  double fmas = 0;
+  for (const Block &b : blocks)
+    if (!permutation_of(b.U, (int)b.qubits.size(), perm))
+      fmas += b.diag ? 4.0 : std::ldexp(4.0, (int)b.qubits.size() - (int)b.controls.size());
+  const double namps = std::ldexp(1.0, s->n), sms = s->sm_count > 0 ? s->sm_count : 152;
+  const double passes = (double)plan_passes(blocks, s->n, m, L, kMaxOpsPerPass, kMaxMatPerPass).size();
+  const double fp64 = passes * (4.0 + 32.0 * namps / 5.5e6) + fmas * namps / 6.3e5;
+  const double oz = (double)oz_blocks * 10.5 * std::ceil(namps / 4096 / sms);
+  return fp64 < oz;
+}
+
 // Append a complex128 program of exact tensor-core passes, if every fused block of at
 // most 5 qubits qualifies: uncontrolled (wider or controlled ones stay on the
 // CUDA cores, and a program is all of one kind), digits within the exact range
@@ -749,7 +773,9 @@ static bool append_oz_program(const sv_state *s, const std::vector<Gate> &gates,
     moves = moves && permutation_of(b.U, (int)b.qubits.size(), perm);
     b.kind = TOP_TC;
   }
-  if (moves || out.prog.mats.size() + blocks.size() * kOzBlockBytes + (64 << 10) > kWsProgBytes) return false;
+  if (moves || out.prog.mats.size() + blocks.size() * kOzBlockBytes + (64 << 10) > kWsProgBytes ||
+      mostly_moves(s, gates, o, blocks.size()))
+    return false;
   std::vector<PassPlan> passes = plan_passes(blocks, n, m, L, kOzMaxBlocks, kOzMaxBlocks * 1024 + 1023);
   if (passes.empty()) return false;
   CachedProgram prog;

@@ -6,7 +6,7 @@ import pytest
 import workloads as W
 from test_programs_cpu import SV_C64, SV_C128, build, toffolis, tool  # noqa: F401
 
-TABLE, MOVES = 0x800, 0x2000   # kPassTable, kPassMoves
+OZ, MOVES = 0x1000, 0x2000   # kPassOz, kPassMoves
 
 
 def large(dt):
@@ -54,3 +54,12 @@ def test_wide_blocks(tool, n):  # noqa: F811
     """Dense 5-qubit blocks that do not qualify for the tensor cores."""
     c = W.block_chain(n, 20, 0)
     assert len(build(tool, c, SV_C128)[1]) == len(build(tool, c, SV_C128, large(SV_C128))[1])
+
+
+@pytest.mark.parametrize("n", [14, 17, 20, 22, 24])
+def test_moves_with_few_dense_gates_keep_fp64(tool, n):  # noqa: F811
+    """A GHZ state: one Hadamard and permutations.  With as much dense work as
+    moves the tensor cores stay."""
+    assert not any(f & OZ for f in build(tool, W.ghz(n), SV_C128)[1])
+    c = W.concat(W.ghz(n), W.remove_qubits(W.grid_random(5, 6, 12, 1), 30 - n, 3))
+    assert all(f & OZ for f in build(tool, c, SV_C128)[1])
