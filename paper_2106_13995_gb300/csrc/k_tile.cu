@@ -426,7 +426,9 @@ static int pass_threads(const sv_state *s, int m, int nvec, uint64_t tiles) {
 // SM is the share: 21 qubits, complex64, QFT 1004 us, 828 with ordinary launches
 // and 813 so; U3 + CZ on 18 qubits, 40 layers, complex64 316 us to 289, complex128
 // 3.78 ms to 2.96; 20 dense 5-qubit blocks, 20 qubits, complex128 6.2 ms to 5.3).
-// Only on the state's own stream: a batch's streams share the SMs.
+// Only on the state's own stream (a batch's streams share the SMs) and for one
+// vector (a gradient of 18 qubits took 476 us with its passes of two held back, 460
+// without).
 static size_t share_smem(const sv_state *s, size_t smem, uint64_t tiles, cudaStream_t stream) {
   const uint64_t sms = (uint64_t)s->sm_count, share = (tiles + sms - 1) / sms;
   if (stream != s->stream || 2 * tiles <= sms || share > 16) return smem;
@@ -557,7 +559,7 @@ sv_status launch_tile_pass_on(sv_state *s, const TilePass &p, int batch, cudaStr
   }
   if (smem > (200u << 10)) return set_error(SV_EINVAL, "tile too large for shared memory");
   dim3 grid((unsigned)(1ull << (p.n - p.m)), (unsigned)batch);
-  const size_t smem_cta = share_smem(s, smem, (uint64_t)grid.x * grid.y, stream);
+  const size_t smem_cta = p.nvec == 1 ? share_smem(s, smem, (uint64_t)grid.x * grid.y, stream) : smem;
   const int threads = pass_threads(s, p.m, (int)p.nvec, (uint64_t)grid.x * grid.y);
   if (host && sites_pass_ok(p, *host)) return launch_tile_sites(s, p, batch, threads, stream);
   sv_status st = SV_OK;
