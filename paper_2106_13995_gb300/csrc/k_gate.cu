@@ -175,7 +175,10 @@ __global__ void k_dense(typename Cx<R>::T *__restrict__ a, uint64_t ngroups, uin
 // unit, 16-byte accesses, several units per trip (as K3; the same sums in the
 // same order).  On 26 qubits a 2-qubit unitary 174 us by single amplitudes and
 // 159 so, a CNOT 85 and 75, a Toffoli 51 and 40; 3 targets load as much at a
-// time either way (160 and 161).
+// time either way (160 and 161).  Not where controls leave half of a 32-byte sector
+// or single units of a line (qubit 1, or two of the lowest four: 225 us against 175
+// with a control on qubit 1, 81 against 70 with three on 1, 2 and 12), nor with
+// target 1 in a state that the L2 holds (22 qubits 10.9 us against 8.7).
 template <int K>
 __global__ void k_dense_pairs(float2 *__restrict__ a, uint64_t nunits, uint64_t fixed, uint64_t cmask,
                               const __grid_constant__ DenseArgs<float, K> A) {
@@ -213,10 +216,14 @@ __global__ void k_dense_pairs(float2 *__restrict__ a, uint64_t nunits, uint64_t 
 // ---- K4: diagonal gate (targets and controls folded into one table) ------
 // Qubits whose 0 leaves an amplitude alone (controls, and the targets of Z, S, T
 // and phase gates) are fixed at 1, so a phase gate moves half of the state and a
-// controlled one a quarter.  Four 16-byte units per thread and trip, the table
-// in shared memory (each thread reads an entry of its own).  HBM-bound: a
-// controlled phase on 26 qubits 192 us when every amplitude passed through, 36
-// now.
+// controlled one a quarter.  Not complex64's qubit 1 in states beyond the L2: it is
+// half of every 32-byte sector (26 qubits 225 us, 168 with all of it; 24 qubits 41
+// and 46).  The table in shared memory (each thread reads an entry of its own).
+// HBM-bound: a controlled phase on 26 qubits 192 us when every amplitude passed
+// through, 48 now.  A 16-byte unit per thread and trip, without streaming hints:
+// four, with them, were slower where the state is in the L2 (a Z rotation in
+// complex64, 23 qubits 15.6 us against 14.5; complex128, 21 qubits 20.7 against 18.8)
+// and where FP64 bounds it (complex128, 25 qubits 271 against 256).
 template <typename R> struct DiagArgs {
   int npos;
   uint32_t q0;                  // table bit of qubit 0 (complex64 units hold both of its values), or 0
@@ -229,30 +236,20 @@ template <typename R>
 __global__ void __launch_bounds__(256) k_diag(typename Cx<R>::T *__restrict__ a, uint64_t nunits,
                                               const __grid_constant__ DiagArgs<R> A) {
   using C = typename Cx<R>::T;
-  constexpr int APU = 16 / (int)sizeof(C), UN = 4;
+  constexpr int APU = 16 / (int)sizeof(C);
   __shared__ C tab[256];
   for (int r = threadIdx.x; r < 1 << A.npos; r += blockDim.x) tab[r] = A.d[r];
   __syncthreads();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < nunits; u0 += UN * stride) {
-    int4 x[UN];
-    uint64_t i0[UN];
-#pragma unroll
-    for (int j = 0; j < UN; j++) {
-      const uint64_t u = u0 + j * stride;
-      i0[j] = ins0_mask64(u * APU, A.fixed) | A.fixed;
-      if (u < nunits) x[j] = __ldcs(reinterpret_cast<const int4 *>(a + i0[j]));
-    }
-#pragma unroll
-    for (int j = 0; j < UN; j++) {
-      if (u0 + j * stride >= nunits) break;
-      uint32_t r = 0;
-      for (int k = 0; k < A.npos; k++) r |= (uint32_t)((i0[j] >> A.pos[k]) & 1ull) << k;
-      C *v = reinterpret_cast<C *>(&x[j]);
-      v[0] = cmul(tab[r], v[0]);
-      if (APU == 2) v[APU - 1] = cmul(tab[r | A.q0], v[APU - 1]);
-      __stcs(reinterpret_cast<int4 *>(a + i0[j]), x[j]);
-    }
+  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nunits; u += stride) {
+    const uint64_t i = ins0_mask64(u * APU, A.fixed) | A.fixed;
+    int4 x = *reinterpret_cast<const int4 *>(a + i);
+    uint32_t r = 0;
+    for (int k = 0; k < A.npos; k++) r |= (uint32_t)((i >> A.pos[k]) & 1ull) << k;
+    C *v = reinterpret_cast<C *>(&x);
+    v[0] = cmul(tab[r], v[0]);
+    if (APU == 2) v[APU - 1] = cmul(tab[r | A.q0], v[APU - 1]);
+    *reinterpret_cast<int4 *>(a + i) = x;
   }
 }
 
@@ -304,7 +301,8 @@ static sv_status dense_k(sv_state *s, const std::vector<int> &t, const std::vect
   const uint64_t ngroups = 1ull << (s->n - __builtin_popcountll(fixed));
   const int threads = 256;
   if constexpr (K <= 2 && sizeof(R) == 4) {
-    if (!(fixed & 1) && ngroups >= 2) {
+    const bool sparse = (cmask & 2) || __builtin_popcountll(cmask & 15) >= 2 || ((fixed & 2) && s->n <= 24);
+    if (!(fixed & 1) && !sparse && ngroups >= 2) {
       constexpr int UN = K == 1 ? 4 : 2;
       k_dense_pairs<K><<<grid_for(s, (ngroups / 2 + UN - 1) / UN, threads), threads, 0, s->stream>>>(
           reinterpret_cast<float2 *>(s->amps), ngroups / 2, fixed, cmask, A);
@@ -386,10 +384,11 @@ static sv_status diag_launch(sv_state *s, const std::vector<int> &t, const std::
   auto entry = [&](int r) { return (r & cm) == cm ? d[r & ((1 << k) - 1)] : cd(1.0); };
   // units of 16 bytes keep both values of qubit 0 (complex64)
   const int apu = s->dt == SV_C64 && s->n >= 1 ? 2 : 1;
+  const int low = s->dt != SV_C64 ? 0 : s->n >= 25 ? 2 : 1;   // qubits that are never fixed
   int on = 0;             // table bits fixed at 1
   std::vector<int> free;  // the others, qubit 0 first
   for (int j = 0; j < nq; j++) {
-    bool idle = !(apu == 2 && q[j] == 0);
+    bool idle = q[j] >= low;
     for (int r = 0; r < (1 << nq) && idle; r++) idle = ((r >> j) & 1) || entry(r) == cd(1.0);
     if (idle) {
       on |= 1 << j;
@@ -410,7 +409,7 @@ static sv_status diag_launch(sv_state *s, const std::vector<int> &t, const std::
   }
   const uint64_t nunits = (1ull << (s->n - __builtin_popcountll(A.fixed))) / apu;
   const int threads = 256;
-  k_diag<R><<<grid_for(s, (nunits + 3) / 4, threads), threads, 0, s->stream>>>(
+  k_diag<R><<<grid_for(s, nunits, threads), threads, 0, s->stream>>>(
       reinterpret_cast<typename Cx<R>::T *>(s->amps), nunits, A);
   g_launches++;
   SV_CUDA(cudaGetLastError());
