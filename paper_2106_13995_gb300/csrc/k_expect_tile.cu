@@ -231,11 +231,15 @@ static int xtile_m(const sv_state *s) { return std::min(s->dt == SV_C64 ? 13 : 1
 constexpr int kXTileL = 3;
 
 // A group of nt strings goes through tile passes when its x mask fits a tile
-// next to the low qubits.  Below 10 qubits, and beyond 8 strings on one
-// mask, the table kernel (k_expect) is used: its cost per amplitude does not
-// grow with the strings.
-bool expect_tile_ok(const sv_state *s, uint64_t xm, int nt) {
-  return s->n >= 10 && xm != 0 && nt <= 8 &&
+// next to the low qubits.  Below 10 qubits, and beyond 8 strings on one mask, the
+// table kernel (k_expect) is used: its cost per amplitude does not grow with the
+// strings.  From 22 qubits on (complex128 21), where amplitudes count more than launches, it is the
+// better one beyond 4 strings, or 3 of the only group (26 qubits, complex64, eight
+// groups of 3, 4 and 6: tiles 1.58, 1.91 and 2.71 ms, tables 2.04 to 2.06; one group
+// of 3, 4 and 8: 268, 314 and 514 us, 300; 18 qubits, one of 8: 31 us and 43).
+bool expect_tile_ok(const sv_state *s, uint64_t xm, int nt, bool only) {
+  const int most = s->n <= (s->dt == SV_C64 ? 21 : 20) ? 8 : only ? 3 : 4;
+  return s->n >= 10 && xm != 0 && nt <= most &&
          __builtin_popcountll(xm >> kXTileL) <= xtile_m(s) - kXTileL;
 }
 

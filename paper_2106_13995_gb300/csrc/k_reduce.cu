@@ -142,12 +142,13 @@ __device__ __forceinline__ void block_sum_to(double v, double *dst) {
 // in turn is a chain of L2 latencies: 43 us for 608 partials against 3.
 __global__ void __launch_bounds__(kRedThreads) k_finalize(const double *__restrict__ partial, int nblocks, double *out) {
   double s = 0;
-  for (int b = threadIdx.x; b < nblocks; b += kRedThreads) s += partial[b];
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += partial[b];
   block_sum_to(s, out);
 }
 
 sv_status launch_finalize(sv_state *s, const double *partial, int nblocks, double *out_dev) {
-  k_finalize<<<1, kRedThreads, 0, s->stream>>>(partial, nblocks, out_dev);
+  // (small states: one warp, 0.3 us less)
+  k_finalize<<<1, nblocks <= 32 ? 32 : kRedThreads, 0, s->stream>>>(partial, nblocks, out_dev);
   g_launches++;
   SV_CUDA(cudaGetLastError());
   return SV_OK;
@@ -558,19 +559,19 @@ __global__ void k_zall_small(const typename Cx<R>::T *__restrict__ a, int n, dou
 // z[q] = total - 2 S_q from the blocks' partial sums: a warp per value, its
 // lanes striding over the blocks.  A thread per value was a chain of one L2
 // latency per block (63-126 us for 608 blocks; now 6).
-constexpr int kZFinishThreads = 1024;
+constexpr int kZFinishThreads = 1024, kZFinishSmall = 128;   // small states: one block's sums, 2 us less
 __global__ void __launch_bounds__(kZFinishThreads) k_zall_finish(const double *__restrict__ partial, int nblocks, int n,
                                                                  double *out) {
   __shared__ double sum[64 + 1];
   const int lane = threadIdx.x & 31;
-  for (int q = threadIdx.x >> 5; q <= n; q += kZFinishThreads / 32) {
+  for (int q = threadIdx.x >> 5; q <= n; q += (int)(blockDim.x >> 5)) {
     double s = 0;
     for (int b = lane; b < nblocks; b += 32) s += partial[(size_t)b * (n + 1) + q];
     s = warp_sum(s);
     if (lane == 0) sum[q] = s;
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < n; q += kZFinishThreads) out[q] = sum[n] - 2.0 * sum[q];
+  for (int q = threadIdx.x; q < n; q += blockDim.x) out[q] = sum[n] - 2.0 * sum[q];
 }
 
 sv_status launch_z_all(sv_state *s, double *out_dev) {
@@ -583,7 +584,7 @@ sv_status launch_z_all(sv_state *s, double *out_dev) {
       k_zall_small<float><<<1, 256, 0, s->stream>>>((const float2 *)s->amps, s->n, partial);
     else
       k_zall_small<double><<<1, 256, 0, s->stream>>>((const double2 *)s->amps, s->n, partial);
-    k_zall_finish<<<1, kZFinishThreads, 0, s->stream>>>(partial, 1, s->n, out_dev);
+    k_zall_finish<<<1, kZFinishSmall, 0, s->stream>>>(partial, 1, s->n, out_dev);
   } else {
     const uint64_t nchunks = namps / chunk_amps;
     const uint64_t warps_per_block = kRedThreads / 32;
@@ -648,7 +649,7 @@ sv_status zall_noalloc(const void *amps, int n, sv_dtype dt, double *out, cudaSt
       k_zall_small<float><<<1, 256, 0, stream>>>((const float2 *)amps, n, partial);
     else
       k_zall_small<double><<<1, 256, 0, stream>>>((const double2 *)amps, n, partial);
-    k_zall_finish<<<1, kZFinishThreads, 0, stream>>>(partial, 1, n, out);
+    k_zall_finish<<<1, kZFinishSmall, 0, stream>>>(partial, 1, n, out);
   } else {
     const uint64_t nchunks = namps / chunk_amps;
     const uint64_t wpb = kRedThreads / 32;

@@ -566,7 +566,7 @@ sv_status launch_expect_group(sv_state *s, uint64_t xmask, const uint64_t *zm, c
                               const int *ipow, int nt, double *out_dev);
 // strings with X or Y factors, many x masks per pass (k_expect_tile.cu); a
 // group lists the terms that share one x mask
-bool expect_tile_ok(const sv_state *s, uint64_t xmask, int nt);
+bool expect_tile_ok(const sv_state *s, uint64_t xmask, int nt, bool only);
 sv_status launch_expect_tiles(sv_state *s, const sv_pauli_term *terms, const std::vector<std::vector<int>> &groups,
                               double *out_dev);
 // *out_dev = sum of nblocks FP64 partial sums

@@ -39,7 +39,7 @@ sv_status sv_expect(sv_state *s, const sv_pauli_term *terms, int nt, double *out
   for (int t = 0; t < nt; t++) groups[terms[t].x_mask].push_back(t);
   std::vector<std::vector<int>> chunks, tiled;
   for (auto &g : groups) {
-    if (expect_tile_ok(s, g.first, (int)g.second.size())) {
+    if (expect_tile_ok(s, g.first, (int)g.second.size(), groups.size() == 1)) {
       tiled.push_back(g.second);
       continue;
     }
