@@ -545,7 +545,7 @@ def main():
         def mult_all(dense: bool):
             for a_, b_ in ab:
                 ms_.set_basis(W.multiplier_basis_index(int(a_), int(b_), 7))
-                if dense:   # forget the basis state: tile passes of permutation ops
+                if dense:   # forget the basis state: a move of every amplitude
                     NM.check(NM.lib().sv_mark_modified(ms_.h))
                 ms_.apply_circuit(mmc)
 
@@ -558,7 +558,8 @@ def main():
         th_ = timed(lambda: (ms_.set_basis(0), ms_.apply_circuit(mmh)), 2) / 2
         out["multiplier"] = {"n_qubits": 29, "native_ops": len(mc.ops), "basis_runs": 64,
                              "runs_per_s": 64 / tm_, "gates_per_s": 64 * len(mc.ops) / tm_,
-                             "path": "tile passes composed into permutation tables (one move per amplitude, no arithmetic)",
+                             "path": "one move of every amplitude within chunks of 2^22 (source indices computed "
+                                     "bit-sliced, no arithmetic)",
                              "basis_fast_path": {"runs_per_s": 64 / tf_, "gates_per_s": 64 * len(mc.ops) / tf_,
                                                  "path": "basis state followed on the host, two amplitudes "
                                                          "rewritten; each run includes the 4 GiB basis-state "
@@ -729,8 +730,8 @@ def main():
                                "circuits": len(circs), "widths": "10..24", "depth": 40,
                                "gates": int(sum(len(c.ops) for c in circs)),
                                "launch": "one CUDA graph per call: a persistent cooperative launch for states "
-                                         "whose passes have fewer tiles than SMs, full-grid tile launches for the "
-                                         "wider ones; plus one basis-state write per state"}
+                                         "below 14 qubits (below 16 where more than 40 have 14 or 15), full-grid "
+                                         "tile launches for the wider ones; plus one basis-state write per state"}
         del ust
 
     # ---- width sweep (Sec. II: random qubit removal from the 5x6 grid) ------------

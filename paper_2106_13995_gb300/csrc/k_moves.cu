@@ -19,9 +19,11 @@
 // moves its own (programmatic launch, and every CTA waits for the last launch
 // before it reads or writes amplitudes or scratch).
 //
-// Bound: the load-store pipe.  The gather reads 8 bytes from each of 32 lines a
-// warp (one line a clock: 14 us a chunk), the words of a 222-gate run add 8 us;
-// a chunk of 32 MB takes 36 us, 10 of them HBM.  The 7-bit multiplier on 29
+// Bound: latency, of the words of the bit-sliced gates in shared memory and of a
+// gather that reads 8 bytes from each of 32 lines a warp: no unit is full (load-
+// store data pipe 50%, L2 41%, DRAM 26%, issue 30% with 37% of the warps; short
+// scoreboard and MIO throttle are the top stalls).  A chunk of 32 MB takes 36 us, 10
+// of them HBM.  The 7-bit multiplier on 29
 // qubits took 15 table passes of 1.6 ms; its moves take 4.6 ms (6.4 with the
 // launches one after the other, 5.9 with the copying CTAs first, 4.8 in chunks
 // of 2^23).

@@ -731,7 +731,7 @@ static void move_to_end(std::vector<Block> &from, std::vector<Block> &to) {
 // Circuits that mostly move amplitudes (a GHZ state, X layers before a few dense
 // gates): a tensor-core block takes its time whatever it does, 10 us a tile and SM,
 // FP64 arithmetic only that of the blocks that are no permutations (GHZ of 14
-// qubits 43 us against 16, of 22 qubits 431 against 298).  Weighed where three fifths
+// qubits 39 us against 19, of 22 qubits 430 against 297).  Weighed where three fifths
 // of the gates are permutations.
 static bool mostly_moves(const sv_state *s, const std::vector<Gate> &gates, const Opts &o, size_t oz_blocks) {
   int perm[64];

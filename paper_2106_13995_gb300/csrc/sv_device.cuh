@@ -94,11 +94,11 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 // complete before it touches amplitudes.  What a launch costs on the way (the time
 // from one pass's end to the next one's start, and the next one's set-up) then
 // passes while the last one works: 20 layers of U3 + CZ in complex128, 12 qubits
-// 481 us to 420, 16 qubits 424 to 377; 40 layers in complex64, 18 qubits 366 to
-// 314; a gradient step of 16 qubits 522 to 462.  Tile passes call pass_start
+// 468 us with ordinary launches, 414 so; 40 layers in complex64, 18 qubits 372 and
+// 316 (289 with share_smem); a gradient step of 16 qubits 528 and 450.  Tile passes call pass_start
 // before their stores: the next pass's CTAs then take the SMs as these leave them
-// (called first thing, 18 qubits took 436 us).  Passes of sites call it first and
-// read their matrices meanwhile (462 us against 471).
+// (called first thing, 18 qubits took 436 us), each SM its share of them (share_smem
+// in k_tile.cu).  Passes of sites call it first and read their matrices meanwhile.
 __device__ __forceinline__ void pass_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
