@@ -77,8 +77,8 @@ typedef enum { SV_C64 = 0, SV_C128 = 1 } sv_dtype;
  * mixes all of those by factors within 2^6 of its largest.  Every amplitude
  * then keeps what FP64 arithmetic gives it: one rounding of the result, and an
  * error of about 2^-53 of the magnitudes added up in it, also beside amplitudes
- * many orders larger.  Other circuits (rotations by small angles, say) take
- * FP64 arithmetic throughout. */
+ * many orders larger.  Other circuits (rotations by small angles, say, or mostly
+ * permutations) take FP64 arithmetic throughout. */
 typedef enum {
   SV_PREC_PLAIN = 0,       /* FP32 FMA on CUDA cores */
   SV_PREC_TC_BF16X3 = 1,   /* tensor cores, split-BF16 (3 products), FP32 accumulate */
@@ -221,9 +221,10 @@ sv_status sv_apply_gate(sv_state *s, const int32_t *targets, int k, const int32_
  * their products) only move amplitudes inside the tile: a pass made only of
  * such blocks is composed on the host into one gather table per setting of
  * its global control qubits (at most 5 of them, tables within half the
- * program area) and moves each amplitude once, exactly.  From 15 qubits on and
- * with fusion_k and tile_m left at 0, a long run of such gates is one move of
- * every amplitude within chunks of 2^22 (see sv_workspace_bytes).  A state
+ * program area) and moves each amplitude once, exactly.  With fusion_k and
+ * tile_m left at 0, a long run of such gates has tiles of its own or, from 15
+ * qubits on, is one move of every amplitude within chunks of 2^22 (see
+ * sv_workspace_bytes), whichever is faster.  A state
  * known to be a basis state (see sv_set_basis) takes no pass at all when every
  * gate maps basis states to basis states; single-qubit gates on it in front of
  * such a run are written as the product state they make (not while the stream
