@@ -50,8 +50,9 @@ Opts resolve(const sv_state *s, const sv_options *o, int nvec) {
   // The few tiles leave the FP64 pipes waiting on each other's results, and
   // a 2-qubit block's chains are half as long (20 layers of U3 + CZ, 7-qubit
   // tiles: 12 qubits 467 against 687 us, 16 qubits 675 against 973; at 18
-  // qubits, 8-qubit tiles, no difference).
-  const bool small128 = s->dt == SV_C128 && s->n <= kSmall128 && nvec == 1 && !(o && o->prec != SV_PREC_PLAIN);
+  // qubits, 8-qubit tiles, no difference).  Not 3 qubits, a whole circuit in one
+  // triple (40 layers 18 us against 79).
+  const bool small128 = s->dt == SV_C128 && s->n > 3 && s->n <= kSmall128 && nvec == 1 && !(o && o->prec != SV_PREC_PLAIN);
   r.fusion_k = (o && o->fusion_k > 0) ? o->fusion_k : (o && o->prec != SV_PREC_PLAIN ? 5 : (small128 ? 2 : 3));
   // default tiles: 13 qubits for single-vector CUDA-core passes on complex64
   // (fewer passes; 32 amplitudes per thread at 256 threads), 12 otherwise

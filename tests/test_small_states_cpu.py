@@ -63,3 +63,9 @@ def test_moves_with_few_dense_gates_keep_fp64(tool, n):  # noqa: F811
     assert not any(f & OZ for f in build(tool, W.ghz(n), SV_C128)[1])
     c = W.concat(W.ghz(n), W.remove_qubits(W.grid_random(5, 6, 12, 1), 30 - n, 3))
     assert all(f & OZ for f in build(tool, c, SV_C128)[1])
+
+
+def test_three_qubits_are_one_block(tool):  # noqa: F811
+    """A complex128 circuit of 3 qubits: no more ops than with fused triples."""
+    c = W.random_u3_cz(3, 40, 1)
+    assert build(tool, c, SV_C128)[0] <= build(tool, c, SV_C128, large(SV_C128))[0]
